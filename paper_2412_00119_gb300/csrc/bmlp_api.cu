@@ -261,7 +261,7 @@ int enqueue_step(bmlp_t* h, cudaStream_t st, bool fork, bool chained = false) {
     }
     prof_begin(h, kProfTrainFwd, st);
     if (h->fwd_impl == BMLP_FWD_TCGEN05)
-      CK(h, launch_train_forward_tc(h->K[l], st, fork && (l > 1 || chained), h->dP, l));
+      CK(h, launch_train_forward_tc(h->bs, h->K[l], h->K[l - 1], st, fork && (l > 1 || chained), h->dP, l));
     else
       k_train_forward<<<train_forward_grid(h->bs, h->K[l]), train_forward_block(), 0, st>>>(h->dP, l);
     prof_end(h, st);
@@ -392,6 +392,19 @@ int ensure_eval(bmlp_t* h, int64_t rows) {
 
 constexpr int64_t kEvalChunk = 65536;
 constexpr int64_t kStageRows = 65536;
+constexpr int64_t kTileRows = 512;
+
+// One layer of forward-only evaluation on the tensor-core engine.  pdl: the
+// launch before it in the stream is another call of this function whose
+// output it reads.
+cudaError_t eval_layer_tc(bmlp_t* h, const DevLayer& D, const uint64_t* in, int64_t m, uint64_t* out,
+                          cudaStream_t st, bool pdl) {
+  if (m <= kTileRows)
+    return launch_forward_tile(in, m, D.nw_in, D.W, D.Kout, D.Kin, out, D.nw_out, &h->dCtrl->timeouts, st,
+                               pdl);
+  launch_forward_eval_tc(in, m, D.nw_in, D.W, D.Kout, D.Kin, out, D.nw_out, &h->dCtrl->timeouts, st);
+  return cudaGetLastError();
+}
 
 }  // namespace
 
@@ -718,8 +731,7 @@ int predict_impl(bmlp_t* h, const uint64_t* x, int64_t n, int32_t* out, void* cu
       const DevLayer& D = h->hp.layer[l - 1];
       prof_begin(h, kProfEvalFwd, st);
       if (h->fwd_impl == BMLP_FWD_TCGEN05)
-        launch_forward_eval_tc(in, m, D.nw_in, D.W, D.Kout, D.Kin, h->evA[cur], D.nw_out,
-                               &h->dCtrl->timeouts, st);
+        CK(h, eval_layer_tc(h, D, in, m, h->evA[cur], st, l > 1 && !every_layer && !h->profiling));
       else
         k_forward_eval<<<eval_forward_grid(m, D.Kout), eval_forward_block(), 0, st>>>(
             in, m, D.nw_in, D.W, D.Kout, D.Kin, h->evA[cur], D.nw_out);
@@ -943,8 +955,7 @@ int bmlp_layer_forward(bmlp_t* h, int32_t layer, const uint64_t* a_in, int64_t n
     uint64_t* out = a_out + s0 * D.nw_out;
     prof_begin(h, kProfEvalFwd, st);
     if (h->fwd_impl == BMLP_FWD_TCGEN05)
-      launch_forward_eval_tc(in, m, D.nw_in, D.W, D.Kout, D.Kin, out, D.nw_out,
-                             &h->dCtrl->timeouts, st);
+      CK(h, eval_layer_tc(h, D, in, m, out, st, false));
     else
       k_forward_eval<<<eval_forward_grid(m, D.Kout), eval_forward_block(), 0, st>>>(
           in, m, D.nw_in, D.W, D.Kout, D.Kin, out, D.nw_out);
@@ -967,7 +978,10 @@ int bmlp_layer_forward_engine(bmlp_t* h, int32_t layer, int32_t engine, const ui
   if (n == 0) return BMLP_OK;
   if (!a_in || !a_out || !is_device_ptr(a_in) || !is_device_ptr(a_out))
     return fail(h, BMLP_EINVAL, "a_in and a_out must be device pointers");
-  if (engine == BMLP_FWD_TCGEN05) CK(h, prepare_forward_eval_tc());
+  if (engine == BMLP_FWD_TCGEN05) {
+    CK(h, prepare_train_forward_tc());
+    CK(h, prepare_forward_eval_tc());
+  }
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const DevLayer& D = h->hp.layer[layer - 1];
   for (int64_t s0 = 0; s0 < n; s0 += kEvalChunk) {
@@ -976,8 +990,7 @@ int bmlp_layer_forward_engine(bmlp_t* h, int32_t layer, int32_t engine, const ui
     uint64_t* out = a_out + s0 * D.nw_out;
     prof_begin(h, kProfEvalFwd, st);
     if (engine == BMLP_FWD_TCGEN05)
-      launch_forward_eval_tc(in, m, D.nw_in, D.W, D.Kout, D.Kin, out, D.nw_out,
-                             &h->dCtrl->timeouts, st);
+      CK(h, eval_layer_tc(h, D, in, m, out, st, false));
     else if (engine == BMLP_FWD_B1MMA)
       CK(h, launch_forward_b1(in, m, D.nw_in, D.W, D.Kout, D.Kin, out, D.nw_out, st));
     else

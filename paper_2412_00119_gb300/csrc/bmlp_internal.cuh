@@ -197,13 +197,18 @@ __global__ void k_transpose_rho(const int8_t* rho, int8_t* rhoT, int Kout, int c
 // Re-derive W from H for one layer (after set_state).
 __global__ void k_repack_w(const uint32_t* H, uint64_t* W, int Kin, int Kout, int ldh, int ngrp,
                            int nplanes, int h_max);
-// Tensor-core forward (tcgen05, +-1 as e4m3, exact fp32 sums), training layer l;
-// needs bs <= 128.  The activations of layer l - 1 (the inputs for l = 1) are
-// read as packed bits.
-size_t train_forward_tc_smem();
+// Tensor-core forward (tcgen05, +-1 as e2m1, exact fp32 sums), training layer
+// l.  The activations of layer l - 1 (the inputs for l = 1) are read as packed
+// bits.  pdl: launched with the programmatic-stream-serialization attribute.
 cudaError_t prepare_train_forward_tc();
-// pdl: launched with the programmatic-stream-serialization attribute.
-cudaError_t launch_train_forward_tc(int Kout, cudaStream_t st, bool pdl, const StepParams* P, int l);
+cudaError_t launch_train_forward_tc(int bs, int Kout, int Kin, cudaStream_t st, bool pdl,
+                                    const StepParams* P, int l);
+// The same tiles for one layer of forward-only evaluation on a small batch: A
+// (M x nw_in) against W -> Aout (M x nw_out); an expired bounded wait adds one
+// to *timeouts.
+cudaError_t launch_forward_tile(const uint64_t* A, int64_t M, int nw_in, const uint64_t* W, int N, int Kin,
+                                uint64_t* Aout, int nw_out, unsigned int* timeouts, cudaStream_t st,
+                                bool pdl);
 // Median binarisation of n x K fp32 patterns into n x nw packed words.
 void launch_binarize_median(const float* x, int64_t n, int K, int nw, uint64_t* out,
                             cudaStream_t st);

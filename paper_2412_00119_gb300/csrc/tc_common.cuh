@@ -22,8 +22,7 @@ __device__ __forceinline__ void mbar_init(unsigned long long* bar, uint32_t coun
 }
 
 __device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
-  asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}"
-               ::"r"(smem_u32(bar)) : "memory");
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 // Bounded wait for the phase with the given parity; false on expiry (after
@@ -32,13 +31,18 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t pari
                                           volatile int* failed,
                                           unsigned long long limit = kWaitCycles) {
   const uint32_t a = smem_u32(bar);
-  const unsigned long long t0 = clock64();
-  while (true) {
-    uint32_t ok;
+  uint32_t ok;
+  auto try_wait = [&]() {
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
         " selp.u32 %0, 1, 0, p;\n}"
         : "=r"(ok) : "r"(a), "r"(parity) : "memory");
+  };
+  try_wait();                       // most waits end here, without reading the clock
+  if (ok) return true;
+  const unsigned long long t0 = clock64();
+  while (true) {
+    try_wait();
     if (ok) return true;
     if (*failed) return false;
     if (clock64() - t0 > limit) {
@@ -102,6 +106,76 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
   asm volatile(
       "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
       ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// +-1 as e2m1 (4 bits), tcgen05.mma kind::mxf4 with unit scales.
+//
+// +-1 (0x2 / 0xA) is exact in e2m1, a zero nibble is 0, and with every block
+// scale 1 (UE8M0 0x7F) each product is +-1 or 0 and every partial sum an
+// integer of magnitude <= K < 2^24, exact in fp32 in any order.  One MMA
+// (M128 N256 K64) takes the time of an e4m3 one with half the K, and a stage
+// row of 128 bytes holds 256 elements: 4,474 T MAC/s (operands in shared
+// memory) and 4,846 T (A in tensor memory) against 1,935 T for e4m3, random
+// +-1 on all 152 SMs.
+//
+// A 32-bit word x of bits becomes four words of eight nibbles: word j holds
+// the sign bits of x's bits 4 n + 3 - j (n = 0..7), so each output word is one
+// shift and one logical operation.  The order of the K-elements inside a
+// group of 32 differs from the bit order, alike in both operands, and so does
+// the sign (a set bit, +1, becomes -1): neither changes a product sum.
+// ---------------------------------------------------------------------------
+constexpr int KF = 256;  // K elements (two e2m1 per byte) per 128-byte stage row
+constexpr uint32_t kUnitScales = 0x7F7F7F7Fu;  // four UE8M0 scales of 1
+
+__device__ __forceinline__ void e2m1_words(uint32_t x, uint32_t (&w)[4]) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) w[j] = ((x << j) & 0x88888888u) ^ 0x22222222u;
+}
+
+// Instruction descriptor, kind::mxf4: A = B = e2m1, UE8M0 scales, both
+// K-major, M x N per instruction (K = 64).
+__host__ __device__ constexpr uint32_t idesc_f4(int M, int N) {
+  return (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | (1u << 23) | ((uint32_t)(M >> 4) << 24);
+}
+
+// A in tensor memory (lane = row, eight e2m1 per 32-bit column), B in shared
+// memory, the block scales of both at tensor-memory columns sf (all 1).
+__device__ __forceinline__ void mma_f4_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc,
+                                          uint32_t idesc, uint32_t sfa, uint32_t sfb,
+                                          uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %6, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], [%1], %2, %3, [%4], [%5], p;\n}"
+      ::"r"(tmem_d), "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(sfa), "r"(sfb), "r"(accumulate));
+}
+
+// 16: every row of a matrix of nw-word rows allows 16-byte copies; else 8.
+__host__ __device__ __forceinline__ int row_align(const void* base, int nw) {
+  return ((reinterpret_cast<uintptr_t>(base) | (uintptr_t)(8 * (uint32_t)nw)) & 15) == 0 ? 16 : 8;
+}
+
+// Asynchronous copy of kBytes (16 past L1, or 8) to shared memory; zeros
+// instead when !live (src is then not read, but must be a valid address).
+template <int kBytes>
+__device__ __forceinline__ void cp_async_or_zero(uint32_t dst, const void* src, bool live) {
+  const int n = live ? kBytes : 0;
+  if constexpr (kBytes == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ uint4 lds128(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts128(uint32_t a, const uint32_t (&v)[4]) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+
+__device__ __forceinline__ void cp_async_wait_all() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // A producer item: one 16-byte chunk of one row of a stage, i.e. 16

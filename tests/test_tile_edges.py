@@ -1,0 +1,59 @@
+"""The evaluation and front-end kernels at the edges of their tiles (MMA tiles,
+K pieces, K splits, odd word counts, single rows), bit for bit against the
+oracle."""
+import os
+
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+import workloads as W
+from paper_2412_00119_gb300 import bmlp as B
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _setup():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    torch.cuda.set_device(DEV)
+    O.set_threads(os.cpu_count() or 1)
+    B.lib()
+
+
+def dev(xp):
+    return torch.from_numpy(np.ascontiguousarray(xp).view(np.int64)).to(DEV)
+
+
+# widths K, N and patterns n: tiles of 128 neurons and 16 .. 112 patterns, pieces
+# of 1024 and k-steps of 256 inputs, splits of 1 .. 4, rows of odd word counts
+SMALL = [(1, 1, 1), (63, 127, 15), (64, 128, 16), (255, 129, 17), (257, 300, 112), (784, 1024, 100),
+         (1000, 525, 113), (1023, 130, 33), (1025, 640, 100), (2049, 70, 7), (3072, 4096, 128),
+         (5000, 257, 200), (8190, 1000, 100), (32767, 33, 9), (960, 8192, 512)]
+
+
+@pytest.mark.parametrize("K,N,n", SMALL)
+def test_small_batch_forward(K, N, n):
+    gpu = B.BMLP((K, N), 4, seed=K + N, bs=64)
+    ref = O.OracleModel([K, N], 4, seed=K + N, bs=64)
+    xp = W.random_packed(n, n, K)
+    _, a = O.layer_forward(W.unpack(xp, K), ref.H(1))
+    want = W.pack(a)
+    out = torch.full((n, W.words(N)), -1, dtype=torch.int64, device=DEV)
+    B.bmlp_layer_forward(gpu.h, 1, dev(xp), out)
+    assert np.array_equal(out.cpu().numpy().view(np.uint64), want)
+    # rows that start 8 bytes off a 16-byte boundary, with pad bits set
+    xp2 = np.zeros(n * W.words(K) + 1, np.uint64)
+    rows = xp2[1:].reshape(n, -1)
+    rows[:] = xp
+    if K % 64:
+        rows[:, -1] |= ~np.uint64((1 << (K % 64)) - 1)
+    x2 = dev(xp2)[1:].view(n, -1)
+    out.fill_(-1)
+    B.bmlp_layer_forward(gpu.h, 1, x2, out)
+    assert np.array_equal(out.cpu().numpy().view(np.uint64), want)
+    gpu.close()
