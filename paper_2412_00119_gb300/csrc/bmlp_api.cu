@@ -731,7 +731,7 @@ int predict_impl(bmlp_t* h, const uint64_t* x, int64_t n, int32_t* out, void* cu
       const DevLayer& D = h->hp.layer[l - 1];
       prof_begin(h, kProfEvalFwd, st);
       if (h->fwd_impl == BMLP_FWD_TCGEN05)
-        CK(h, eval_layer_tc(h, D, in, m, h->evA[cur], st, l > 1 && !every_layer && !h->profiling));
+        CK(h, eval_layer_tc(h, D, in, m, h->evA[cur], st, l > 1 && !h->profiling));
       else
         k_forward_eval<<<eval_forward_grid(m, D.Kout), eval_forward_block(), 0, st>>>(
             in, m, D.nw_in, D.W, D.Kout, D.Kin, h->evA[cur], D.nw_out);
@@ -743,7 +743,11 @@ int predict_impl(bmlp_t* h, const uint64_t* x, int64_t n, int32_t* out, void* cu
       int32_t* dst = out + (every_layer ? (int64_t)(l - 1) * n : 0) + s0;
       int32_t* o = odev ? dst : h->stOut;
       prof_begin(h, kProfOut, st);
-      k_predict_out<<<(unsigned)((m + 7) / 8), 256, 0, st>>>(in, m, D.nw_out, D.PT, h->c, D.Kout, o);
+      if (h->fwd_impl == BMLP_FWD_TCGEN05 && h->c <= kPredictTileClasses)
+        CK(h, launch_predict_tile(in, m, D.nw_out, D.PT, h->c, D.Kout, o, &h->dCtrl->timeouts, st,
+                                  m <= kTileRows && !h->profiling));
+      else
+        k_predict_out<<<(unsigned)((m + 7) / 8), 256, 0, st>>>(in, m, D.nw_out, D.PT, h->c, D.Kout, o);
       prof_end(h, st);
       CK(h, cudaGetLastError());
       h->launches += 1;

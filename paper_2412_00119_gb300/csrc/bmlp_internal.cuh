@@ -209,6 +209,12 @@ cudaError_t launch_train_forward_tc(int bs, int Kout, int Kin, cudaStream_t st, 
 cudaError_t launch_forward_tile(const uint64_t* A, int64_t M, int nw_in, const uint64_t* W, int N, int Kin,
                                 uint64_t* Aout, int nw_out, unsigned int* timeouts, cudaStream_t st,
                                 bool pdl);
+// The evaluation output on the same tiles, for at most kPredictTileClasses
+// classes: labels[mu] = argmax_j of row mu of A against the c rows of PT (lowest
+// j on ties), K the width of the layer.
+constexpr int kPredictTileClasses = 128;
+cudaError_t launch_predict_tile(const uint64_t* A, int64_t M, int nw, const uint64_t* PT, int c, int K,
+                                int32_t* labels, unsigned int* timeouts, cudaStream_t st, bool pdl);
 // Median binarisation of n x K fp32 patterns into n x nw packed words.
 void launch_binarize_median(const float* x, int64_t n, int K, int nw, uint64_t* out,
                             cudaStream_t st);
@@ -217,8 +223,10 @@ void launch_binarize_median(const float* x, int64_t n, int K, int nw, uint64_t* 
 void launch_expand_weights(uint64_t seed, int K, int D, uint64_t* E, cudaStream_t st);
 void launch_expand_sign(const uint8_t* x, int64_t n, int D, const uint64_t* E, int K,
                         uint64_t* out, cudaStream_t st);
-// Tensor-core forward for evaluation: A (M x nw_in) against W -> Aout
-// (M x nw_out), 256-pattern x 256-neuron tiles per CTA pair; an expired
+// SMs of the current device (looked up once).
+int sm_count();
+// Tensor-core forward for evaluation on large batches: A (M x nw_in) against W
+// -> Aout (M x nw_out), 256-pattern x 256-neuron tiles per CTA pair; an expired
 // bounded wait adds one to *timeouts.
 cudaError_t prepare_forward_eval_tc();
 // One CTA waiting (bounded by limit_cycles) on an mbarrier that completes only

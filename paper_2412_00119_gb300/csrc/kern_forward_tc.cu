@@ -56,6 +56,18 @@
 #include "tc_common.cuh"
 
 namespace bk {
+
+int sm_count() {
+  static const int n = [] {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1)
+      v = 152;
+    return v;
+  }();
+  return n;
+}
+
 namespace {
 
 using namespace tc;
@@ -132,22 +144,6 @@ __device__ __forceinline__ void load_cols16(int (&z)[16], uint32_t taddr) {
   for (int j = 0; j < 16; ++j) z[j] = __float2int_rn(__uint_as_float(v[j]));
 }
 
-// 32 TMEM columns of this warp's 32 lanes from each lane's 256 bits.
-__device__ __forceinline__ void tmem_store_row256(uint32_t taddr, const uint32_t (&x)[8]) {
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {   // 16 columns at a time (registers)
-    uint32_t v[4][4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) e2m1_words(x[4 * h + q], v[q]);
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
-        "%12, %13, %14, %15, %16};"
-        ::"r"(taddr + 16u * (uint32_t)h), "r"(v[0][0]), "r"(v[0][1]), "r"(v[0][2]), "r"(v[0][3]),
-          "r"(v[1][0]), "r"(v[1][1]), "r"(v[1][2]), "r"(v[1][3]), "r"(v[2][0]), "r"(v[2][1]),
-          "r"(v[2][2]), "r"(v[2][3]), "r"(v[3][0]), "r"(v[3][1]), "r"(v[3][2]), "r"(v[3][3]) : "memory");
-  }
-}
-
 // A piece (words w0 .. w0 + 15) of nrows rows of nw words -> the bit rows from
 // `dst` on; rows >= live and words >= nw become 0.
 template <int kAlign>
@@ -190,6 +186,7 @@ struct TileIn {
   int16_t* Z;          // [pattern][N], or null
   uint64_t* Aout;      // [pattern][nw_out]
   int nw_out;
+  int32_t* labels;     // kLabels: the row's argmax of W A (lowest index on ties)
 };
 
 // Barriers and tensor memory, set up before the inputs are waited for.
@@ -216,7 +213,9 @@ __device__ __forceinline__ void tile_setup(TcShared* sh, int warp, int lane) {
 
 // One tile.  ready(): waits for the inputs and returns the rows of pattern 0
 // and the number of patterns; w_early: the weights may be read before that.
-template <int kAlign, typename Ready>
+// kLabels: W's rows are the classes (one tile, S = 1) and the output is the
+// argmax over them instead of z and the signs.
+template <int kAlign, bool kLabels = false, typename Ready>
 __device__ __forceinline__ void run_tile(TileIn T, const Place& pl, int pat, bool w_early, Ready ready,
                                          unsigned int* timeouts) {
   TcShared* sh = pl.sh;
@@ -397,6 +396,18 @@ __device__ __forceinline__ void run_tile(TileIn T, const Place& pl, int pat, boo
       const int64_t mb = m0 + 16 * b;
       const int rows = min(16, mt - 16 * b);
       uint32_t mine = 0;
+      if constexpr (kLabels) {
+        // largest score, then lowest class, of this warp's 32 classes: scores
+        // are within +-32767, a class never needs more than 7 bits
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const uint32_t k = n < T.N ? ((uint32_t)(z[j] + 32768) << 7) | (uint32_t)(TN - 1 - n) : 0u;
+          const uint32_t best = __reduce_max_sync(kFull, k);
+          if (lane == j) mine = best;
+        }
+        if (lane < 16) part[TN * q + 16 * b + lane] = mine;
+        continue;
+      }
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         const uint32_t bits = __ballot_sync(kFull, n < T.N && z[j] >= 0);
@@ -418,6 +429,14 @@ __device__ __forceinline__ void run_tile(TileIn T, const Place& pl, int pat, boo
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if constexpr (kLabels) {
+    if ((int)threadIdx.x < mt && !*failed) {
+      uint32_t best = 0u;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) best = max(best, part[TN * e + threadIdx.x]);
+      T.labels[m0 + threadIdx.x] = TN - 1 - (int)(best & 127u);
+    }
+  }
   if (threadIdx.x == 0 && *failed) atomicAdd(timeouts, 1u);
   if (warp == kProdWarps)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
@@ -430,7 +449,7 @@ __global__ void __launch_bounds__(THREADS, 2) k_train_forward_tc(const StepParam
   extern __shared__ uint8_t smem_raw[];
   const DevLayer& Ly = P->layer[l - 1];
   const uint64_t* x = l == 1 ? P->x : P->layer[l - 2].A;
-  const TileIn T{x, Ly.W, Ly.nw_in, Ly.Kout, Ly.Kin, Ly.Z, Ly.A, Ly.nw_out};
+  const TileIn T{x, Ly.W, Ly.nw_in, Ly.Kout, Ly.Kin, Ly.Z, Ly.A, Ly.nw_out, nullptr};
   const int64_t ncall = P->n;
   const int bs = P->bs;
   // Layers >= 2: the weights (the previous step's update), the batch index
@@ -458,13 +477,29 @@ __global__ void __launch_bounds__(THREADS, 2)
                    int Kin, uint64_t* __restrict__ Aout, int nw_out, unsigned int* __restrict__ timeouts,
                    int pat) {
   extern __shared__ uint8_t smem_raw[];
-  const TileIn T{A, W, nw, N, Kin, nullptr, Aout, nw_out};
+  const TileIn T{A, W, nw, N, Kin, nullptr, Aout, nw_out, nullptr};
   auto ready = [&](const uint64_t*&, int64_t& m) {
     pdl_wait();
     pdl_trigger();
     m = M;
   };
   run_tile<kAlign>(T, place(smem_raw), pat, true, ready, timeouts);
+}
+
+// Evaluation output on at most 128 classes: labels = argmax_j (A PT^T)_j, lowest j
+// on ties (PT: the packed classifier columns, c rows of nw words; K = its bits).
+template <int kAlign>
+__global__ void __launch_bounds__(THREADS, 2)
+    k_predict_tile(const uint64_t* __restrict__ A, int64_t M, int nw, const uint64_t* __restrict__ PT, int c,
+                   int K, int32_t* __restrict__ labels, unsigned int* __restrict__ timeouts, int pat) {
+  extern __shared__ uint8_t smem_raw[];
+  const TileIn T{A, PT, nw, c, K, nullptr, nullptr, 0, labels};
+  auto ready = [&](const uint64_t*&, int64_t& m) {
+    pdl_wait();
+    pdl_trigger();
+    m = M;
+  };
+  run_tile<kAlign, true>(T, place(smem_raw), pat, true, ready, timeouts);
 }
 
 // Patterns per tile, pattern tiles and K split of M patterns on an N x Kin
@@ -489,17 +524,6 @@ Shape shape_of(int64_t M, int N, int Kin, int sms) {
   s.pat = (int)(((M + mt - 1) / mt + 15) / 16 * 16);
   s.mtiles = (int)((M + s.pat - 1) / s.pat);
   return s;
-}
-
-int sm_count() {
-  static const int n = [] {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1)
-      v = 152;
-    return v;
-  }();
-  return n;
 }
 
 template <typename... KArgs, typename... Args>
@@ -532,6 +556,8 @@ cudaError_t prepare_train_forward_tc() {
   cudaError_t e = allow_smem(k_train_forward_tc);
   if (e == cudaSuccess) e = allow_smem(k_forward_tile<8>);
   if (e == cudaSuccess) e = allow_smem(k_forward_tile<16>);
+  if (e == cudaSuccess) e = allow_smem(k_predict_tile<8>);
+  if (e == cudaSuccess) e = allow_smem(k_predict_tile<16>);
   return e;
 }
 
@@ -548,6 +574,14 @@ cudaError_t launch_forward_tile(const uint64_t* A, int64_t M, int nw_in, const u
   const bool wide = row_align(A, nw_in) == 16 && row_align(W, nw_in) == 16;
   return launch_tiles(wide ? k_forward_tile<16> : k_forward_tile<8>, s, st, pdl, A, M, nw_in, W, N, Kin, Aout,
                       nw_out, timeouts, s.pat);
+}
+
+cudaError_t launch_predict_tile(const uint64_t* A, int64_t M, int nw, const uint64_t* PT, int c, int K,
+                                int32_t* labels, unsigned int* timeouts, cudaStream_t st, bool pdl) {
+  Shape s = shape_of(M, TN, TN, sm_count());   // one tile of classes, never split
+  const bool wide = row_align(A, nw) == 16 && row_align(PT, nw) == 16;
+  return launch_tiles(wide ? k_predict_tile<16> : k_predict_tile<8>, s, st, pdl, A, M, nw, PT, c, K, labels,
+                      timeouts, s.pat);
 }
 
 }  // namespace bk

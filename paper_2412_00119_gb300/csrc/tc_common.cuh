@@ -85,16 +85,6 @@ __device__ __forceinline__ void mma_commit(unsigned long long* bar) {
                ::"r"(smem_u32(bar)) : "memory");
 }
 
-// 8 bits -> 8 e4m3 bytes (+1 = 0x38, -1 = 0xB8) as two words.  Byte j of the
-// replicated value keeps bit j of b; adding (0x80 - 2^j) per byte moves it to
-// bit 7 without carries between bytes.
-__device__ __forceinline__ uint2 expand8(uint32_t b) {
-  const uint32_t rep = b * 0x01010101u;
-  const uint32_t lo = (rep & 0x08040201u) + 0x787C7E7Fu;
-  const uint32_t hi = (rep & 0x80402010u) + 0x00406070u;
-  return make_uint2((lo & 0x80808080u) ^ 0xB8B8B8B8u, (hi & 0x80808080u) ^ 0xB8B8B8B8u);
-}
-
 __device__ __forceinline__ void mbar_arrive_tx(unsigned long long* bar, uint32_t bytes) {
   asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}"
                ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
@@ -155,7 +145,7 @@ __host__ __device__ __forceinline__ int row_align(const void* base, int nw) {
   return ((reinterpret_cast<uintptr_t>(base) | (uintptr_t)(8 * (uint32_t)nw)) & 15) == 0 ? 16 : 8;
 }
 
-// Asynchronous copy of kBytes (16 past L1, or 8) to shared memory; zeros
+// Asynchronous copy of kBytes (16 past L1, or 8 or 4) to shared memory; zeros
 // instead when !live (src is then not read, but must be a valid address).
 template <int kBytes>
 __device__ __forceinline__ void cp_async_or_zero(uint32_t dst, const void* src, bool live) {
@@ -163,7 +153,11 @@ __device__ __forceinline__ void cp_async_or_zero(uint32_t dst, const void* src, 
   if constexpr (kBytes == 16)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
   else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %3, %2;" ::"r"(dst), "l"(src), "r"(n), "n"(kBytes) : "memory");
+}
+// Arrive on the barrier when this thread's copies so far have completed.
+__device__ __forceinline__ void cp_async_arrive(unsigned long long* bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 __device__ __forceinline__ uint4 lds128(uint32_t a) {
   uint4 v;
@@ -178,110 +172,43 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
-// A producer item: one 16-byte chunk of one row of a stage, i.e. 16
-// K-elements (two bytes of bits) -> 16 e4m3 bytes.  The chunk's logical index
-// c (K-elements 16c .. 16c + 15 of the stage's 128) is stored at physical
-// chunk c ^ (r % 8) of row r (SWIZZLE_128B).
-struct Chunk {
-  const uint16_t* src;  // the row's bits as 16-bit pieces; null: no item
-  uint32_t dst;         // byte offset of the chunk inside a stage
-  int c;                // logical chunk 0..7
-};
-
-// Item for row r (of a matrix whose rows start `soff` bytes into the stage).
-__device__ __forceinline__ Chunk make_chunk(const uint64_t* row, int soff, int r, int c) {
-  return Chunk{reinterpret_cast<const uint16_t*>(row),
-               (uint32_t)(soff + r * KB + 16 * (c ^ (r & 7))), c};
+// 16 TMEM columns of this warp's 32 lanes.
+__device__ __forceinline__ void tmem_store16(uint32_t taddr, const uint32_t (&v)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
+      "%12, %13, %14, %15, %16};"
+      ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
+        "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]) : "memory");
 }
 
-// The item's 16 bits for k-block kb (0 past the row's nw words).
-__device__ __forceinline__ uint32_t load_chunk(const Chunk& ch, int kb, int nw) {
-  const int pi = 8 * kb + ch.c;
-  return (ch.src != nullptr && pi < 4 * nw) ? (uint32_t)__ldg(ch.src + pi) : 0u;
-}
-
-// Bytes of a 4-byte group to keep when n_ok of its elements are real.
-__device__ __forceinline__ uint32_t keep_mask(int n_ok) {
-  return n_ok >= 4 ? 0xFFFFFFFFu : (n_ok <= 0 ? 0u : ((1u << (8 * n_ok)) - 1u));
-}
-
-// Four K-elements, bits P .. P + 3 of x (P = 0 or 4), as four e4m3 bytes
-// (bit 1 -> 0x38 = +1, bit 0 -> 0xB8 = -1): the product places bit P + j at
-// bit 8 j + 7; its four shifted copies of the masked nibble do not overlap,
-// so it carries nothing.
-template <int P>
-__device__ __forceinline__ uint32_t e4m3_quad(uint32_t x) {
-  static_assert(P == 0 || P == 4, "nibble position");
-  constexpr uint32_t kMul = P == 0 ? 0x10204080u : 0x01020408u;
-  return ((x & (0xFu << P)) * kMul & 0x80808080u) ^ 0xB8B8B8B8u;
-}
-
-// 16 K-elements (bits 0..15 of h) -> one 16-byte chunk.
-__device__ __forceinline__ uint4 chunk16(uint32_t h) {
-  return make_uint4(e4m3_quad<0>(h), e4m3_quad<4>(h), e4m3_quad<0>(h >> 8), e4m3_quad<4>(h >> 8));
-}
-
-// The same with the elements at index >= valid set to 0 (ragged K only).
-__device__ __forceinline__ uint4 chunk16_masked(uint32_t h, int valid) {
-  uint4 v = chunk16(h);
-  v.x &= keep_mask(valid);
-  v.y &= keep_mask(valid - 4);
-  v.z &= keep_mask(valid - 8);
-  v.w &= keep_mask(valid - 12);
-  return v;
-}
-
-// Expand the item's bits into its stage chunk; elements at K >= Kin are 0.
-__device__ __forceinline__ void store_chunk(uint8_t* stage, const Chunk& ch, uint32_t bits, int kb,
-                                            int Kin) {
-  const uint2 e0 = expand8(bits & 0xFFu);
-  const uint2 e1 = expand8(bits >> 8);
-  uint4 v = make_uint4(e0.x, e0.y, e1.x, e1.y);
-  const int valid = Kin - (KB * kb + 16 * ch.c);
-  if (valid < 16) {
-    v.x &= keep_mask(valid);
-    v.y &= keep_mask(valid - 4);
-    v.z &= keep_mask(valid - 8);
-    v.w &= keep_mask(valid - 12);
-  }
-  *reinterpret_cast<uint4*>(stage + ch.dst) = v;
-}
-
-// A producer item of 64 K-elements: one (row, half) of a stage row, i.e. one
-// 64-bit word of bits -> four 16-byte chunks (chunks 4 half .. 4 half + 3).
-struct Item {
-  const uint64_t* src;  // row start (bit words), or null when the thread has no item
-  uint32_t dst;         // byte offset of the row inside a stage
-  int r;                // row index inside its matrix (for the swizzle)
-  int half;             // which of the stage's two words
-};
-
-__device__ __forceinline__ uint64_t load_word(const Item& it, int kb, int nw) {
-  const int wi = 2 * kb + it.half;
-  return (it.src != nullptr && wi < nw) ? __ldg(it.src + wi) : 0ull;
-}
-
-// Expand the item's word for k-block kb into its four chunks; elements at
-// K >= Kin are 0.
-__device__ __forceinline__ void store_word(uint8_t* stage, const Item& it, uint64_t w, int kb,
-                                           int Kin) {
-  const int valid = Kin - (KB * kb + 64 * it.half);
+// 32 TMEM columns of this warp's 32 lanes from each lane's 256 bits.
+__device__ __forceinline__ void tmem_store_row256(uint32_t taddr, const uint32_t (&x)[8]) {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {  // chunk 4 half + q: elements 16 q .. 16 q + 15 of the word
-    const uint32_t bits = (uint32_t)(w >> (16 * q)) & 0xFFFFu;
-    const uint2 e0 = expand8(bits & 0xFFu);
-    const uint2 e1 = expand8(bits >> 8);
-    uint4 v = make_uint4(e0.x, e0.y, e1.x, e1.y);
-    if (valid < 64) {
-      const int n = valid - 16 * q;
-      v.x &= keep_mask(n);
-      v.y &= keep_mask(n - 4);
-      v.z &= keep_mask(n - 8);
-      v.w &= keep_mask(n - 12);
+  for (int h = 0; h < 2; ++h) {   // 16 columns at a time (registers)
+    uint32_t v[16];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      uint32_t w[4];
+      e2m1_words(x[4 * h + q], w);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[4 * q + j] = w[j];
     }
-    const int c = 4 * it.half + q;
-    *reinterpret_cast<uint4*>(stage + it.dst + 16 * (c ^ (it.r & 7))) = v;
+    tmem_store16(taddr + 16u * (uint32_t)h, v);
   }
+}
+
+// 32 TMEM columns of this warp's 32 lanes, waited for.
+__device__ __forceinline__ void tmem_load32(uint32_t (&v)[32], uint32_t taddr) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+        "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
+        "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]),
+        "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]),
+        "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
 }  // namespace tc

@@ -57,3 +57,40 @@ def test_small_batch_forward(K, N, n):
     B.bmlp_layer_forward(gpu.h, 1, x2, out)
     assert np.array_equal(out.cpu().numpy().view(np.uint64), want)
     gpu.close()
+
+
+# more than 512 patterns: pairs of CTAs on 256 x 256 tiles, several tiles per pair
+LARGE = [(1, 1, 513), (255, 255, 700), (784, 257, 1300), (1000, 525, 2000), (2049, 300, 1025),
+         (4096, 512, 900), (32767, 33, 600), (64, 2048, 11000)]
+
+
+@pytest.mark.parametrize("K,N,n", LARGE)
+def test_large_batch_forward(K, N, n):
+    gpu = B.BMLP((K, N), 4, seed=K + N, bs=64)
+    ref = O.OracleModel([K, N], 4, seed=K + N, bs=64)
+    xp = W.random_packed(n, n, K)
+    _, a = O.layer_forward(W.unpack(xp, K), ref.H(1))
+    out = torch.full((n, W.words(N)), -1, dtype=torch.int64, device=DEV)
+    x2 = np.array(xp)
+    if K % 64:
+        x2[:, -1] |= ~np.uint64((1 << (K % 64)) - 1)   # pad bits set: ignored
+    B.bmlp_layer_forward(gpu.h, 1, dev(x2), out)
+    assert np.array_equal(out.cpu().numpy().view(np.uint64), W.pack(a))
+    gpu.close()
+
+
+@pytest.mark.parametrize("classes", [2, 33, 100, 128, 129])
+@pytest.mark.parametrize("n", [1, 113, 700])
+def test_labels_of_every_layer(classes, n):
+    widths = [300, 257, 1030]
+    gpu = B.BMLP(widths, classes, seed=classes, bs=64)
+    ref = O.OracleModel(widths, classes, seed=classes, bs=64)
+    xp = W.random_packed(7 * n, n, widths[0])
+    x = W.unpack(xp, widths[0])
+    out = torch.full((2, n), -1, dtype=torch.int32, device=DEV)
+    gpu.predict_layers(dev(xp), out)
+    assert np.array_equal(out.cpu().numpy(), ref.predict_layers(x))
+    last = torch.full((n,), -1, dtype=torch.int32, device=DEV)
+    gpu.predict(dev(xp), last)
+    assert np.array_equal(last.cpu().numpy(), ref.predict(x))
+    gpu.close()
