@@ -94,3 +94,21 @@ def test_labels_of_every_layer(classes, n):
     gpu.predict(dev(xp), last)
     assert np.array_equal(last.cpu().numpy(), ref.predict(x))
     gpu.close()
+
+
+# widths at every change of registers per lane and warps per pattern
+@pytest.mark.parametrize("K", [1, 2, 31, 33, 256, 257, 512, 513, 799, 800, 801, 1024, 1025, 2048, 2049, 4096, 4097])
+@pytest.mark.parametrize("kind", ["pixels", "gauss", "ties", "wide"])
+def test_binarize_edges(K, kind):
+    n = 37
+    if kind == "wide":   # every magnitude, infinities, constant rows, denormals
+        rng = np.random.default_rng(K)
+        x = (rng.standard_normal((n, K)) * 10.0 ** rng.uniform(-40, 38, (n, K))).astype(np.float32)
+        x[0] = 3.0
+        x[1, ::2], x[1, 1::2] = np.float32(np.inf), np.float32(-np.inf)
+        x[2, : K // 2] = np.float32(-0.0)
+    else:
+        x = W.real_patterns(K, n, K, kind)
+    out = torch.full((n, W.words(K)), -1, dtype=torch.int64, device=DEV)
+    B.bmlp_binarize_median(torch.from_numpy(x).to(DEV), out)
+    assert np.array_equal(out.cpu().numpy().view(np.uint64), W.pack(O.binarize_median(x)))
