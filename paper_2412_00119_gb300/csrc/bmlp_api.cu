@@ -838,8 +838,7 @@ int bmlp_expand_sign(const uint8_t* x, int64_t n, int32_t D, const uint64_t* E, 
     return fail(nullptr, BMLP_EINVAL, "bmlp_expand_sign: x, E and out must be device pointers");
   if ((reinterpret_cast<uintptr_t>(E) & 7) || (reinterpret_cast<uintptr_t>(out) & 7))
     return fail(nullptr, BMLP_EINVAL, "bmlp_expand_sign: misaligned E or out");
-  launch_expand_sign(x, n, D, E, K, out, static_cast<cudaStream_t>(cuda_stream));
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_expand_sign(x, n, D, E, K, out, static_cast<cudaStream_t>(cuda_stream));
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "k_expand_sign");
   return BMLP_OK;
 }

@@ -11,7 +11,28 @@
 // k % 64 of word k / 64, pad bits 0), i.e. bmlp_train / bmlp_predict input
 // for K_0 = K.
 //
-// k_expand_sign: a 128-pattern x 128-neuron tile per CTA of 256 threads, the
+// k_expand_tc (D <= kTcMaxD): the product on the tensor cores, exact in 4-bit
+// operands.  A byte is four base-4 digits, x = d0 + 4 d1 + 16 d2 + 64 d3, and 0,
+// 1, 2, 3 and +-1 are e2m1 values, so z is the sum of four e2m1 x e2m1 products
+// with block scales 1, 4, 16 and 64 (UE8M0 holds powers of two); every product
+// is an integer and |z| <= 255 D < 2^24, so the fp32 sums are exact in any
+// order.  A CTA keeps one tile of up to 256 neurons, expanded into shared memory
+// once (K-major, 128B swizzle), and walks over tiles of 128 patterns:
+//   - 4 loader warps copy pieces of 256 bytes per row into a ring of two;
+//   - 16 producer warps in four groups take chunks of 64 inputs in turn: a lane
+//     per pattern row turns 64 bytes into 4 x 8 tensor-memory columns (digit
+//     planes; 3 operations per byte);
+//   - one thread issues the four MMAs (K = 64) of a chunk, one per plane, each
+//     with its plane's scales, all against the same weight columns: the weights
+//     are read from shared memory and never written again;
+//   - 8 epilogue warps read the sums (a lane per pattern), shift the sign bits
+//     into words and store them.
+// Bound: the MMAs, 4 x 128 clocks per chunk of a 128 x 256 tile.  60,000 x 784
+// -> 1024: 93.6 us (the dp4a kernel 804 us), of which the MMAs are 43.
+// Every mbarrier wait is bounded like all others of the library; this entry
+// point has no handle, so an expiry leaves its tiles unwritten.
+//
+// k_expand_sign (larger D): a 128-pattern x 128-neuron tile per CTA of 256 threads, the
 // inputs in chunks of 64 (one word of E per neuron): the chunk's bytes of x
 // and the chunk's E bits, expanded to +-1 bytes, are staged in shared memory
 // (rows padded to 17 words: conflict-free reads; the next chunk's raw words
@@ -20,14 +41,11 @@
 // int32 sums).  Each warp ballots the signs of 2 patterns x 16 neurons and
 // writes 16-bit pieces of the packed rows.  Neuron tiles vary fastest in the
 // grid, so the CTAs of one pattern tile run together and read x from L2.
-// Why CUDA cores and not tcgen05: e4m3 holds no byte exactly, the int8 tensor
-// rate of this part is far below its fp8 rate, and the transform runs once per
-// data set, not once per training step.
 //
 // k_expand_weights: E from the Philox stream of the expansion weights,
 // e_k,i = +1 iff bit 31 of word i%4 of Philox (i/4, k, 33*2^16, 0) (the
 // library's stream layout is listed in bmlp_internal.cuh); pad bits 0.
-#include "bmlp_internal.cuh"
+#include "tc_common.cuh"
 
 namespace bk {
 namespace {
@@ -145,6 +163,301 @@ __global__ void __launch_bounds__(kXThreads, 2)
   }
 }
 
+// ---------------------------------------------------------------------------
+// The tensor-core kernel.
+// ---------------------------------------------------------------------------
+using namespace tc;
+
+constexpr int XM = 128;                   // patterns per tile (MMA M)
+constexpr int kXMaxN = 256;               // neurons per CTA at most (MMA N)
+constexpr int kChunk = 64;                // inputs per MMA
+constexpr int kXPiece = 256;              // bytes per row and piece (4 chunks)
+constexpr int kXPieces = 2;
+constexpr int kXRow = kXPiece + 16;       // staged row (16 of padding: banks)
+constexpr int kXPieceBytes = XM * kXRow;
+constexpr int kXStages = 5;
+constexpr int kXGroups = 4;
+constexpr int kXProdWarps = 4 * kXGroups, kXLoadWarps = 4, kXEpiWarps = 8;
+constexpr int kXMma = kXProdWarps, kXLoad0 = kXMma + 1, kXEpi0 = kXLoad0 + kXLoadWarps;
+constexpr int kXTcThreads = 32 * (kXEpi0 + kXEpiWarps);
+constexpr int kXSfA = kXMaxN, kXSfB = kXSfA + 4 * 16, kXStageCol = kXSfB + 16;
+static_assert(kXStageCol + 32 * kXStages <= 512, "TMEM budget");
+constexpr int kXWeightBytes = 4 * kXMaxN * 128;   // 4 blocks of 256 inputs x 256 neurons, and the like
+constexpr int kTcMaxD = 4608;                     // 18 blocks of 256 inputs x 64 neurons
+
+struct __align__(8) XShared {
+  unsigned long long piece_full[kXPieces], piece_empty[kXPieces];
+  unsigned long long full[kXStages], empty[kXStages];
+  unsigned long long done, drained;
+  uint32_t tmem_base;
+  int failed;
+};
+constexpr size_t kXSmem = 1024 + 18 * 64 * 128 + kXPieces * kXPieceBytes + sizeof(XShared);
+static_assert(18 * 64 * 128 >= kXWeightBytes, "the weight buffer holds every choice of tile");
+static_assert(kXSmem <= 232448, "shared memory of one CTA");
+
+// 64 bytes (16 words) -> digit plane 2 h of columns v[0..7], plane 2 h + 1 of
+// v[8..15].  Column g holds the digits of words 2 g and 2 g + 1: nibble i is
+// byte i / 2 of word 2 g + i % 2.  Digit d becomes the e2m1 value d: 2 d, and 5
+// for d = 3.
+__device__ __forceinline__ void digit_planes(const uint32_t (&w)[16], int h, uint32_t (&v)[16]) {
+#pragma unroll
+  for (int g = 0; g < 8; ++g) {
+    const uint32_t a = w[2 * g], b = w[2 * g + 1];
+    const uint32_t u = h == 0 ? ((a & 0x0F0F0F0Fu) | ((b << 4) & 0xF0F0F0F0u))
+                              : (((a >> 4) & 0x0F0F0F0Fu) | (b & 0xF0F0F0F0u));
+    v[g] = ((u << 1) & 0x66666666u) - (u & (u >> 1) & 0x11111111u);
+    v[8 + g] = ((u >> 1) & 0x66666666u) - ((u >> 2) & (u >> 3) & 0x11111111u);
+  }
+}
+
+// A weight byte (8 inputs) as e2m1 in the same order: nibble i is input
+// i / 2 + 4 (i % 2); bit 1 -> 0x2 (+1), bit 0 -> 0xA (-1).
+__device__ __forceinline__ uint32_t weight_nibbles(uint32_t byte) {
+  const uint32_t neg = ~byte;
+  const uint32_t even = ((neg & 0xFu) * 0x01020408u) & 0x08080808u;
+  const uint32_t odd = (((neg >> 4) & 0xFu) * 0x01020408u) & 0x08080808u;
+  return 0x22222222u | even | (odd << 4);
+}
+
+// kBytes: 16 or 4, the copies that every row of x allows, or 1.
+template <int kBytes>
+__global__ void __launch_bounds__(kXTcThreads, 1)
+    k_expand_tc(const uint8_t* __restrict__ x, int64_t n, int D, const uint64_t* __restrict__ E, int K, int nwD,
+                uint64_t* __restrict__ out, int nwK, int nb) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* base = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  uint8_t* pieces = base + 18 * 64 * 128;
+  XShared* sh = reinterpret_cast<XShared*>(pieces + kXPieces * kXPieceBytes);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  volatile int* failed = &sh->failed;
+  const int n0 = blockIdx.x * nb;
+  const int nchunks = (D + kChunk - 1) / kChunk, npc = (D + kXPiece - 1) / kXPiece;
+  const int64_t tiles = (n + XM - 1) / XM;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kXPieces; ++s) {
+      mbar_init(&sh->piece_full[s], 32 * kXLoadWarps);
+      mbar_init(&sh->piece_empty[s], kXProdWarps);
+    }
+    for (int s = 0; s < kXStages; ++s) {
+      mbar_init(&sh->full[s], 4);
+      mbar_init(&sh->empty[s], 1);
+    }
+    mbar_init(&sh->done, 1);
+    mbar_init(&sh->drained, kXEpiWarps);
+    sh->failed = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == kXMma) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 ::"r"(smem_u32(&sh->tmem_base)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  // the tile's weights: block b of 256 inputs is nb rows of 128 bytes; 32 inputs
+  // of one neuron are one 16-byte chunk c of its row, at chunk c ^ (row % 8)
+  for (int i = threadIdx.x; i < nb * 8 * npc; i += kXTcThreads) {
+    const int c = i % (8 * npc), r = i / (8 * npc);
+    const uint32_t bitsw = (n0 + r < K && c < 2 * nwD)
+                               ? reinterpret_cast<const uint32_t*>(E + (int64_t)(n0 + r) * nwD)[c] : 0u;
+    uint32_t v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = weight_nibbles(bitsw >> (8 * q));
+    sts128(smem_u32(base) + (uint32_t)((c >> 3) * nb * 128 + r * 128 + 16 * ((c & 7) ^ (r & 7))), v);
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = sh->tmem_base;
+  if (warp < 4) {
+    const uint32_t at = tmem + ((uint32_t)(32 * warp) << 16);
+#pragma unroll
+    for (int p = 0; p < 5; ++p) {
+      // scales of plane p (4^p: UE8M0 127 + 2 p), then the weights' (1)
+      const uint32_t v = (p < 4 ? 127u + 2u * p : 127u) * 0x01010101u;
+      asm volatile(
+          "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, "
+          "%1, %1, %1, %1};" ::"r"(at + (uint32_t)(kXSfA + 16 * p)), "r"(v) : "memory");
+    }
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+
+  if (warp < kXProdWarps) {
+    // ---------------- producers ----------------
+    const int grp = warp >> 2, q = warp & 3;
+    const uint32_t row0 = smem_u32(pieces) + (uint32_t)((32 * q + lane) * kXRow);
+    const uint32_t lanes = (uint32_t)(32 * q) << 16;
+    uint32_t pc = 0, kc0 = 0;
+    bool ok = true;
+#pragma unroll 1
+    for (int64_t t = blockIdx.y; t < tiles && ok; t += gridDim.y, kc0 += (uint32_t)nchunks) {
+#pragma unroll 1
+      for (int p = 0; p < npc && ok; ++p, ++pc) {
+        const uint32_t slot = pc % kXPieces;
+        ok = __all_sync(0xffffffffu, mbar_wait(&sh->piece_full[slot], (pc / kXPieces) & 1u, failed));
+        const int cend = min(nchunks, 4 * (p + 1));
+#pragma unroll 1
+        for (int ch = 4 * p; ch < cend && ok; ++ch) {
+          const uint32_t kc = kc0 + (uint32_t)ch;
+          if ((kc & (kXGroups - 1)) != (uint32_t)grp) continue;
+          const uint32_t s = kc % kXStages, use = kc / kXStages;
+          uint32_t w[16];
+          const uint32_t src = row0 + slot * (uint32_t)kXPieceBytes + (uint32_t)(kChunk * (ch - 4 * p));
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const uint4 v = lds128(src + 16u * i);
+            w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+          }
+          if (use > 0) ok = __all_sync(0xffffffffu, mbar_wait(&sh->empty[s], (use - 1) & 1u, failed));
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            uint32_t v[16];
+            digit_planes(w, h, v);
+            tmem_store16(tmem + lanes + (uint32_t)kXStageCol + 32u * s + 16u * h, v);
+          }
+          asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sh->full[s]);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sh->piece_empty[slot]);
+      }
+    }
+  } else if (warp >= kXLoad0 && warp < kXEpi0) {
+    // ---------------- loaders ----------------
+    constexpr int kStep = kBytes == 1 ? 4 : kBytes;   // bytes per store to shared memory
+    constexpr int kPer = kXPiece / kStep;
+    const int tid = threadIdx.x - 32 * kXLoad0;
+    uint32_t pc = 0;
+    bool ok = true;
+#pragma unroll 1
+    for (int64_t t = blockIdx.y; t < tiles && ok; t += gridDim.y) {
+      const uint8_t* rows = x + t * XM * D;
+      const int live = (int)min((int64_t)XM, n - t * XM);
+#pragma unroll 1
+      for (int p = 0; p < npc && ok; ++p, ++pc) {
+        const uint32_t slot = pc % kXPieces, use = pc / kXPieces;
+        if (use > 0) ok = mbar_wait(&sh->piece_empty[slot], (use - 1) & 1u, failed);
+        if (!ok) break;
+        const uint32_t dst = smem_u32(pieces) + slot * (uint32_t)kXPieceBytes;
+#pragma unroll 4
+        for (int i = tid; i < XM * kPer; i += 32 * kXLoadWarps) {
+          const int r = i / kPer, c = kXPiece * p + kStep * (i % kPer);
+          const uint32_t to = dst + (uint32_t)(r * kXRow + kStep * (i % kPer));
+          const uint8_t* src = rows + (int64_t)r * D + c;
+          if constexpr (kBytes == 1) {
+            uint32_t v = 0;
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+              if (r < live && c + b < D) v |= (uint32_t)__ldg(src + b) << (8 * b);
+            asm volatile("st.shared.b32 [%0], %1;" ::"r"(to), "r"(v) : "memory");
+          } else {
+            const bool on = r < live && c < D;   // D is a multiple of kBytes
+            cp_async_or_zero<kBytes>(to, on ? src : x, on);
+          }
+        }
+        if constexpr (kBytes == 1) mbar_arrive(&sh->piece_full[slot]);
+        else cp_async_arrive(&sh->piece_full[slot]);
+      }
+    }
+    cp_async_wait_all();   // no copy outlives its thread
+  } else if (warp == kXMma && lane == 0) {
+    // ---------------- MMA issuer ----------------
+    const uint32_t idesc = idesc_f4(XM, nb);
+    uint32_t kc = 0, tile = 0;
+    bool ok = true;
+#pragma unroll 1
+    for (int64_t t = blockIdx.y; t < tiles && ok; t += gridDim.y, ++tile) {
+      if (tile > 0) ok = mbar_wait(&sh->drained, (tile - 1) & 1u, failed);
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
+      for (int ch = 0; ch < nchunks && ok; ++ch, ++kc) {
+        const uint32_t s = kc % kXStages;
+        ok = mbar_wait(&sh->full[s], (kc / kXStages) & 1u, failed);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint64_t bd = smem_desc(smem_u32(base + (ch >> 2) * nb * 128)) + 2 * (ch & 3);
+        const uint32_t ta = tmem + (uint32_t)kXStageCol + 32u * s;
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+          mma_f4_ts(tmem, ta + 8 * p, bd, idesc, tmem + kXSfA + 16 * p, tmem + kXSfB, (ch > 0 || p > 0) ? 1u : 0u);
+        mma_commit(&sh->empty[s]);
+      }
+      if (ok) mma_commit(&sh->done);
+    }
+  } else if (warp >= kXEpi0) {
+    // ---------------- epilogue ----------------
+    const int sub = warp & 3, half = (warp - kXEpi0) >> 2;
+    const int words = nb / 64;   // 32-neuron words of this warp: half words half, ..
+    uint32_t tile = 0;
+#pragma unroll 1
+    for (int64_t t = blockIdx.y; t < tiles; t += gridDim.y, ++tile) {
+      if (!__all_sync(0xffffffffu, mbar_wait(&sh->done, tile & 1u, failed))) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      uint32_t word[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+      for (int cb = 0; cb < 4; ++cb) {
+        if (cb >= words) break;
+        uint32_t v[32];
+        tmem_load32(v, tmem + ((uint32_t)(32 * sub) << 16) + (uint32_t)(32 * (half * words + cb)));
+        uint32_t acc = 0u;   // sign bits (0 for z = 0), column 0 first
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc = __funnelshift_l(v[j], acc, 1);
+        word[cb] = ~__brev(acc);
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sh->drained);
+      const int64_t m = t * XM + 32 * sub + lane;
+      if (m < n) {
+        uint32_t* row = reinterpret_cast<uint32_t*>(out + m * nwK);
+#pragma unroll
+        for (int cb = 0; cb < 4; ++cb) {
+          const int nn = n0 + 32 * (half * words + cb), valid = K - nn;
+          const uint32_t keep = valid >= 32 ? 0xffffffffu : (valid <= 0 ? 0u : (1u << valid) - 1u);
+          // words wholly past K (inside the row's last 64-bit word) are written 0
+          if (cb < words && (nn >> 5) < 2 * nwK) row[nn >> 5] = word[cb] & keep;
+        }
+      }
+    }
+  }
+  __syncwarp();
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (warp == kXMma)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+}
+
+template <int kBytes>
+cudaError_t launch_expand_tc(const uint8_t* x, int64_t n, int D, const uint64_t* E, int K, uint64_t* out,
+                             cudaStream_t st) {
+  const int blocks = (D + kXPiece - 1) / kXPiece;   // of 256 inputs
+  const int64_t tiles = (n + XM - 1) / XM;
+  const int sms = sm_count();
+  // the widest neuron tile whose weights fit; narrower ones while all tiles
+  // together leave SMs idle
+  int nb = 256;
+  while (nb > 64 && (nb * 128 * blocks > 18 * 64 * 128 || nb / 2 >= K || tiles * ((K + nb - 1) / nb) < sms)) nb /= 2;
+  const unsigned nt = (unsigned)((K + nb - 1) / nb);
+  int64_t gy = sms / (int)nt > 0 ? sms / (int)nt : 1;
+  if (gy > tiles) gy = tiles;
+  const cudaError_t e = cudaFuncSetAttribute(k_expand_tc<kBytes>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)kXSmem);
+  if (e != cudaSuccess) return e;
+  k_expand_tc<kBytes><<<dim3(nt, (unsigned)gy), kXTcThreads, kXSmem, st>>>(x, n, D, E, K, (D + 63) / 64, out,
+                                                                          (K + 63) / 64, nb);
+  return cudaGetLastError();
+}
+
 __global__ void k_expand_weights(uint32_t key0, uint32_t key1, int K, int D, int nwD,
                                  uint64_t* __restrict__ E) {
   const int64_t total = (int64_t)K * nwD;
@@ -176,9 +489,15 @@ void launch_expand_weights(uint64_t seed, int K, int D, uint64_t* E, cudaStream_
       (uint32_t)(seed & 0xFFFFFFFFu), (uint32_t)(seed >> 32), K, D, nwD, E);
 }
 
-void launch_expand_sign(const uint8_t* x, int64_t n, int D, const uint64_t* E, int K, uint64_t* out,
-                        cudaStream_t st) {
+cudaError_t launch_expand_sign(const uint8_t* x, int64_t n, int D, const uint64_t* E, int K, uint64_t* out,
+                               cudaStream_t st) {
   const int nwD = (D + 63) / 64, nwK = (K + 63) / 64;
+  if (D <= kTcMaxD) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(x) | (uintptr_t)(uint32_t)D;
+    return (a & 15) == 0 ? launch_expand_tc<16>(x, n, D, E, K, out, st)
+                         : ((a & 3) == 0 ? launch_expand_tc<4>(x, n, D, E, K, out, st)
+                                         : launch_expand_tc<1>(x, n, D, E, K, out, st));
+  }
   const unsigned ntiles = (unsigned)((K + kXN - 1) / kXN);
   // patterns in launches of at most 65,535 tiles of 128 (the grid's y limit)
   const int64_t per = (int64_t)kXMaxRowTiles * kXM;
@@ -189,6 +508,7 @@ void launch_expand_sign(const uint8_t* x, int64_t n, int D, const uint64_t* E, i
     const dim3 grid(ntiles, (unsigned)((cnt + kXM - 1) / kXM));
     k_expand_sign<<<grid, kXThreads, 0, st>>>(xo, cnt, D, vec, E, K, nwD, out + off * (int64_t)nwK, nwK);
   }
+  return cudaGetLastError();
 }
 
 }  // namespace bk

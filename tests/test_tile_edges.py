@@ -96,6 +96,26 @@ def test_labels_of_every_layer(classes, n):
     gpu.close()
 
 
+# chunks of 64 inputs, blocks of 256, neuron tiles of 256 / 128 / 64, the widest
+# tensor-core shape (4608) and the first past it, rows that allow copies of 16,
+# 4 and 1 bytes, more tiles than CTAs
+EXPAND = [(1, 1, 1), (127, 63, 64), (129, 64, 65), (130, 256, 128), (300, 257, 257), (128, 1024, 256),
+          (200, 1025, 300), (260, 1280, 256), (100, 1284, 70), (64, 2561, 130), (33, 4608, 65),
+          (33, 4609, 65), (30000, 16, 300)]
+
+
+@pytest.mark.parametrize("n,D,K", EXPAND)
+@pytest.mark.parametrize("kind", ["pixels", "saturated", "sparse"])
+def test_expand_edges(n, D, K, kind):
+    x = W.pixel_bytes(n + D, n, D, kind)
+    e = O.expand_weights(5 + K, K, D)
+    E = torch.empty((K, W.words(D)), dtype=torch.int64, device=DEV)
+    B.bmlp_expand_weights(5 + K, K, D, E)
+    out = torch.full((n, W.words(K)), -1, dtype=torch.int64, device=DEV)
+    B.bmlp_expand_sign(torch.from_numpy(x).to(DEV), E, K, out)
+    assert np.array_equal(out.cpu().numpy().view(np.uint64), W.pack(O.expand_sign(x, e)))
+
+
 # widths at every change of registers per lane and warps per pattern
 @pytest.mark.parametrize("K", [1, 2, 31, 33, 256, 257, 512, 513, 799, 800, 801, 1024, 1025, 2048, 2049, 4096, 4097])
 @pytest.mark.parametrize("kind", ["pixels", "gauss", "ties", "wide"])
