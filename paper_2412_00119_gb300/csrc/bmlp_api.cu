@@ -87,8 +87,9 @@ struct bmlp {
   cudaStream_t capStream = nullptr;
   cudaStream_t sideStream = nullptr;  // the event-draw branch of the step graph
   cudaEvent_t evFork = nullptr, evJoin = nullptr;
-  int updCtas = 0;
-  size_t updSmem = 0;
+  UpdArgs upd{};
+  unsigned updCtas = 0, evCtas = 0;
+  bool updRing = false;   // the update streams through a shared-memory ring (large models)
   // profiling
   bool profiling = false;       // events around the kernels being enqueued now
   int32_t profEvery = 0;        // 0 off, 1 every mini-batch, S every S-th mini-batch
@@ -237,26 +238,24 @@ int prof_collect(bmlp_t* h, cudaStream_t st) {
 // Mini-batch steps per captured training graph (a shorter run, or one that
 // has sampled steps in the way, uses the one-step graph).
 constexpr int kGraphSteps = 8;
+// Models of more hidden weights than this update through the shared-memory ring
+// with their events drawn by a kernel of its own on a branch of the graph; the
+// others in one kernel that draws them too.  Step time at bs 100 (us), ring with
+// branch / one kernel: 63 M weights (3072-4096x4) 67.0 / 70.4, 105 M (5120x4) 98.7 /
+// 113.6, 268 M (8192x4) 152.7 / 198.7; 2.9 M (784-1024x3) 41.3 / 30.0, and at 15 M
+// (3072-2048x3) the ring alone, without the draws, 36.7 / 35.5.
+constexpr int64_t kRowsWeights = 20ll << 20;
 
 // One mini-batch step.  fork: the graph form (event draws on a branch,
 // programmatic dependent launches); chained: the step follows another step in
 // the same graph, so its first forward is a dependent of that step's update.
 int enqueue_step(bmlp_t* h, cudaStream_t st, bool fork, bool chained = false) {
-  if (!fork) {
-    prof_begin(h, kProfEvents, st);
-    launch_r_events((unsigned)h->hp.ev_ctas_total, st, h->dP, h->hp.key0, h->hp.key1);
-    prof_end(h, st);
-  }
-  // one hidden layer whose forward pass leaves most SMs free (at most 64
-  // CTAs): the event draws start with the step
-  const bool early = h->L == 1 && ((h->K[1] + 255) / 256) * 4 <= 64;
   for (int l = 1; l <= h->L; ++l) {
-    if (fork && l == (early ? 1 : 2)) {
-      // otherwise fork after the first forward pass: its CTAs hold the SMs,
-      // and the event draws and the second pass become ready together
+    if (fork && h->updRing && l == 2) {
+      // the events are drawn on a branch beside the other layers' passes
       CK(h, cudaEventRecord(h->evFork, st));
       CK(h, cudaStreamWaitEvent(h->sideStream, h->evFork, 0));
-      launch_r_events((unsigned)h->hp.ev_ctas_total, h->sideStream, h->dP, h->hp.key0, h->hp.key1);
+      launch_r_events(h->evCtas, h->sideStream, h->dP, h->hp.key0, h->hp.key1);
       CK(h, cudaEventRecord(h->evJoin, h->sideStream));
     }
     prof_begin(h, kProfTrainFwd, st);
@@ -277,15 +276,17 @@ int enqueue_step(bmlp_t* h, cudaStream_t st, bool fork, bool chained = false) {
   CK(h, launch_kernel(k_cls_select, dim3((unsigned)h->bs, (unsigned)h->L), dim3(kClsThreads), 0, st,
                       fork && h->fwd_impl == BMLP_FWD_TCGEN05, h->dP));
   prof_end(h, st);
-  if (fork && h->L == 1 && !early) {
-    CK(h, cudaEventRecord(h->evFork, st));
-    CK(h, cudaStreamWaitEvent(h->sideStream, h->evFork, 0));
-    launch_r_events((unsigned)h->hp.ev_ctas_total, h->sideStream, h->dP, h->hp.key0, h->hp.key1);
-    CK(h, cudaEventRecord(h->evJoin, h->sideStream));
+  if (fork && h->updRing && h->L > 1) CK(h, cudaStreamWaitEvent(st, h->evJoin, 0));
+  if (h->updRing && (!fork || h->L == 1)) {
+    prof_begin(h, kProfEvents, st);
+    launch_r_events(h->evCtas, st, h->dP, h->hp.key0, h->hp.key1);
+    prof_end(h, st);
   }
-  if (fork) CK(h, cudaStreamWaitEvent(st, h->evJoin, 0));
   prof_begin(h, kProfUpd, st);
-  CK(h, launch_update_ws(h->hp.nplanes, h->h_max, h->bs, (unsigned)h->updCtas, st, fork, h->dP));
+  if (h->updRing)
+    CK(h, launch_update_ws(h->hp.nplanes, h->h_max, h->bs, (unsigned)sm_count(), st, fork, h->dP));
+  else
+    CK(h, launch_update_rows(h->hp.nplanes, h->updCtas, st, fork, h->upd));
   prof_end(h, st);
   CK(h, cudaGetLastError());
   return BMLP_OK;
@@ -364,7 +365,7 @@ int run_steps(bmlp_t* h, const uint64_t* xd, const int32_t* yd, int64_t n, cudaS
     s += multi ? kGraphSteps : 1;
   }
   h->profiling = h->profEvery > 0;
-  h->launches += steps * (h->L + 3 + (h->group_mode == BMLP_GROUPS_RESHUFFLED ? 1 : 0));
+  h->launches += steps * (h->L + 2 + (h->group_mode == BMLP_GROUPS_RESHUFFLED ? 1 : 0));
   h->t_host += steps;
   return BMLP_OK;
 }
@@ -518,7 +519,9 @@ int bmlp_create(const int32_t* widths, int32_t n_widths, int32_t classes, int16_
   P.nplanes = upd::planes_of(P.nbits);
   P.key0 = (uint32_t)(seed & 0xffffffffu);
   P.key1 = (uint32_t)(seed >> 32);
-  int ev_cta = 0, rows_total = 0;
+  UpdArgs& U = h->upd;
+  int upd_cta = 0, ev_cta = 0;
+  int64_t weights = 0;
   for (int l = 1; l <= L; ++l) {
     DevLayer& D = P.layer[l - 1];
     D.Kin = h->K[l - 1]; D.Kout = h->K[l];
@@ -526,9 +529,9 @@ int bmlp_create(const int32_t* widths, int32_t n_widths, int32_t classes, int16_
     D.ngrp = (D.Kin + 31) / 32;
     D.ldh = (D.ngrp * P.nplanes + 3) & ~3;
     D.gamma = gam[l]; D.G = D.Kout / D.gamma;
-    D.row_base = rows_total;
-    rows_total += D.Kout;
     D.ev_cta_base = ev_cta;
+    D.row_base = P.rows_total;
+    P.rows_total += D.Kout;
     ev_cta += (D.Kout + kEvRowsPerCta - 1) / kEvRowsPerCta;
     D.nblk = (D.Kin + 63) / 64;
     D.ev_stride = (D.nblk + 1) & ~1;
@@ -548,24 +551,31 @@ int bmlp_create(const int32_t* widths, int32_t n_widths, int32_t classes, int16_
         ((rc = dalloc(h, &D.member, (size_t)D.Kout)) || (rc = dalloc(h, &D.group_of, (size_t)D.Kout))))
       return bail(rc);
   }
-  P.rows_total = rows_total;
-  P.ev_ctas_total = ev_cta;
   P.nblk_max = 0;
   for (int l = 1; l <= L; ++l) P.nblk_max = std::max(P.nblk_max, (widths[l - 1] + 63) / 64);
-  {
-    // the update grid is persistent, one CTA per SM (its slot ring fills most
-    // of the shared memory)
-    h->updSmem = update_ws_smem(P.nplanes, bs);
-    const cudaError_t ea = prepare_update_ws();
-    if (ea != cudaSuccess) return bail(cuda_fail(h, ea, "update kernel shared memory attribute"));
-    h->updCtas = prop.multiProcessorCount;
-    P.upd_ctas_total = h->updCtas;
-  }
   if ((rc = dalloc(h, &h->dP, 1)) || (rc = dalloc(h, &h->dCtrl, 1)) ||
       (rc = dalloc(h, &h->dRT, BMLP_MAX_LAYERS)))
     return bail(rc);
   P.ctrl = h->dCtrl;
   P.rt = h->dRT;
+  for (int l = 1; l <= L; ++l) {
+    const DevLayer& D = P.layer[l - 1];
+    UpdLayer& o = U.layer[l - 1];
+    o.H = D.H; o.W = D.W; o.sel = D.sel; o.group_of = D.group_of;
+    weights += (int64_t)D.Kin * D.Kout;
+    o.aprev = l == 1 ? nullptr : P.layer[l - 2].A;
+    o.Kin = D.Kin; o.Kout = D.Kout; o.gamma = D.gamma; o.ldh = D.ldh; o.nw_in = D.nw_in;
+    upd_cta = update_rows_layout(o, upd_cta);
+  }
+  U.P = h->dP; U.ctrl = h->dCtrl; U.rt = h->dRT;
+  U.L = L; U.bs = bs; U.nw0 = P.nw0; U.h_max = h_max; U.key0 = P.key0; U.key1 = P.key1;
+  h->updCtas = (unsigned)upd_cta;
+  h->evCtas = (unsigned)ev_cta;
+  h->updRing = weights > kRowsWeights;
+  if (h->updRing) {
+    const cudaError_t ea = prepare_update_ws();
+    if (ea != cudaSuccess) return bail(cuda_fail(h, ea, "update kernel shared memory attribute"));
+  }
   if (injected_alloc_failure())
     return bail(fail(h, BMLP_ENOMEM, "cudaMallocHost failed (injected)"));
   if (cudaMallocHost(&h->hostPinned, 4 * sizeof(unsigned long long)) != cudaSuccess) {
@@ -1100,10 +1110,13 @@ int bmlp_debug_last_step(const bmlp_t* hc, int32_t layer, int16_t* Z, uint64_t* 
   if (mark) CK(h, cudaMemcpy(mark, D.mark, (size_t)h->bs, cudaMemcpyDeviceToHost));
   if (sel) {
     // device layout [G][bs] -> the documented [bs][G]
-    std::vector<int16_t> t((size_t)h->bs * D.G);
-    CK(h, cudaMemcpy(t.data(), D.sel, sizeof(int16_t) * t.size(), cudaMemcpyDeviceToHost));
+    std::vector<uint16_t> t((size_t)h->bs * D.G);
+    CK(h, cudaMemcpy(t.data(), D.sel, sizeof(uint16_t) * t.size(), cudaMemcpyDeviceToHost));
     for (int g = 0; g < D.G; ++g)
-      for (int m = 0; m < h->bs; ++m) sel[(size_t)m * D.G + g] = t[(size_t)g * h->bs + m];
+      for (int m = 0; m < h->bs; ++m) {
+        const uint16_t v = t[(size_t)g * h->bs + m];
+        sel[(size_t)m * D.G + g] = v == kNoSel ? (int16_t)-1 : (int16_t)(v & 0x7FFF);
+      }
   }
   return BMLP_OK;
 }
@@ -1134,13 +1147,19 @@ int bmlp_update_stats(bmlp_t* h, int64_t* rows_out, int64_t* streamed_out, int64
                       int32_t reset) {
   if (!h) return BMLP_EINVAL;
   h->err.clear();
-  unsigned long long v[3];
+  UpdStat slots[kStatSlots];
+  unsigned long long v[3] = {0, 0, 0};
   CK(h, cudaDeviceSynchronize());
-  CK(h, cudaMemcpy(v, &h->dCtrl->upd_rows, sizeof(v), cudaMemcpyDeviceToHost));
+  CK(h, cudaMemcpy(slots, h->dCtrl->stat, sizeof(slots), cudaMemcpyDeviceToHost));
+  for (const UpdStat& s : slots) {
+    v[0] += s.rows;
+    v[1] += s.streamed;
+    v[2] += s.bytes;
+  }
   if (rows_out) *rows_out = (int64_t)v[0];
   if (streamed_out) *streamed_out = (int64_t)v[1];
   if (bytes_out) *bytes_out = (int64_t)v[2];
-  if (reset) CK(h, cudaMemset(&h->dCtrl->upd_rows, 0, sizeof(v)));
+  if (reset) CK(h, cudaMemset(h->dCtrl->stat, 0, sizeof(slots)));
   return BMLP_OK;
 }
 

@@ -42,39 +42,55 @@ struct DevLayer {
   int16_t* Z;
   uint64_t* A;
   uint8_t* mark;
-  int16_t* sel;       // [G][bs] selected neuron per group and pattern, or -1 (group-major)
+  uint16_t* sel;      // [G][bs] selected neuron per group and pattern (group-major), bit 15
+                      // set where its rho_{k,y} is -1; kNoSel: none
   int16_t* member;    // [K_out] group order (neuron at position j), or null: contiguous groups
   int16_t* group_of;  // [K_out] group of neuron k (with member)
   int32_t Kin, Kout, nw_in, nw_out, ldh, gamma, G;
   int32_t ngrp;          // groups of 32 inputs per neuron row (ceil(K_in / 32))
   int32_t ev_cta_base;   // first CTA of this layer in the event-draw grid
-  int32_t row_base;      // first row of this layer in the update's row numbering
+  int32_t row_base;      // first row of this layer in the numbering of the large models' update
   int32_t nblk;          // blocks of 64 inputs per neuron row (ceil(K_in / 64))
-  uint64_t* EV;          // [K_out][ev_stride] reinforcement events of the current step,
-                         // bit i % 64 of word i / 64 = input i reinforced
+  uint64_t* EV;          // [K_out][ev_stride] reinforcement events of the current step (large
+                         // models), bit i % 64 of word i / 64 = input i reinforced
   int32_t ev_stride;     // words per EV row: nblk rounded up to even (16-byte rows)
 };
 
-// Device-resident step control.  The update kernel's last CTA advances t and s
-// and clears the per-step flags, so that one captured graph replays step after
-// step without host involvement.
+// Statistics of the update kernel, accumulated until read with reset: neuron
+// rows visited (layers with M_l non-empty), rows streamed (at least one CP
+// tuple) and algorithmic bytes (H read + write and W write of the streamed rows,
+// the planes of a group read + written per group with an event of a row without
+// tuple).  Spread over slots, so that CTAs do not queue for one address.
+struct UpdStat {
+  unsigned long long rows, streamed, bytes;
+};
+constexpr int kStatSlots = 64;
+
+// Device-resident step control, so that one captured graph replays step after
+// step without host involvement.  The first layer's forward pass copies s and t
+// to s_cur and t_cur and clears the marks; the update kernel, which reads only
+// the copies, advances s and t when it ends.
 struct Ctrl {
   unsigned long long t;         // global mini-batch counter since creation
   unsigned long long err;       // last-layer 01-loss count since the last epoch end
   unsigned long long bad_labels;// labels outside 0..c-1 seen by the kernels
   uint32_t s;                   // mini-batch index within the current train call
-  uint32_t done;                // CTAs of the update kernel finished this step
+  uint32_t s_cur;               // the mini-batch in progress
+  unsigned long long t_cur;
   uint32_t timeouts;            // bounded device waits that expired (BMLP_ETIMEOUT)
-  uint32_t upd_next;            // next row for the update kernel's warps this step
+  uint32_t upd_next;            // next row for the warps of the large models' update
   uint32_t any_mark[BMLP_MAX_LAYERS];
-  // update-kernel statistics, accumulated until read with reset
-  unsigned long long upd_rows;       // neuron rows visited (layers with M_l non-empty)
-  unsigned long long upd_streamed;   // rows streamed (at least one CP tuple)
-  unsigned long long upd_bytes;      // algorithmic bytes: H read + write and W write of the
-                                     // streamed rows, the planes of a group read + written
-                                     // per group with an event of a row without tuple
+  UpdStat stat[kStatSlots];
   unsigned long long layer_err[BMLP_MAX_LAYERS];  // local 01-loss count of each layer
 };
+
+// One thread of the first layer's forward pass, after its wait.
+__device__ __forceinline__ void begin_step(Ctrl* c, int L) {
+  c->s_cur = c->s;
+  c->t_cur = c->t;
+  c->upd_next = 0u;
+  for (int i = 0; i < L; ++i) c->any_mark[i] = 0u;
+}
 
 // Thresholds of the reinforcement sampler of one layer (Alg. 3 l.5-12): the
 // events of a neuron row are drawn per block of 64 inputs (the last block
@@ -98,12 +114,14 @@ struct StepParams {
   const RTables* rt;            // [L] reinforcement sampler thresholds
   int32_t nblk_max;             // max over layers of ceil(K_in / 64)
   Ctrl* ctrl;
-  int32_t L, c, bs, h_max, r_num, r_den, nw0, upd_ctas_total, ev_ctas_total;
-  int32_t rows_total;           // sum of K_l over the layers (update rows)
+  int32_t L, c, bs, h_max, r_num, r_den, nw0;
+  int32_t rows_total;           // sum of K_l over the layers
   int32_t nbits, nplanes;       // bit-planes of H used / stored per group (see H above)
   uint32_t key0, key1;          // Philox key = (seed mod 2^32, seed div 2^32)
 };
 
+
+constexpr uint16_t kNoSel = 0xFFFFu;   // K_l <= 32767, so no neuron has index 0x7FFF
 
 constexpr int kClsThreads = 512;
 
@@ -175,10 +193,9 @@ __global__ void k_cls_select(const StepParams* P);
 cudaError_t prepare_group_order(int max_K);  // shared-memory attribute, once
 cudaError_t launch_group_order(int L, int max_K, bool redraw, cudaStream_t st, const StepParams* P);
 // Reinforcement events of every neuron row of every layer for the current
-// step into DevLayer::EV (Alg. 3 l.5-12); grid = P->ev_ctas_total CTAs.
-void launch_r_events(unsigned grid, cudaStream_t st, const StepParams* P, uint32_t key0,
-                     uint32_t key1);
-constexpr int kEvRowsPerCta = 4;   // one warp per row
+// step into DevLayer::EV (Alg. 3 l.5-12).
+void launch_r_events(unsigned grid, cudaStream_t st, const StepParams* P, uint32_t key0, uint32_t key1);
+constexpr int kEvRowsPerCta = 8;   // one warp per row
 constexpr int kEvThreads = 32 * kEvRowsPerCta;
 // Generic forward for evaluation: A (M x nw_in) against W -> Aout (M x nw_out).
 __global__ void k_forward_eval(const uint64_t* __restrict__ A, int64_t M, int nw_in,
@@ -241,13 +258,36 @@ void launch_forward_eval_tc(const uint64_t* A, int64_t M, int nw_in, const uint6
 // = packed sign(A W^T), sign(0) = +1, pad bits 0.
 cudaError_t launch_forward_b1(const uint64_t* A, int64_t M, int nw_in, const uint64_t* W, int N,
                               int Kin, uint64_t* Aout, int nw_out, cudaStream_t st);
-// CP + R + repack of every layer with a non-empty M_l, then advance the step
-// (kern_update_ws.cu): bulk copies into a ring of shared-memory slots, the
-// bit-sliced steps by consumer warps; one CTA per SM (grid = the SM count).
+// CP + R + repack of every layer with a non-empty M_l, its reinforcement events
+// drawn by the kernel, then advance the step (kern_update_rows.cu).  UpdArgs: what the kernel needs of the model, passed by
+// value.
+struct UpdLayer {
+  uint32_t* H;
+  uint64_t* W;
+  const uint16_t* sel;
+  const int16_t* group_of;
+  const uint64_t* aprev;   // the layer's input activations of this mini-batch (null: layer 1)
+  int32_t Kin, Kout, gamma, ldh, nw_in;
+  int32_t lanes;           // lanes of a warp per row
+  int32_t upr;             // warps per row
+  int32_t cta_base;        // first CTA of the layer
+};
+struct UpdArgs {
+  UpdLayer layer[BMLP_MAX_LAYERS];
+  const StepParams* P;
+  Ctrl* ctrl;
+  const RTables* rt;
+  int32_t L, bs, nw0, h_max;
+  uint32_t key0, key1;
+};
+// Sets lanes, upr and cta_base of a layer (Kin and Kout given); returns the first
+// CTA of the next one.
+int update_rows_layout(UpdLayer& Ly, int cta_base);
 // pdl: launched with the programmatic-stream-serialization attribute.
-// nplanes: DevLayer's planes per group (StepParams::nplanes); bs: the
-// mini-batch size (the tuple lists of the slot ring).
-size_t update_ws_smem(int nplanes, int bs);
+cudaError_t launch_update_rows(int nplanes, unsigned grid, cudaStream_t st, bool pdl, const UpdArgs& U);
+// The same for large models (kern_update_ws.cu): bulk copies into a ring of
+// shared-memory slots, one CTA per SM (grid = the SM count); reads the events
+// from DevLayer::EV.
 cudaError_t prepare_update_ws();
 cudaError_t launch_update_ws(int nplanes, int h_max, int bs, unsigned grid, cudaStream_t st, bool pdl,
                              const StepParams* P);

@@ -462,7 +462,10 @@ __global__ void __launch_bounds__(THREADS, 2) k_train_forward_tc(const StepParam
     pdl_trigger();
     const int64_t start = (int64_t)P->ctrl->s * bs;
     M = min((int64_t)bs, ncall - start);
-    if (l == 1) A = x + start * T.nw;
+    if (l == 1) {
+      A = x + start * T.nw;
+      if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) begin_step(P->ctrl, P->L);
+    }
   };
   if (row_align(T.A, T.nw) == 16 && row_align(T.W, T.nw) == 16)
     run_tile<16>(T, place(smem_raw), pat, l > 1, ready, &P->ctrl->timeouts);

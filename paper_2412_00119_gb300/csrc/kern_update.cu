@@ -40,16 +40,26 @@ __device__ __forceinline__ int64_t batch_size(const StepParams* P, int64_t start
 // Every CTA waits before it lets the next kernel start, so a kernel two
 // launches back has always completed.
 // ---------------------------------------------------------------------------
+// A candidate's sort key (neuron, then the sign of its rho: delta = z rho < 0,
+// so rho is -1 exactly where z > 0) and the selection it becomes.
+__device__ __forceinline__ int sel_key(int k, int z) { return 2 * k + (z > 0 ? 1 : 0); }
+__device__ __forceinline__ uint16_t sel_of(int key) { return (uint16_t)((key >> 1) | ((key & 1) << 15)); }
+
 __device__ __forceinline__ void cls_select_body(const StepParams* __restrict__ P, int li, int mu);
 
 __global__ void __launch_bounds__(kClsThreads) k_cls_select(const StepParams* __restrict__ P) {
   const int li = blockIdx.y;
   const int mu = blockIdx.x;
   const bool early = li < P->L - 1;
-  if (!early) pdl_wait();
+  if (!early) {
+    pdl_wait();
+    pdl_trigger();
+  }
   cls_select_body(P, li, mu);
-  if (early) pdl_wait();
-  pdl_trigger();
+  if (early) {
+    pdl_wait();
+    pdl_trigger();
+  }
 }
 
 __device__ __forceinline__ void cls_select_body(const StepParams* __restrict__ P, int li, int mu) {
@@ -111,10 +121,10 @@ __device__ __forceinline__ void cls_select_body(const StepParams* __restrict__ P
 
   // selections are stored group-major (sel[g][mu]): the update kernel reads a
   // group's bs selections as one contiguous run
-  int16_t* sel = Ly.sel + mu;
+  uint16_t* sel = Ly.sel + mu;
   const int64_t sstride = P->bs;
   if (!s_mark) {
-    for (int g = threadIdx.x; g < Ly.G; g += blockDim.x) sel[g * sstride] = -1;
+    for (int g = threadIdx.x; g < Ly.G; g += blockDim.x) sel[g * sstride] = kNoSel;
     return;
   }
   const int y = s_y;
@@ -141,7 +151,7 @@ __device__ __forceinline__ void cls_select_body(const StepParams* __restrict__ P
           const int d = zj * rj;
           if (d < 0 && d > bestd) {  // ascending k: strict '>' keeps the lowest
             bestd = d;
-            bestk = 8 * ci + j;
+            bestk = sel_key(8 * ci + j, zj);
           }
         }
       }
@@ -154,7 +164,7 @@ __device__ __forceinline__ void cls_select_body(const StepParams* __restrict__ P
         }
       }
       if (ci < nchunk && (ci & (per - 1)) == 0)
-        sel[(ci / per) * sstride] = (bestd == INT_MIN) ? (int16_t)-1 : (int16_t)bestk;
+        sel[(ci / per) * sstride] = bestd == INT_MIN ? kNoSel : sel_of(bestk);
     }
     return;
   }
@@ -166,9 +176,9 @@ __device__ __forceinline__ void cls_select_body(const StepParams* __restrict__ P
     for (int kk = lane; kk < gamma; kk += 32) {
       const int k = member ? (int)member[g * gamma + kk] : g * gamma + kk;
       const int d = (int)z[k] * (int)Ly.rho[(int64_t)k * c + y];
-      if (d < 0 && (d > bestd || (d == bestd && k < bestk))) {
+      if (d < 0 && (d > bestd || (d == bestd && sel_key(k, z[k]) < bestk))) {
         bestd = d;
-        bestk = k;
+        bestk = sel_key(k, z[k]);
       }
     }
 #pragma unroll
@@ -180,53 +190,13 @@ __device__ __forceinline__ void cls_select_body(const StepParams* __restrict__ P
         bestk = ok;
       }
     }
-    if (lane == 0) sel[g * sstride] = (bestd == INT_MIN) ? (int16_t)-1 : (int16_t)bestk;
+    if (lane == 0) sel[g * sstride] = bestd == INT_MIN ? kNoSel : sel_of(bestk);
   }
 }
 
 namespace {
 
 using namespace upd;
-
-// Least j in [0, hi] with V < tab[j], or hi when there is none (tab
-// nondecreasing).
-__device__ __forceinline__ int least_below(uint32_t V, const unsigned long long* tab, int hi) {
-  int lo = 0;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if ((unsigned long long)V < tab[mid]) hi = mid;
-    else lo = mid + 1;
-  }
-  return lo;
-}
-
-// The events of block b (n inputs, tables index x) of neuron k at step t,
-// given that the block holds at least one: the first from the first-event
-// table, the next ones by geometric gaps cut at the block's end; the draws
-// are the words of Philox((b, k, (4 + r) 2^16 + l, t)), r = 0, 1, ... in order.
-__device__ __forceinline__ uint64_t block_events(const RTables& R, int x, int n, uint32_t b,
-                                                 uint32_t k, uint32_t l, uint32_t t, uint32_t key0,
-                                                 uint32_t key1) {
-  uint32_t r = 0;
-  uint4 v = philox4x32_10(make_uint4(b, k, (4u << 16) + l, t), key0, key1);
-  int used = 1;
-  int p = least_below(v.x, R.first[x], n - 1);
-  uint64_t mask = 1ull << p;
-#pragma unroll 1
-  while (p < n - 1) {
-    if (used == 4) {
-      ++r;
-      v = philox4x32_10(make_uint4(b, k, ((4u + r) << 16) + l, t), key0, key1);
-      used = 0;
-    }
-    const uint32_t V = word_of(v, used++);
-    const int gmax = n - 2 - p;
-    if (!((unsigned long long)V < R.gap[gmax])) break;  // no further event in the block
-    p += 1 + least_below(V, R.gap, gmax);
-    mask |= 1ull << p;
-  }
-  return mask;
-}
 
 }  // namespace
 
@@ -239,23 +209,19 @@ __device__ __forceinline__ uint64_t block_events(const RTables& R, int x, int n,
 // runs beside the forward passes.
 __global__ void __launch_bounds__(kEvThreads) k_r_events(const StepParams* __restrict__ P,
                                                          uint32_t key0, uint32_t key1) {
-  __shared__ RTables s_rt;
+  __shared__ Tables s_rt;
   __shared__ uint16_t s_cand[kEvRowsPerCta][128];  // blocks with an event, per warp
   const int bid = blockIdx.x;
   int li = 0;
   while (li + 1 < P->L && bid >= P->layer[li + 1].ev_cta_base) ++li;
   const DevLayer& Ly = P->layer[li];
-  {
-    const unsigned long long* src = reinterpret_cast<const unsigned long long*>(P->rt + li);
-    unsigned long long* dst = reinterpret_cast<unsigned long long*>(&s_rt);
-    for (int i = threadIdx.x; i < (int)(sizeof(RTables) / 8); i += blockDim.x) dst[i] = src[i];
-  }
+  load_tables(s_rt, P->rt[li]);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int k = (bid - Ly.ev_cta_base) * kEvRowsPerCta + warp;
   if (k >= Ly.Kout) return;
   const uint32_t l = (uint32_t)li + 1u;
-  const uint32_t tt = (uint32_t)P->ctrl->t;
+  const uint32_t tt = (uint32_t)P->ctrl->t_cur;
   const int Kin = Ly.Kin, nblk = Ly.nblk;
   uint64_t* ev = Ly.EV + (int64_t)k * Ly.ev_stride;
   uint16_t* cand = s_cand[warp];
@@ -371,8 +337,7 @@ cudaError_t launch_group_order(int L, int max_K, bool redraw, cudaStream_t st, c
   return cudaGetLastError();
 }
 
-void launch_r_events(unsigned grid, cudaStream_t st, const StepParams* P, uint32_t key0,
-                     uint32_t key1) {
+void launch_r_events(unsigned grid, cudaStream_t st, const StepParams* P, uint32_t key0, uint32_t key1) {
   k_r_events<<<grid, kEvThreads, 0, st>>>(P, key0, key1);
 }
 

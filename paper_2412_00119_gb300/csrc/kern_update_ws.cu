@@ -1,6 +1,7 @@
 // kern_update_ws.cu -- the hidden-weight update of one training step (Alg. 3:
 // clipped perceptron, then reinforcement; Sec. 3.1: W = sign(H) re-packed in
-// the same pass), with its memory traffic driven by bulk copies.
+// the same pass) for large models, with its memory traffic driven by bulk
+// copies.
 //
 // The hidden weights are bit-sliced (DevLayer::H, update_common.cuh): a group
 // of 32 inputs of a neuron row is kP words, word p holding bit p of the
@@ -16,8 +17,8 @@
 // The update streams every hidden weight of every neuron row that received a
 // CP tuple: read, the steps, write.
 //   - kSched scheduler warps take rows from the step's row counter, find the
-//     row's CP tuples (Alg. 2's selections of the neuron's group; labels in
-//     shared memory), and fill one slot of a shared-memory ring per segment
+//     row's CP tuples (Alg. 2's selections of the neuron's group, with the sign
+//     of their rho), and fill one slot of a shared-memory ring per segment
 //     of the row: bulk copies (cp.async.bulk, completing on the slot's "full"
 //     mbarrier) of the segment's planes, of its part of the reinforcement-
 //     event bitmap and of the first tuples' activation words, plus the tuple
@@ -32,8 +33,7 @@
 // with an event are stepped in place in global memory, and its W is
 // unchanged.  Layers with an empty M_l are skipped (no CP, no R).  Every
 // mbarrier wait is bounded; an expiry stops the CTA's loops, waits (bounded)
-// for the copies it issued, and is counted in the control block.  The last
-// CTA to finish advances the step counters.
+// for the copies it issued, and is counted in the control block.
 #include "tc_common.cuh"
 #include "update_common.cuh"
 
@@ -88,8 +88,7 @@ struct LayerSh {
   uint32_t* H;
   uint64_t* W;
   const uint64_t* EV;
-  const int16_t* sel;
-  const int8_t* rho;
+  const uint16_t* sel;
   const int16_t* group_of;
   const uint32_t* aprev;   // the layer's input activations of this mini-batch, row 0
   int row_base, gamma, ngrp, ldh, nw_in, ev_stride, Kin, pad;
@@ -99,7 +98,6 @@ struct __align__(16) WsShared {
   LayerSh lay[BMLP_MAX_LAYERS];
   unsigned long long full[kMaxSlots];
   unsigned long long empty[kMaxSlots];
-  int16_t y[kMaxT];                   // labels of the mini-batch (bad ones as 0)
   unsigned long long stats[3];        // rows visited, rows streamed, algorithmic bytes
   int issued[kMaxSlots];              // last use of each slot with copies issued (-1: none)
   int failed;
@@ -144,7 +142,6 @@ struct RowFetch {
   int gr;          // global row number (>= rows_total: none)
   int li, k;       // layer index, neuron
   int sv[4];       // this lane's selections of patterns 32 q + lane (the first 128)
-  int rho_lane;    // rho_{k, lane} for c <= 32
   bool skip;       // M_l empty, or the step's forward pass failed: no CP, no R
 };
 
@@ -156,7 +153,6 @@ __device__ __forceinline__ void ws_scheduler(const StepParams* __restrict__ P, W
   const uint32_t nslots = (uint32_t)R.nslots;
   Ctrl* ctrl = P->ctrl;
   volatile int* failed = &sh->failed;
-  const int c = P->c;
   const int L = P->L;
   const int bs = P->bs;
   const int rows_total = P->rows_total;
@@ -179,39 +175,29 @@ __device__ __forceinline__ void ws_scheduler(const StepParams* __restrict__ P, W
     f.li = __popc(__ballot_sync(kFull, lane >= 1 && lane < L && gr >= rb_lane));
     f.skip = gr >= rows_total || step_failed || __shfl_sync(kFull, am_lane, f.li) == 0u;
     f.k = 0;
-    f.rho_lane = 0;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) f.sv[q] = -1;
+    for (int q = 0; q < 4; ++q) f.sv[q] = kNoSel;
     if (!f.skip) {
       const LayerSh& Ly = sh->lay[f.li];
       f.k = gr - Ly.row_base;
       const int g = Ly.group_of ? (int)Ly.group_of[f.k] : f.k / Ly.gamma;
-      const int16_t* selg = Ly.sel + (int64_t)g * bs;
+      const uint16_t* selg = Ly.sel + (int64_t)g * bs;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int m = 32 * q + lane;
         if (m < bsz) f.sv[q] = (int)selg[m];
       }
-      if (c <= 32 && lane < c) f.rho_lane = (int)Ly.rho[(int64_t)f.k * c + lane];
     }
     return f;
   };
   // tuples from selections sv of patterns m0 + 32 q + lane, appended to list
   auto scan4 = [&](const RowFetch& f, const int (&sv)[4], int m0, int n_t) -> int {
-    const LayerSh& Ly = sh->lay[f.li];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int m = m0 + 32 * q + lane;
-      const bool hit = sv[q] == f.k;
+      const bool hit = (sv[q] & 0x7FFF) == f.k;
       const unsigned bal = __ballot_sync(kFull, hit);
-      if (bal != 0u) {
-        const int yv = hit ? (int)sh->y[m] : 0;
-        const int rs = __shfl_sync(kFull, f.rho_lane, yv & 31);
-        if (hit) {
-          const int rho = (c <= 32) ? rs : (int)Ly.rho[(int64_t)f.k * c + yv];
-          list[n_t + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(m | ((rho > 0) ? 0 : 0x8000));
-        }
-      }
+      if (hit) list[n_t + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(m | (sv[q] & 0x8000));
       n_t += __popc(bal);
     }
     return n_t;
@@ -235,14 +221,14 @@ __device__ __forceinline__ void ws_scheduler(const StepParams* __restrict__ P, W
     int n_t = scan4(cur, cur.sv, 0, 0);
     if (bsz > 128) {
       const int g = Ly.group_of ? (int)Ly.group_of[k] : k / Ly.gamma;
-      const int16_t* selg = Ly.sel + (int64_t)g * bs;
+      const uint16_t* selg = Ly.sel + (int64_t)g * bs;
 #pragma unroll 1
       for (int m0 = 128; m0 < bsz; m0 += 128) {
         int sv[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int m = m0 + 32 * q + lane;
-          sv[q] = (m < bsz) ? (int)selg[m] : -1;
+          sv[q] = (m < bsz) ? (int)selg[m] : (int)kNoSel;
         }
         n_t = scan4(cur, sv, m0, n_t);
       }
@@ -452,8 +438,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_ws(const StepParams* __r
   }
   pdl_wait();
   pdl_trigger();
-  const unsigned long long t = ctrl->t;
-  const uint32_t sidx = ctrl->s;
+  const uint32_t sidx = ctrl->s_cur;
   const int64_t start = (int64_t)sidx * P->bs;
   const int64_t rem = P->n - start;
   const int bsz = (int)(rem < P->bs ? rem : P->bs);
@@ -464,15 +449,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_ws(const StepParams* __r
     const int li = threadIdx.x;
     const DevLayer& D = P->layer[li];
     LayerSh& o = sh->lay[li];
-    o.H = D.H; o.W = D.W; o.EV = D.EV; o.sel = D.sel; o.rho = D.rho; o.group_of = D.group_of;
+    o.H = D.H; o.W = D.W; o.EV = D.EV; o.sel = D.sel; o.group_of = D.group_of;
     o.aprev = li == 0 ? reinterpret_cast<const uint32_t*>(P->x + start * P->nw0)
                       : reinterpret_cast<const uint32_t*>(P->layer[li - 1].A);
     o.row_base = D.row_base; o.gamma = D.gamma; o.ngrp = D.ngrp; o.ldh = D.ldh; o.nw_in = D.nw_in;
     o.ev_stride = D.ev_stride; o.Kin = D.Kin; o.pad = 0;
-  }
-  for (int i = threadIdx.x; i < bsz; i += kThreads) {
-    const int yv = P->y[start + i];
-    sh->y[i] = (int16_t)((yv < 0 || yv >= P->c) ? 0 : yv);   // memory-safe stand-in; the host reports bad labels
   }
   __syncthreads();
   if (warp < kSched)
@@ -488,20 +469,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_ws(const StepParams* __r
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    atomicAdd(&ctrl->upd_rows, sh->stats[0]);
-    atomicAdd(&ctrl->upd_streamed, sh->stats[1]);
-    atomicAdd(&ctrl->upd_bytes, sh->stats[2]);
+    UpdStat& o = ctrl->stat[blockIdx.x % kStatSlots];
+    atomicAdd(&o.rows, sh->stats[0]);
+    atomicAdd(&o.streamed, sh->stats[1]);
+    atomicAdd(&o.bytes, sh->stats[2]);
     if (sh->failed) atomicAdd(&ctrl->timeouts, 1u);
-    // step completion: the last CTA to finish advances the counters
-    __threadfence();
-    const unsigned prev = atomicAdd(&ctrl->done, 1u);
-    if (prev == gridDim.x - 1) {
-      ctrl->t = t + 1;
+    if (blockIdx.x == 0) {
+      // the next step's counters (this kernel reads only the copies)
       ctrl->s = sidx + 1;
-      for (int i = 0; i < P->L; ++i) ctrl->any_mark[i] = 0u;
-      ctrl->upd_next = 0u;
-      ctrl->done = 0u;
-      __threadfence();
+      ctrl->t = ctrl->t_cur + 1;
     }
   }
 }
@@ -537,10 +513,6 @@ cudaError_t prepare_update_ws() {
       (e = set_smem<16, false>()) != cudaSuccess)
     return e;
   return cudaSuccess;
-}
-
-cudaError_t update_kernel_image(cudaFuncAttributes* fa) {
-  return cudaFuncGetAttributes(fa, k_update_ws<8, true>);
 }
 
 cudaError_t launch_update_ws(int nplanes, int h_max, int bs, unsigned grid, cudaStream_t st, bool pdl,

@@ -126,6 +126,66 @@ __device__ __forceinline__ uint32_t word_of(const uint4& v, int i) {
   return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w));
 }
 
+// The sampler tables of one layer as inclusive 32-bit thresholds (V < T <=> V <=
+// T - 1 for T in 1 .. 2^32; a T of 0 occurs only where no block has an event).
+struct Tables {
+  unsigned long long any[2];
+  uint32_t first[2][64], gap[64];
+  float scale[2];   // any / 2^32: the probability that a block has an event
+  float inv;        // 1 / log2(1 - q)
+};
+
+// All threads of a CTA of at least kTableThreads.
+constexpr int kTableThreads = 195;
+__device__ __forceinline__ void load_tables(Tables& tab, const RTables& R) {
+  const int i = threadIdx.x;
+  if (i < 128) tab.first[i >> 6][i & 63] = (uint32_t)(R.first[i >> 6][i & 63] - 1ull);
+  else if (i < 192) tab.gap[i - 128] = (uint32_t)(R.gap[i - 128] - 1ull);
+  else if (i < 194) {
+    tab.any[i - 192] = R.any[i - 192];
+    tab.scale[i - 192] = (float)R.any[i - 192] * 2.3283064365386963e-10f;
+  } else if (i == 194) {
+    tab.inv = 1.0f / __log2f(1.0f - (float)R.gap[0] * 2.3283064365386963e-10f);
+  }
+}
+
+// Least j in [0, hi] with V <= tab[j], or hi when there is none (tab
+// nondecreasing).  Where the thresholds are those of a geometric law the
+// logarithm gives j to within rounding; the table decides.
+__device__ __forceinline__ int least_at(uint32_t V, const uint32_t* tab, int hi, float scale, float inv) {
+  const float u = (float)V * 2.3283064365386963e-10f * scale;   // V / 2^32
+  int j = __float2int_rd(__log2f(1.0f - u) * inv);
+  j = max(0, min(j, hi));
+  while (j > 0 && V <= tab[j - 1]) --j;
+  while (j < hi && V > tab[j]) ++j;
+  return j;
+}
+
+// The events of block b (n inputs, tables index x) of neuron k at step t, given
+// that the block holds at least one (draws as bmlp.h documents them).
+__device__ __forceinline__ uint64_t block_events(const Tables& R, int x, int n, uint32_t b, uint32_t k,
+                                                 uint32_t l, uint32_t t, uint32_t key0, uint32_t key1) {
+  uint32_t r = 0;
+  uint4 v = philox4x32_10(make_uint4(b, k, (4u << 16) + l, t), key0, key1);
+  int used = 1;
+  int p = least_at(v.x, R.first[x], n - 1, R.scale[x], R.inv);
+  uint64_t mask = 1ull << p;
+#pragma unroll 1
+  while (p < n - 1) {
+    if (used == 4) {
+      ++r;
+      v = philox4x32_10(make_uint4(b, k, ((4u + r) << 16) + l, t), key0, key1);
+      used = 0;
+    }
+    const uint32_t V = word_of(v, used++);
+    const int gmax = n - 2 - p;
+    if (V > R.gap[gmax]) break;  // no further event in the block
+    p += 1 + least_at(V, R.gap, gmax, 1.0f, R.inv);
+    mask |= 1ull << p;
+  }
+  return mask;
+}
+
 // Valid-input mask of group g of a row of Kin inputs.
 __host__ __device__ __forceinline__ uint32_t group_mask(int g, int Kin) {
   const int n = Kin - 32 * g;

@@ -1,0 +1,63 @@
+"""The two update kernels at the edges of their layouts, bit for bit against the
+oracle: rows of fewer blocks than a warp has lanes, several warps per row, short
+last blocks, every plane count, and the ring kernel of large models (more than
+20 M hidden weights)."""
+import os
+
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+import workloads as W
+from paper_2412_00119_gb300 import bmlp as B
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _setup():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    torch.cuda.set_device(DEV)
+    O.set_threads(os.cpu_count() or 1)
+    B.lib()
+
+
+def check(widths, h_max, n, bs, p_r0=0.5, gamma=None, group_mode=0):
+    gpu = B.BMLP(widths, 7, h_max=h_max, seed=n, bs=bs, p_r0=p_r0, gamma=gamma, group_mode=group_mode)
+    ref = O.OracleModel(list(widths), 7, h_max=h_max, seed=n, bs=bs, p_r0=p_r0, gamma=gamma)
+    ref.set_group_mode(group_mode)
+    xp = W.random_packed(n + 1, n, widths[0])
+    y = np.random.default_rng(n).integers(0, 7, n).astype(np.int32)
+    x = torch.from_numpy(xp.view(np.int64)).to(DEV)
+    e = gpu.train(x, torch.from_numpy(y).to(DEV), count_errors=True)
+    assert e == ref.train(W.unpack(xp, widths[0]), y)
+    for l in range(1, len(widths)):
+        H, Wb, _, p_r, step = gpu.state(l)
+        assert np.array_equal(H.astype(np.int32), ref.H(l).T), (widths, l)
+        assert np.array_equal(Wb, W.pack(np.where(ref.H(l).T > 0, 1, -1))), (widths, l)
+        assert step == ref.step
+    gpu.close()
+
+
+# one block, 1 / 2 / 3 .. 31 / 32 / 33 blocks per row, groups across warps
+@pytest.mark.parametrize("h_max", [1, 3, 15, 13, 255, 127, 1001])
+@pytest.mark.parametrize("widths", [(1, 5, 40), (64, 37, 65), (130, 64, 33), (2047, 12, 96), (2049, 60, 31),
+                                    (4500, 18, 128)])
+def test_rows_kernel(widths, h_max):
+    check(widths, h_max, 210, 100)
+
+
+@pytest.mark.parametrize("bs", [1, 127, 129, 300])
+def test_rows_kernel_batches(bs):
+    check((300, 96, 200), 255, 2 * bs + 1, bs, p_r0=3.0, gamma=[96, 8], group_mode=2)
+
+
+# more than 20 M weights: the ring kernel, whole rows and ragged ones
+@pytest.mark.parametrize("h_max,widths", [(255, (5000, 4500)), (13, (5000, 4500)), (127, (6160, 3600)),
+                                          (1001, (2100, 10010))])
+def test_ring_kernel(h_max, widths):
+    check(widths, h_max, 60, 20)
