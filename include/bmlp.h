@@ -81,9 +81,10 @@ extern "C" {
 #define BMLP_EPOCH_END 1u  /* after these n patterns, close the epoch (Alg. 1 l.21) */
 
 /* forward-contraction engines (hparams.fwd_impl) */
-#define BMLP_FWD_AUTO 0     /* library's choice */
+#define BMLP_FWD_AUTO 0     /* library's choice: the tensor cores (bmlp_get_info reports
+                             * BMLP_FWD_TCGEN05 up to bs = 128 and BMLP_FWD_POPC above) */
 #define BMLP_FWD_POPC 1     /* CUDA-core XOR + popcount */
-#define BMLP_FWD_TCGEN05 2  /* 5th-gen tensor cores, +-1 as e4m3, fp32 accumulate (exact) */
+#define BMLP_FWD_TCGEN05 2  /* 5th-gen tensor cores, +-1 as e2m1, fp32 accumulate (exact) */
 /* Further contraction units, measured by bmlp_engine_peak (and, for B1MMA,
  * bmlp_layer_forward_engine) for the engine comparison; training uses POPC or
  * TCGEN05.  tcgen05.mma.kind::i8 does not exist on sm_103a, so +-1 as int8 on

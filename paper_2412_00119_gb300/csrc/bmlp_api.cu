@@ -60,6 +60,9 @@ enum ProfKind { kProfTrainFwd = 0, kProfCls = 1, kProfUpd = 2, kProfEvalFwd = 3,
 struct bmlp {
   int device = 0;
   int L = 0, c = 0, h_max = 0, bs = 0, r_num = 0, r_den = 1, fwd_impl = BMLP_FWD_POPC;
+  // the forward passes run on the tensor cores: fwd_impl, or the library's choice above 128 patterns,
+  // where bmlp_get_info reports BMLP_FWD_POPC for BMLP_FWD_AUTO
+  bool tc = false;
   int group_mode = BMLP_GROUPS_CONTIGUOUS, max_K = 0;  // group membership (Sec. 4.3), widest layer
   uint64_t seed = 0;
   std::vector<int> K, gamma;
@@ -259,7 +262,7 @@ int enqueue_step(bmlp_t* h, cudaStream_t st, bool fork, bool chained = false) {
       CK(h, cudaEventRecord(h->evJoin, h->sideStream));
     }
     prof_begin(h, kProfTrainFwd, st);
-    if (h->fwd_impl == BMLP_FWD_TCGEN05)
+    if (h->tc)
       CK(h, launch_train_forward_tc(h->bs, h->K[l], h->K[l - 1], st, fork && (l > 1 || chained), h->dP, l));
     else
       k_train_forward<<<train_forward_grid(h->bs, h->K[l]), train_forward_block(), 0, st>>>(h->dP, l);
@@ -274,7 +277,7 @@ int enqueue_step(bmlp_t* h, cudaStream_t st, bool fork, bool chained = false) {
   // programmatic dependent of the one before it (launch and prologue overlap
   // the previous kernel's tail); the event-draw branch joins with a full edge
   CK(h, launch_kernel(k_cls_select, dim3((unsigned)h->bs, (unsigned)h->L), dim3(kClsThreads), 0, st,
-                      fork && h->fwd_impl == BMLP_FWD_TCGEN05, h->dP));
+                      fork && h->tc, h->dP));
   prof_end(h, st);
   if (fork && h->updRing && h->L > 1) CK(h, cudaStreamWaitEvent(st, h->evJoin, 0));
   if (h->updRing && (!fork || h->L == 1)) {
@@ -365,7 +368,7 @@ int run_steps(bmlp_t* h, const uint64_t* xd, const int32_t* yd, int64_t n, cudaS
     s += multi ? kGraphSteps : 1;
   }
   h->profiling = h->profEvery > 0;
-  h->launches += steps * (h->L + 2 + (h->group_mode == BMLP_GROUPS_RESHUFFLED ? 1 : 0));
+  h->launches += steps * (h->L + 2 + (h->updRing ? 1 : 0) + (h->group_mode == BMLP_GROUPS_RESHUFFLED ? 1 : 0));
   h->t_host += steps;
   return BMLP_OK;
 }
@@ -504,6 +507,7 @@ int bmlp_create(const int32_t* widths, int32_t n_widths, int32_t classes, int16_
     return fail(nullptr, BMLP_ENODEV, "device has no sm_103a kernel image (needs a GB300)");
   }
   h->L = L; h->c = classes; h->h_max = h_max; h->bs = bs; h->r_num = r_num; h->r_den = r_den;
+  h->tc = fwd == BMLP_FWD_TCGEN05 || hp.fwd_impl == BMLP_FWD_AUTO;
   h->fwd_impl = fwd; h->seed = seed; h->p_r = p_r0;
   h->group_mode = group_mode; h->max_K = max_K;
   h->K.assign(widths, widths + n_widths);
@@ -600,7 +604,7 @@ int bmlp_create(const int32_t* widths, int32_t n_widths, int32_t classes, int16_
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return bail(cuda_fail(h, e, "init kernels"));
-  if (fwd == BMLP_FWD_TCGEN05 &&
+  if (h->tc &&
       ((e = prepare_train_forward_tc()) != cudaSuccess || (e = prepare_forward_eval_tc()) != cudaSuccess))
     return bail(cuda_fail(h, e, "tcgen05 forward smem attribute"));
   if ((e = cudaMemset(h->dCtrl, 0, sizeof(Ctrl))) != cudaSuccess) return bail(cuda_fail(h, e, "memset"));
@@ -740,7 +744,7 @@ int predict_impl(bmlp_t* h, const uint64_t* x, int64_t n, int32_t* out, void* cu
     for (int l = 1; l <= h->L; ++l) {
       const DevLayer& D = h->hp.layer[l - 1];
       prof_begin(h, kProfEvalFwd, st);
-      if (h->fwd_impl == BMLP_FWD_TCGEN05)
+      if (h->tc)
         CK(h, eval_layer_tc(h, D, in, m, h->evA[cur], st, l > 1 && !h->profiling));
       else
         k_forward_eval<<<eval_forward_grid(m, D.Kout), eval_forward_block(), 0, st>>>(
@@ -753,7 +757,7 @@ int predict_impl(bmlp_t* h, const uint64_t* x, int64_t n, int32_t* out, void* cu
       int32_t* dst = out + (every_layer ? (int64_t)(l - 1) * n : 0) + s0;
       int32_t* o = odev ? dst : h->stOut;
       prof_begin(h, kProfOut, st);
-      if (h->fwd_impl == BMLP_FWD_TCGEN05 && h->c <= kPredictTileClasses)
+      if (h->tc && h->c <= kPredictTileClasses)
         CK(h, launch_predict_tile(in, m, D.nw_out, D.PT, h->c, D.Kout, o, &h->dCtrl->timeouts, st,
                                   m <= kTileRows && !h->profiling));
       else
@@ -770,11 +774,11 @@ int predict_impl(bmlp_t* h, const uint64_t* x, int64_t n, int32_t* out, void* cu
     h->launches += h->L;
   }
   if (!odev) {
-    if (h->fwd_impl == BMLP_FWD_TCGEN05)
+    if (h->tc)
       CK(h, cudaMemcpyAsync(&h->hostPinned[3], &h->dCtrl->timeouts, sizeof(uint32_t),
                             cudaMemcpyDeviceToHost, st));
     CK(h, cudaStreamSynchronize(st));
-    if (h->fwd_impl == BMLP_FWD_TCGEN05 && (uint32_t)h->hostPinned[3] != 0) {
+    if (h->tc && (uint32_t)h->hostPinned[3] != 0) {
       CK(h, cudaMemsetAsync(&h->dCtrl->timeouts, 0, sizeof(uint32_t), st));
       h->hostPinned[3] = 0;
       return fail(h, BMLP_ETIMEOUT, "a bounded device-side wait expired");
@@ -967,7 +971,7 @@ int bmlp_layer_forward(bmlp_t* h, int32_t layer, const uint64_t* a_in, int64_t n
     const uint64_t* in = a_in + s0 * D.nw_in;
     uint64_t* out = a_out + s0 * D.nw_out;
     prof_begin(h, kProfEvalFwd, st);
-    if (h->fwd_impl == BMLP_FWD_TCGEN05)
+    if (h->tc)
       CK(h, eval_layer_tc(h, D, in, m, out, st, false));
     else
       k_forward_eval<<<eval_forward_grid(m, D.Kout), eval_forward_block(), 0, st>>>(
