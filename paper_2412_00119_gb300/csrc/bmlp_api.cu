@@ -270,7 +270,7 @@ int enqueue_step(bmlp_t* h, cudaStream_t st, bool fork, bool chained = false) {
   }
   if (h->group_mode == BMLP_GROUPS_RESHUFFLED) {
     // this step's partition (keyed by the step counter) before the selection
-    CK(h, launch_group_order(h->L, h->max_K, true, st, h->dP));
+    CK(h, launch_group_order(h->L, h->max_K, true, st, false, h->dP));
   }
   prof_begin(h, kProfCls, st);
   // inside the step graph each kernel after the first is launched as a
@@ -614,7 +614,7 @@ int bmlp_create(const int32_t* widths, int32_t n_widths, int32_t classes, int16_
   // the partition of step 0 (the fixed one, or the first redrawn one)
   if (group_mode != BMLP_GROUPS_CONTIGUOUS &&
       ((e = prepare_group_order(max_K)) != cudaSuccess ||
-       (e = launch_group_order(L, max_K, false, 0, h->dP)) != cudaSuccess))
+       (e = launch_group_order(L, max_K, false, 0, false, h->dP)) != cudaSuccess))
     return bail(cuda_fail(h, e, "group order"));
   if ((e = cudaDeviceSynchronize()) != cudaSuccess) return bail(cuda_fail(h, e, "init"));
   h->launches += 4 * L;

@@ -191,7 +191,7 @@ __global__ void k_cls_select(const StepParams* P);
 // Group order of every layer with a random partition (DevLayer::member /
 // group_of); redraw: keyed by the current step (else by step 0).
 cudaError_t prepare_group_order(int max_K);  // shared-memory attribute, once
-cudaError_t launch_group_order(int L, int max_K, bool redraw, cudaStream_t st, const StepParams* P);
+cudaError_t launch_group_order(int L, int max_K, bool redraw, cudaStream_t st, bool pdl, const StepParams* P);
 // Reinforcement events of every neuron row of every layer for the current
 // step into DevLayer::EV (Alg. 3 l.5-12).
 void launch_r_events(unsigned grid, cudaStream_t st, const StepParams* P, uint32_t key0, uint32_t key1);
