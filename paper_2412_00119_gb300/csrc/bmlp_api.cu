@@ -91,6 +91,7 @@ struct bmlp {
   cudaStream_t sideStream = nullptr;  // the event-draw branch of the step graph
   cudaEvent_t evFork = nullptr, evJoin = nullptr;
   UpdArgs upd{};
+  ClsArgs cls{};
   unsigned updCtas = 0, evCtas = 0;
   bool updRing = false;   // the update streams through a shared-memory ring (large models)
   // profiling
@@ -270,14 +271,13 @@ int enqueue_step(bmlp_t* h, cudaStream_t st, bool fork, bool chained = false) {
   }
   if (h->group_mode == BMLP_GROUPS_RESHUFFLED) {
     // this step's partition (keyed by the step counter) before the selection
-    CK(h, launch_group_order(h->L, h->max_K, true, st, false, h->dP));
+    CK(h, launch_group_order(h->L, h->max_K, true, st, fork && h->tc, h->dP));
   }
   prof_begin(h, kProfCls, st);
   // inside the step graph each kernel after the first is launched as a
   // programmatic dependent of the one before it (launch and prologue overlap
   // the previous kernel's tail); the event-draw branch joins with a full edge
-  CK(h, launch_kernel(k_cls_select, dim3((unsigned)h->bs, (unsigned)h->L), dim3(kClsThreads), 0, st,
-                      fork && h->tc, h->dP));
+  CK(h, launch_cls_select(h->cls, h->max_K, st, fork && h->tc));
   prof_end(h, st);
   if (fork && h->updRing && h->L > 1) CK(h, cudaStreamWaitEvent(st, h->evJoin, 0));
   if (h->updRing && (!fork || h->L == 1)) {
@@ -571,6 +571,13 @@ int bmlp_create(const int32_t* widths, int32_t n_widths, int32_t classes, int16_
     o.Kin = D.Kin; o.Kout = D.Kout; o.gamma = D.gamma; o.ldh = D.ldh; o.nw_in = D.nw_in;
     upd_cta = update_rows_layout(o, upd_cta);
   }
+  ClsArgs& C = h->cls;
+  for (int l = 1; l <= L; ++l) {
+    const DevLayer& D = P.layer[l - 1];
+    C.layer[l - 1] = ClsLayer{D.A, D.PT, D.Z, D.rhoT, D.sel, D.mark, D.member, D.Kout, D.nw_out, D.gamma, D.G};
+  }
+  C.P = h->dP; C.ctrl = h->dCtrl; C.L = L; C.c = classes; C.bs = bs; C.r_num = r_num; C.r_den = r_den;
+  C.early = group_mode != BMLP_GROUPS_RESHUFFLED;
   U.P = h->dP; U.ctrl = h->dCtrl; U.rt = h->dRT;
   U.L = L; U.bs = bs; U.nw0 = P.nw0; U.h_max = h_max; U.key0 = P.key0; U.key1 = P.key1;
   h->updCtas = (unsigned)upd_cta;

@@ -123,7 +123,6 @@ struct StepParams {
 
 constexpr uint16_t kNoSel = 0xFFFFu;   // K_l <= 32767, so no neuron has index 0x7FFF
 
-constexpr int kClsThreads = 512;
 
 // ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11), device version.
@@ -187,7 +186,25 @@ __device__ __forceinline__ int clip_h(int h, int h_max) {
 // Forward of layer l (1-based) for the current training mini-batch.
 __global__ void k_train_forward(const StepParams* P, int l);
 // Local classifier, 01-loss, margin, marks, and the group selection, all layers.
-__global__ void k_cls_select(const StepParams* P);
+// ClsArgs: what the kernel needs of the model, passed by value.
+struct ClsLayer {
+  const uint64_t* A;
+  const uint64_t* PT;
+  const int16_t* Z;
+  const int8_t* rhoT;
+  uint16_t* sel;
+  uint8_t* mark;
+  const int16_t* member;
+  int32_t Kout, nw_out, gamma, G;
+};
+struct ClsArgs {
+  ClsLayer layer[BMLP_MAX_LAYERS];
+  const StepParams* P;
+  Ctrl* ctrl;
+  int32_t L, c, bs, r_num, r_den;
+  int32_t early;   // the CTAs of the layers below the last work before they wait
+};
+cudaError_t launch_cls_select(const ClsArgs& C, int max_K, cudaStream_t st, bool pdl);
 // Group order of every layer with a random partition (DevLayer::member /
 // group_of); redraw: keyed by the current step (else by step 0).
 cudaError_t prepare_group_order(int max_K);  // shared-memory attribute, once

@@ -14,15 +14,6 @@ __device__ __forceinline__ int warp_sum(int v) {
   return v;
 }
 
-__device__ __forceinline__ int64_t batch_start(const StepParams* P) {
-  return (int64_t)P->ctrl->s * P->bs;
-}
-
-__device__ __forceinline__ int64_t batch_size(const StepParams* P, int64_t start) {
-  const int64_t rem = P->n - start;
-  return rem < P->bs ? rem : P->bs;
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -32,47 +23,70 @@ __device__ __forceinline__ int64_t batch_size(const StepParams* P, int64_t start
 //   pred = argmax (lowest j), loss = [pred != y], tau = top1 - top2   (Eq. 1, l.12-13)
 //   mark = loss or tau * r_den < r_num * K_l                         (l.14-15)
 //   for marked mu, group g: sel = argmax_{k in g} {delta_k < 0},
-//   delta_k = z_k rho_{k,y}, ties to the lowest k; -1 if none        (Alg. 2 l.4-8)
+//   delta_k = z_k rho_{k,y}, ties to the lowest k; none if there is none
+//                                                                    (Alg. 2 l.4-8)
 // Launched as a programmatic dependent of the last layer's forward pass: the
 // CTAs of layers l < L read only what kernels two or more launches back wrote
 // (their layer's Z and A, the batch index), so they do all their work before
-// waiting, overlapping that forward pass; the CTAs of layer L wait first.
-// Every CTA waits before it lets the next kernel start, so a kernel two
-// launches back has always completed.
+// waiting, overlapping that forward pass; the CTAs of layer L wait first (all
+// CTAs where the kernel before this one writes the group order).  Every CTA
+// waits before it lets the next kernel start, so a kernel two launches back
+// has always completed.
+// Bound: a chain of dependent L2 loads (batch index, label, rho) and two
+// barriers, so the model comes as a kernel parameter, z and rho are loaded
+// beside the classifier's words, and one warp finds the two largest scores
+// (with one thread walking over 100 classes the launch of 3072-4096x4 took 16.3 us,
+// now 12.3, 5 of them the two events around it).
 // ---------------------------------------------------------------------------
-// A candidate's sort key (neuron, then the sign of its rho: delta = z rho < 0,
-// so rho is -1 exactly where z > 0) and the selection it becomes.
-__device__ __forceinline__ int sel_key(int k, int z) { return 2 * k + (z > 0 ? 1 : 0); }
-__device__ __forceinline__ uint16_t sel_of(int key) { return (uint16_t)((key >> 1) | ((key & 1) << 15)); }
+namespace {
 
-__device__ __forceinline__ void cls_select_body(const StepParams* __restrict__ P, int li, int mu);
-
-__global__ void __launch_bounds__(kClsThreads) k_cls_select(const StepParams* __restrict__ P) {
-  const int li = blockIdx.y;
-  const int mu = blockIdx.x;
-  const bool early = li < P->L - 1;
-  if (!early) {
-    pdl_wait();
-    pdl_trigger();
-  }
-  cls_select_body(P, li, mu);
-  if (early) {
-    pdl_wait();
-    pdl_trigger();
-  }
+// A candidate: larger is better.  delta < 0 first, then the lowest neuron; the
+// low half is the complement of 2 k + [rho = -1] (delta = z rho < 0, so rho is -1
+// exactly where z > 0).  0: no candidate.
+__device__ __forceinline__ uint32_t candidate(int k, int z, int rho) {
+  const int d = z * rho;
+  return d < 0 ? ((uint32_t)(d + 32768) << 16) | (0xFFFFu - (uint32_t)(2 * k + (z > 0 ? 1 : 0))) : 0u;
+}
+__device__ __forceinline__ uint16_t selection(uint32_t cand) {
+  const uint32_t key = 0xFFFFu - (cand & 0xFFFFu);
+  return cand == 0u ? kNoSel : (uint16_t)((key >> 1) | ((key & 1u) << 15));
 }
 
-__device__ __forceinline__ void cls_select_body(const StepParams* __restrict__ P, int li, int mu) {
-  const DevLayer& Ly = P->layer[li];
-  Ctrl* ctrl = P->ctrl;
-  const int64_t start = batch_start(P);
-  const int64_t bsz = batch_size(P, start);
-  if (mu >= bsz) return;
+__device__ __forceinline__ void cls_select_body(const ClsArgs& C, int li, int mu) {
+  const ClsLayer& Ly = C.layer[li];
+  Ctrl* ctrl = C.ctrl;
   __shared__ int yh[BMLP_MAX_CLASSES];
-  __shared__ int s_mark, s_y, s_timeout;
+  __shared__ int s_mark, s_timeout;
+  const int64_t start = (int64_t)ctrl->s * C.bs;
+  if (mu >= C.P->n - start) return;
+  const int c = C.c;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+  const int label = C.P->y[start + mu];
+  const int y = (label < 0 || label >= c) ? 0 : label;  // memory-safe stand-in; the host reports BMLP_EINVAL
   // one read of the counter for the whole CTA (the last forward pass may be
   // running beside an early CTA and could raise it meanwhile)
   if (threadIdx.x == 0) s_timeout = ctrl->timeouts != 0u;
+  const int K = Ly.Kout, gamma = Ly.gamma;
+  const int16_t* z = Ly.Z + (int64_t)mu * K;
+  const int8_t* rt = Ly.rhoT + (int64_t)y * K;
+  // contiguous groups of 8, 16, .. 256 neurons: one thread per 8 neurons
+  const int per = gamma >> 3;  // 8-neuron chunks per group
+  const bool chunks = Ly.member == nullptr && (gamma & 7) == 0 && per <= 32 && (per & (per - 1)) == 0;
+  const int nchunk = K >> 3;
+  uint4 zv = make_uint4(0, 0, 0, 0);
+  uint2 rv = make_uint2(0, 0);
+  if (chunks && (int)threadIdx.x < nchunk) {
+    zv = *reinterpret_cast<const uint4*>(z + 8 * threadIdx.x);
+    rv = *reinterpret_cast<const uint2*>(rt + 8 * threadIdx.x);
+  }
+  const uint64_t* a = Ly.A + (int64_t)mu * Ly.nw_out;
+  for (int j = warp; j < c; j += nwarps) {
+    const uint64_t* pt = Ly.PT + (int64_t)j * Ly.nw_out;
+    int cnt = 0;
+    for (int w = lane; w < Ly.nw_out; w += 32) cnt += __popcll(a[w] ^ pt[w]);
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0) yh[j] = K - 2 * cnt;
+  }
   __syncthreads();
   if (s_timeout) {
     // a bounded wait of this step's forward pass expired (or an earlier one
@@ -83,115 +97,95 @@ __device__ __forceinline__ void cls_select_body(const StepParams* __restrict__ P
     if (threadIdx.x == 0) Ly.mark[mu] = 0;
     return;
   }
-  const int c = P->c;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-
-  const uint64_t* a = Ly.A + (int64_t)mu * Ly.nw_out;
-  for (int j = warp; j < c; j += nwarps) {
-    const uint64_t* pt = Ly.PT + (int64_t)j * Ly.nw_out;
-    int cnt = 0;
-    for (int w = lane; w < Ly.nw_out; w += 32) cnt += __popcll(a[w] ^ pt[w]);
-    cnt = warp_sum(cnt);
-    if (lane == 0) yh[j] = Ly.Kout - 2 * cnt;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int yv = P->y[start + mu];
-    if (yv < 0 || yv >= c) {
-      if (li == 0) atomicAdd(&ctrl->bad_labels, 1ull);
-      yv = 0;  // memory-safe stand-in; the host reports BMLP_EINVAL
+  if (warp == 0) {
+    // the two largest scores; equal ones differ in the class (lowest first)
+    uint32_t b1 = 0u, b2 = 0u;
+    for (int j = lane; j < c; j += 32) {
+      const uint32_t v = ((uint32_t)(yh[j] + 32768) << 10) | (uint32_t)(BMLP_MAX_CLASSES - 1 - j);
+      b2 = max(b2, min(b1, v));
+      b1 = max(b1, v);
     }
-    int jmax = 0;
-    for (int j = 1; j < c; ++j)
-      if (yh[j] > yh[jmax]) jmax = j;
-    int second = INT_MIN;
-    for (int j = 0; j < c; ++j)
-      if (j != jmax && yh[j] > second) second = yh[j];
-    const int tau = yh[jmax] - second;
-    const int loss = (jmax != yv) ? 1 : 0;
-    const int mark = loss || ((long long)tau * P->r_den < (long long)P->r_num * Ly.Kout);
-    Ly.mark[mu] = (uint8_t)mark;
-    if (mark) atomicOr(&ctrl->any_mark[li], 1u);
-    if (loss) atomicAdd(&ctrl->layer_err[li], 1ull);
-    if (li == P->L - 1 && loss) atomicAdd(&ctrl->err, 1ull);
-    s_mark = mark;
-    s_y = yv;
+    const uint32_t m1 = __reduce_max_sync(0xffffffffu, b1);
+    const uint32_t m2 = __reduce_max_sync(0xffffffffu, b1 == m1 ? b2 : b1);
+    if (lane == 0) {
+      if (label != y && li == 0) atomicAdd(&ctrl->bad_labels, 1ull);
+      const int tau = (int)(m1 >> 10) - (int)(m2 >> 10);
+      const int loss = (BMLP_MAX_CLASSES - 1 - (int)(m1 & 1023u)) != y ? 1 : 0;
+      const int mark = loss || ((long long)tau * C.r_den < (long long)C.r_num * K);
+      Ly.mark[mu] = (uint8_t)mark;
+      if (mark) atomicOr(&ctrl->any_mark[li], 1u);
+      if (loss) atomicAdd(&ctrl->layer_err[li], 1ull);
+      if (li == C.L - 1 && loss) atomicAdd(&ctrl->err, 1ull);
+      s_mark = mark;
+    }
   }
   __syncthreads();
 
   // selections are stored group-major (sel[g][mu]): the update kernel reads a
   // group's bs selections as one contiguous run
   uint16_t* sel = Ly.sel + mu;
-  const int64_t sstride = P->bs;
+  const int64_t sstride = C.bs;
   if (!s_mark) {
     for (int g = threadIdx.x; g < Ly.G; g += blockDim.x) sel[g * sstride] = kNoSel;
     return;
   }
-  const int y = s_y;
-  const int16_t* z = Ly.Z + (int64_t)mu * Ly.Kout;
-  const int gamma = Ly.gamma;
-  const int per = gamma >> 3;  // 8-neuron chunks per group
-  if (Ly.member == nullptr && (gamma & 7) == 0 && per <= 32 && (per & (per - 1)) == 0) {
-    // one thread per 8 neurons: 16-byte z loads, 8 bytes of rho^T, then the
-    // group's per lanes (consecutive, aligned) reduce with shuffles
-    const int8_t* rt = Ly.rhoT + (int64_t)y * Ly.Kout;
-    const int nchunk = Ly.Kout >> 3;
+  if (chunks) {
+    // the group's per lanes (consecutive, aligned) reduce with shuffles
     for (int base = 0; base < nchunk; base += blockDim.x) {
       const int ci = base + threadIdx.x;
-      int bestd = INT_MIN, bestk = INT_MAX;
+      if (base > 0 && ci < nchunk) {
+        zv = *reinterpret_cast<const uint4*>(z + 8 * ci);
+        rv = *reinterpret_cast<const uint2*>(rt + 8 * ci);
+      }
+      uint32_t best = 0u;
       if (ci < nchunk) {
-        const uint4 zv = *reinterpret_cast<const uint4*>(z + 8 * ci);
-        const uint2 rv = *reinterpret_cast<const uint2*>(rt + 8 * ci);
         const uint32_t zw[4] = {zv.x, zv.y, zv.z, zv.w};
         const uint32_t rw[2] = {rv.x, rv.y};
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int zj = (int)(int16_t)(zw[j >> 1] >> (16 * (j & 1)));
-          const int rj = (int)(int8_t)(rw[j >> 2] >> (8 * (j & 3)));
-          const int d = zj * rj;
-          if (d < 0 && d > bestd) {  // ascending k: strict '>' keeps the lowest
-            bestd = d;
-            bestk = sel_key(8 * ci + j, zj);
-          }
-        }
+        for (int j = 0; j < 8; ++j)
+          best = max(best, candidate(8 * ci + j, (int)(int16_t)(zw[j >> 1] >> (16 * (j & 1))),
+                                     (int)(int8_t)(rw[j >> 2] >> (8 * (j & 3)))));
       }
-      for (int off = per >> 1; off > 0; off >>= 1) {
-        const int od = __shfl_xor_sync(0xffffffffu, bestd, off);
-        const int ok = __shfl_xor_sync(0xffffffffu, bestk, off);
-        if (od > bestd || (od == bestd && ok < bestk)) {
-          bestd = od;
-          bestk = ok;
-        }
-      }
-      if (ci < nchunk && (ci & (per - 1)) == 0)
-        sel[(ci / per) * sstride] = bestd == INT_MIN ? kNoSel : sel_of(bestk);
+      for (int off = per >> 1; off > 0; off >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, off));
+      if (ci < nchunk && (ci & (per - 1)) == 0) sel[(ci / per) * sstride] = selection(best);
     }
     return;
   }
   // warp per group; the group's neurons are contiguous or listed by the group
-  // order (random partition), so ties compare neuron indices explicitly
+  // order (random partition)
   const int16_t* member = Ly.member;
   for (int g = warp; g < Ly.G; g += nwarps) {
-    int bestd = INT_MIN, bestk = INT_MAX;
+    uint32_t best = 0u;
     for (int kk = lane; kk < gamma; kk += 32) {
       const int k = member ? (int)member[g * gamma + kk] : g * gamma + kk;
-      const int d = (int)z[k] * (int)Ly.rho[(int64_t)k * c + y];
-      if (d < 0 && (d > bestd || (d == bestd && sel_key(k, z[k]) < bestk))) {
-        bestd = d;
-        bestk = sel_key(k, z[k]);
-      }
+      best = max(best, candidate(k, (int)z[k], (int)rt[k]));
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const int od = __shfl_xor_sync(0xffffffffu, bestd, off);
-      const int ok = __shfl_xor_sync(0xffffffffu, bestk, off);
-      if (od > bestd || (od == bestd && ok < bestk)) {
-        bestd = od;
-        bestk = ok;
-      }
-    }
-    if (lane == 0) sel[g * sstride] = bestd == INT_MIN ? kNoSel : sel_of(bestk);
+    best = __reduce_max_sync(0xffffffffu, best);
+    if (lane == 0) sel[g * sstride] = selection(best);
   }
+}
+
+__global__ void __launch_bounds__(512) k_cls_select(const __grid_constant__ ClsArgs C) {
+  const int li = blockIdx.y;
+  const int mu = blockIdx.x;
+  const bool early = C.early && li < C.L - 1;
+  if (!early) {
+    pdl_wait();
+    pdl_trigger();
+  }
+  cls_select_body(C, li, mu);
+  if (early) {
+    pdl_wait();
+    pdl_trigger();
+  }
+}
+
+}  // namespace
+
+cudaError_t launch_cls_select(const ClsArgs& C, int max_K, cudaStream_t st, bool pdl) {
+  // a thread per 8 neurons of the widest layer, 4 to 16 warps
+  const int threads = max_K <= 1024 ? 128 : (max_K <= 2048 ? 256 : 512);
+  return launch_kernel(k_cls_select, dim3((unsigned)C.bs, (unsigned)C.L), dim3(threads), 0, st, pdl, C);
 }
 
 namespace {
