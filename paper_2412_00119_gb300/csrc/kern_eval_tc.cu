@@ -24,13 +24,17 @@
 //   - 16 producer warps in two groups take alternate k-steps of 256 elements: in
 //     a group four warps expand the pattern rows into 32 tensor-memory columns
 //     and four the weight rows into a 16 KB stage (128B swizzle);
-//   - one thread of the even CTA issues the MMAs (a relay thread of the odd CTA
-//     forwards its "full" barrier, so no thread with copies in flight executes
-//     a cluster-scope release) and commits to the "empty" barriers of both;
+//   - one thread of the even CTA issues the MMAs and commits to the "empty"
+//     barriers of both; kRelays threads of the odd CTA, each in a warp of its own,
+//     take its k-steps in turn and forward their "full" barriers (a remote
+//     arrival with cluster-scope release takes 720 clocks; one thread doing them
+//     all set the pace, 1,000 clocks per k-step);
 //   - 8 epilogue warps read D (a lane per pattern), shift the sign bits into
 //     words and store 128 neurons of a row at once.
-// Measured, 65,536 patterns through 8192 -> 8192: 1.86 ms = 4.75 PFLOP/s (the e4m3
-// kernel before it 2.79 ms).
+// Measured, 65,536 patterns through 8192 -> 8192x4: 4.60 ms = 7.67 PFLOP/s (the
+// e4m3 kernel before it 11.2 ms; this one with one relay and the MMAs issued
+// under `lane == 0` 7.43 ms).  A k-step takes 566 clocks where its MMAs take 512,
+// and a tile 3,100 more until both CTAs' accumulators are read.
 // Every mbarrier wait is bounded; the first expiry stops every other wait of
 // the CTA and the kernel counts it in *timeouts, releases its tensor memory
 // and returns.
@@ -54,14 +58,15 @@ constexpr int B_BYTES = TB * 128;        // one weight stage
 constexpr int kGroups = 2;
 constexpr int kProdWarps = 8 * kGroups;
 constexpr int kLoadWarps = 4, kEpiWarps = 8;
+constexpr int kRelays = 4;               // the MMA warp (of the odd CTA) and three more
 constexpr int kMmaWarp = kProdWarps;
-constexpr int kLoad0 = kMmaWarp + 1, kEpi0 = kLoad0 + kLoadWarps;
+constexpr int kLoad0 = kMmaWarp + kRelays, kEpi0 = kLoad0 + kLoadWarps;
 constexpr int THREADS = 32 * (kEpi0 + kEpiWarps);
 constexpr int TMEM_COLS = 512;
 constexpr int kSfCol = TN;               // 16 + 16 columns of unit scales (A, B)
 constexpr int kStageCol = kSfCol + 32;   // pattern stages of 32 columns
 static_assert(kStageCol + 32 * kStages <= TMEM_COLS, "TMEM budget");
-static_assert(kEpi0 % 4 == 1, "an epilogue warp's lane quarter is its number modulo 4");
+static_assert(THREADS <= 1024, "threads of a CTA");
 constexpr uint32_t kIdesc = idesc_f4(2 * TM, TN);
 
 struct __align__(8) EvShared {
@@ -93,13 +98,18 @@ __device__ __forceinline__ void pair_sync() {
 __device__ __forceinline__ bool mbar_wait_cluster(unsigned long long* bar, uint32_t parity,
                                                   volatile int* failed) {
   const uint32_t a = smem_u32(bar);
-  const unsigned long long t0 = clock64();
-  while (true) {
-    uint32_t ok;
+  uint32_t ok;
+  auto try_wait = [&]() {
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
         " selp.u32 %0, 1, 0, p;\n}"
         : "=r"(ok) : "r"(a), "r"(parity) : "memory");
+  };
+  try_wait();
+  if (ok) return true;
+  const unsigned long long t0 = clock64();
+  while (true) {
+    try_wait();
     if (ok) return true;
     if (*failed) return false;
     if (clock64() - t0 > kWaitCycles) {
@@ -197,28 +207,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     const uint32_t brow0 = smem_u32(bits) + (uint32_t)((awarp ? r : TM + r) * kBitRow);
     const uint32_t srow = smem_u32(base) + 128u * (uint32_t)r;
     const uint32_t lanes = (uint32_t)(32 * q) << 16;
-    uint32_t pc = 0;          // pieces so far: ring slot pc % kPieces
-    uint32_t kc0 = 0;         // k-steps of the finished tiles
+    const uint32_t sw = 16u * (uint32_t)(r & 7);
+    uint32_t slot = 0, bph = 0;                        // ring slot of the piece, its parity
+    uint32_t s = (uint32_t)grp, eph = 1;               // stage of the group's next k-step, parity of "empty"
+    int ks = grp;                                      // that k-step, counted in the current tile
     bool ok = true;
 #pragma unroll 1
-    for (int64_t t = pair; t < tiles && ok; t += pairs, kc0 += (uint32_t)nks) {
+    for (int64_t t = pair; t < tiles && ok; t += pairs, ks -= nks) {
 #pragma unroll 1
-      for (int p = 0; p < npc && ok; ++p, ++pc) {
-        const uint32_t slot = pc % kPieces;
-        ok = __all_sync(kFull, mbar_wait(&sh->bits_full[slot], (pc / kPieces) & 1u, failed));
+      for (int p = 0; p < npc && ok; ++p) {
+        ok = __all_sync(kFull, mbar_wait(&sh->bits_full[slot], bph, failed));
         const uint32_t brow = brow0 + slot * (uint32_t)kBitBytes;
         const int kend = min(nks, kSteps * (p + 1));
 #pragma unroll 1
-        for (int ks = kSteps * p; ks < kend && ok; ++ks) {
-          const uint32_t kc = kc0 + (uint32_t)ks;          // stage kc % kStages
-          if ((kc & (kGroups - 1)) != (uint32_t)grp) continue;
-          const uint32_t s = kc % kStages, use = kc / kStages;
-          if (use > 0) ok = __all_sync(kFull, mbar_wait(&sh->empty[s], (use - 1) & 1u, failed));
-          if (!ok) break;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        for (; ks < kend && ok; ks += kGroups) {
           const uint32_t src = brow + 32u * (uint32_t)(ks - kSteps * p);
           const uint4 lo = lds128(src), hi = lds128(src + 16);
           uint32_t x[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+          ok = __all_sync(kFull, mbar_wait(&sh->empty[s], eph, failed));
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           if (awarp) {
             if (Kin - KF * ks < KF) {
               // pad bits, whatever the caller left in the rows' last word, count as +1
@@ -231,19 +239,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
           } else {
+            const uint32_t row = (srow + s * (uint32_t)B_BYTES) | sw;   // chunk c at row ^ 16 c
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
               uint32_t v[4];
               e2m1_words(x[c], v);
-              sts128(srow + s * (uint32_t)B_BYTES + 16u * (uint32_t)(c ^ (r & 7)), v);
+              sts128(row ^ (16u * c), v);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(&sh->full[s]);
+          s += kGroups;
+          if (s >= kStages) {
+            s -= kStages;
+            eph ^= 1u;
+          }
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&sh->bits_empty[slot]);
+        if (++slot == kPieces) {
+          slot = 0;
+          bph ^= 1u;
+        }
       }
     }
   } else if (warp >= kLoad0 && warp < kEpi0) {
@@ -251,71 +269,87 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     constexpr int kPer = 128 / kAlign;      // copies per row
     const int tid = threadIdx.x - 32 * kLoad0;
     const int c = tid % kPer, r0 = tid / kPer;
-    uint32_t pc = 0;
+    constexpr int kStep = 32 * kLoadWarps / kPer;   // rows between a thread's copies
+    uint32_t slot = 0, ph = 1;
     bool ok = true;
+    const uint32_t dst0 = smem_u32(bits) + (uint32_t)(r0 * kBitRow + kAlign * c);
 #pragma unroll 1
     for (int64_t t = pair; t < tiles && ok; t += pairs) {
       const int64_t m0 = (t / ntiles) * (2 * TM) + (int64_t)rank * TM;
       const int nb = (int)(t % ntiles) * TN + (int)rank * TB;
-      const int64_t alive = M - m0, wlive = N - nb;
+      // copies of this thread that are inside the operands' rows
+      const int la = (int)max((int64_t)0, min((int64_t)(TM / kStep), (M - m0 - r0 + kStep - 1) / kStep));
+      const int lw = max(0, min(TB / kStep, (N - nb - r0 + kStep - 1) / kStep));
+      const uint64_t* arow = A + (m0 + r0) * nw + (kAlign / 8) * c;
+      const uint64_t* wrow = W + (int64_t)(nb + r0) * nw + (kAlign / 8) * c;
 #pragma unroll 1
-      for (int p = 0; p < npc && ok; ++p, ++pc) {
-        const uint32_t slot = pc % kPieces, use = pc / kPieces;
-        if (use > 0) ok = mbar_wait(&sh->bits_empty[slot], (use - 1) & 1u, failed);
+      for (int p = 0; p < npc && ok; ++p) {
+        ok = mbar_wait(&sh->bits_empty[slot], ph, failed);
         if (!ok) break;
-        const uint32_t dst = smem_u32(bits) + slot * (uint32_t)kBitBytes + (uint32_t)(kAlign * c);
-        const int w = kPieceWords * p + (kAlign / 8) * c;
-        const bool won = w < nw;
+        const uint32_t dst = dst0 + slot * (uint32_t)kBitBytes;
+        const bool won = kPieceWords * p + (kAlign / 8) * c < nw;
+        const uint64_t* pa = arow + kPieceWords * p;
+        const uint64_t* pw = wrow + kPieceWords * p;
 #pragma unroll 4
-        for (int r = r0; r < TM; r += 32 * kLoadWarps / kPer) {
-          const bool on = won && r < alive;
-          cp_async_or_zero<kAlign>(dst + (uint32_t)(r * kBitRow), on ? A + (m0 + r) * nw + w : A, on);
+        for (int i = 0; i < TM / kStep; ++i, pa += kStep * nw) {
+          const bool on = won && i < la;
+          cp_async_or_zero<kAlign>(dst + (uint32_t)(i * kStep * kBitRow), on ? pa : A, on);
         }
 #pragma unroll 4
-        for (int r = r0; r < TB; r += 32 * kLoadWarps / kPer) {
-          const bool on = won && r < wlive;
-          cp_async_or_zero<kAlign>(dst + (uint32_t)((TM + r) * kBitRow), on ? W + (int64_t)(nb + r) * nw + w : W,
-                                   on);
+        for (int i = 0; i < TB / kStep; ++i, pw += kStep * nw) {
+          const bool on = won && i < lw;
+          cp_async_or_zero<kAlign>(dst + (uint32_t)((TM + i * kStep) * kBitRow), on ? pw : W, on);
         }
         cp_async_arrive(&sh->bits_full[slot]);
+        if (++slot == kPieces) {
+          slot = 0;
+          ph ^= 1u;
+        }
       }
     }
     cp_async_wait_all();   // no copy outlives its thread
-  } else if (warp == kMmaWarp && lane == 0) {
-    uint32_t kc = 0, tile = 0;
+  } else if (warp >= kMmaWarp && warp < kLoad0) {
     bool ok = true;
-    if (rank == 0) {
+    if (rank == 0 && warp == kMmaWarp) {
       // ---------------- MMA issuer of the pair ----------------
-#pragma unroll 1
-      for (int64_t t = pair; t < tiles && ok; t += pairs, ++tile) {
-        if (tile > 0) ok = mbar_wait_cluster(&sh->drained, (tile - 1) & 1u, failed);
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll 1
-        for (int ks = 0; ks < nks && ok; ++ks, ++kc) {
-          const uint32_t s = kc % kStages;
-          ok = mbar_wait_cluster(&sh->full[s], (kc / kStages) & 1u, failed);
-          if (!ok) break;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint64_t bd = smem_desc(smem_u32(base + s * B_BYTES));
-          const uint32_t ta = tmem + (uint32_t)kStageCol + 32u * s;
-#pragma unroll
-          for (int e = 0; e < 4; ++e)
-            mma_f4_pair(tmem, ta + 8 * e, bd + 2 * e, tmem + kSfCol, tmem + kSfCol + 16,
-                        (ks > 0 || e > 0) ? 1u : 0u);
-          mma_commit_pair(&sh->empty[s]);
-        }
-        if (ok) mma_commit_pair(&sh->done);
-      }
-    } else {
-      // relay of the odd CTA: its stage is full -> one arrival on the even CTA's
+      const bool lead = elect_one();
+      const uint32_t d = uniform(tmem);
+      const uint64_t bd0 = smem_desc(uniform(smem_u32(base)));
+      uint32_t s = 0, ph = 0, dph = 1;
 #pragma unroll 1
       for (int64_t t = pair; t < tiles && ok; t += pairs) {
+        ok = __all_sync(kFull, mbar_wait_cluster(&sh->drained, dph, failed));
+        dph ^= 1u;
 #pragma unroll 1
-        for (int ks = 0; ks < nks && ok; ++ks, ++kc) {
-          const uint32_t s = kc % kStages;
-          ok = mbar_wait(&sh->full[s], (kc / kStages) & 1u, failed);
-          if (ok) mbar_arrive_rank0(&sh->full[s]);
+        for (int ks = 0; ks < nks && ok; ++ks) {
+          ok = __all_sync(kFull, mbar_wait_cluster(&sh->full[s], ph, failed));
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint64_t bd = bd0 + (uint64_t)(s * (uint32_t)(B_BYTES >> 4));
+          const uint32_t ta = d + (uint32_t)kStageCol + 32u * s;
+          if (lead) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              mma_f4_pair(d, ta + 8 * e, bd + 2 * e, d + kSfCol, d + kSfCol + 16, (ks > 0 || e > 0) ? 1u : 0u);
+            mma_commit_pair(&sh->empty[s]);
+          }
+          if (++s == kStages) {
+            s = 0;
+            ph ^= 1u;
+          }
         }
+        if (ok && lead) mma_commit_pair(&sh->done);
+        __syncwarp();
+      }
+    } else if (rank != 0 && lane == 0) {
+      // relays of the odd CTA: its stage is full -> one arrival on the even CTA's
+      const int64_t mine = (tiles - pair + pairs - 1) / pairs;   // tiles of this pair
+      const uint64_t last = pair < tiles ? (uint64_t)mine * (uint64_t)nks : 0ull;
+#pragma unroll 1
+      for (uint64_t k = (uint64_t)(warp - kMmaWarp); k < last && ok; k += kRelays) {
+        const uint32_t s = (uint32_t)(k % kStages);
+        ok = mbar_wait(&sh->full[s], (uint32_t)(k / kStages) & 1u, failed);
+        if (ok) mbar_arrive_rank0(&sh->full[s]);
       }
     }
   } else if (warp >= kEpi0) {
@@ -330,17 +364,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       if (!__all_sync(kFull, mbar_wait(&sh->done, tile & 1u, failed))) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       uint32_t word[4];
-#pragma unroll
-      for (int cb = 0; cb < 4; ++cb) {
-        uint32_t v[32];
-        tmem_load32(v, tmem + ((uint32_t)(32 * sub) << 16) + (uint32_t)(128 * half + 32 * cb));
-        // z = sum - npad; its sign bit (0 for z = 0) into the word, column 0 first
-        uint32_t acc = 0u;
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          acc = __funnelshift_l(__float_as_uint(__uint_as_float(v[j]) - npad), acc, 1);
-        word[cb] = ~__brev(acc);
-      }
+      sign_words<4>(word, tmem + ((uint32_t)(32 * sub) << 16) + (uint32_t)(128 * half), 4, npad);
       // D is read: the pair's next tile may overwrite it
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();

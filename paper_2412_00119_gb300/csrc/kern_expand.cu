@@ -28,7 +28,8 @@
 //   - 8 epilogue warps read the sums (a lane per pattern), shift the sign bits
 //     into words and store them.
 // Bound: the MMAs, 4 x 128 clocks per chunk of a 128 x 256 tile.  60,000 x 784
-// -> 1024: 93.6 us (the dp4a kernel 804 us), of which the MMAs are 43.
+// -> 1024: 76 us (the dp4a kernel 804 us), of which the MMAs are 43; a chunk takes
+// 590 clocks where its MMAs take 512, a tile 2,200 more for its epilogue.
 // Every mbarrier wait is bounded like all others of the library; this entry
 // point has no handle, so an expiry leaves its tiles unwritten.
 //
@@ -292,20 +293,18 @@ __global__ void __launch_bounds__(kXTcThreads, 1)
     const int grp = warp >> 2, q = warp & 3;
     const uint32_t row0 = smem_u32(pieces) + (uint32_t)((32 * q + lane) * kXRow);
     const uint32_t lanes = (uint32_t)(32 * q) << 16;
-    uint32_t pc = 0, kc0 = 0;
+    uint32_t slot = 0, pph = 0;                        // ring slot of the piece, its parity
+    uint32_t s = (uint32_t)grp, eph = 1;               // stage of the group's next chunk, parity of "empty"
+    int ch = grp;                                      // that chunk, counted in the current tile
     bool ok = true;
 #pragma unroll 1
-    for (int64_t t = blockIdx.y; t < tiles && ok; t += gridDim.y, kc0 += (uint32_t)nchunks) {
+    for (int64_t t = blockIdx.y; t < tiles && ok; t += gridDim.y, ch -= nchunks) {
 #pragma unroll 1
-      for (int p = 0; p < npc && ok; ++p, ++pc) {
-        const uint32_t slot = pc % kXPieces;
-        ok = __all_sync(0xffffffffu, mbar_wait(&sh->piece_full[slot], (pc / kXPieces) & 1u, failed));
+      for (int p = 0; p < npc && ok; ++p) {
+        ok = __all_sync(0xffffffffu, mbar_wait(&sh->piece_full[slot], pph, failed));
         const int cend = min(nchunks, 4 * (p + 1));
 #pragma unroll 1
-        for (int ch = 4 * p; ch < cend && ok; ++ch) {
-          const uint32_t kc = kc0 + (uint32_t)ch;
-          if ((kc & (kXGroups - 1)) != (uint32_t)grp) continue;
-          const uint32_t s = kc % kXStages, use = kc / kXStages;
+        for (; ch < cend && ok; ch += kXGroups) {
           uint32_t w[16];
           const uint32_t src = row0 + slot * (uint32_t)kXPieceBytes + (uint32_t)(kChunk * (ch - 4 * p));
 #pragma unroll
@@ -313,7 +312,7 @@ __global__ void __launch_bounds__(kXTcThreads, 1)
             const uint4 v = lds128(src + 16u * i);
             w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
           }
-          if (use > 0) ok = __all_sync(0xffffffffu, mbar_wait(&sh->empty[s], (use - 1) & 1u, failed));
+          ok = __all_sync(0xffffffffu, mbar_wait(&sh->empty[s], eph, failed));
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
@@ -326,9 +325,18 @@ __global__ void __launch_bounds__(kXTcThreads, 1)
           asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
           __syncwarp();
           if (lane == 0) mbar_arrive(&sh->full[s]);
+          s += kXGroups;
+          if (s >= kXStages) {
+            s -= kXStages;
+            eph ^= 1u;
+          }
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&sh->piece_empty[slot]);
+        if (++slot == kXPieces) {
+          slot = 0;
+          pph ^= 1u;
+        }
       }
     }
   } else if (warp >= kXLoad0 && warp < kXEpi0) {
@@ -336,62 +344,80 @@ __global__ void __launch_bounds__(kXTcThreads, 1)
     constexpr int kStep = kBytes == 1 ? 4 : kBytes;   // bytes per store to shared memory
     constexpr int kPer = kXPiece / kStep;
     const int tid = threadIdx.x - 32 * kXLoad0;
-    uint32_t pc = 0;
+    constexpr int kRows = 32 * kXLoadWarps / kPer > 0 ? 32 * kXLoadWarps / kPer : 1;   // rows per round of copies
+    constexpr int kCols = kPer / (32 * kXLoadWarps) > 0 ? kPer / (32 * kXLoadWarps) : 1;   // columns of a thread
+    const int r0 = tid / kPer, c0 = kStep * (tid % kPer);
+    uint32_t slot = 0, ph = 1;
     bool ok = true;
 #pragma unroll 1
     for (int64_t t = blockIdx.y; t < tiles && ok; t += gridDim.y) {
-      const uint8_t* rows = x + t * XM * D;
-      const int live = (int)min((int64_t)XM, n - t * XM);
+      const uint8_t* rows = x + (t * XM + r0) * D + c0;
+      const int live = (int)min((int64_t)XM, n - t * XM) - r0;
 #pragma unroll 1
-      for (int p = 0; p < npc && ok; ++p, ++pc) {
-        const uint32_t slot = pc % kXPieces, use = pc / kXPieces;
-        if (use > 0) ok = mbar_wait(&sh->piece_empty[slot], (use - 1) & 1u, failed);
+      for (int p = 0; p < npc && ok; ++p) {
+        ok = mbar_wait(&sh->piece_empty[slot], ph, failed);
         if (!ok) break;
-        const uint32_t dst = smem_u32(pieces) + slot * (uint32_t)kXPieceBytes;
+#pragma unroll 1
+        for (int e = 0; e < kCols; ++e) {
+          const int c = kXPiece * p + c0 + e * 32 * kXLoadWarps * kStep;   // the copy's first input
+          const uint8_t* src = rows + kXPiece * p + e * 32 * kXLoadWarps * kStep;
+          uint32_t to = smem_u32(pieces) + slot * (uint32_t)kXPieceBytes +
+                        (uint32_t)(r0 * kXRow + c0 + e * 32 * kXLoadWarps * kStep);
 #pragma unroll 4
-        for (int i = tid; i < XM * kPer; i += 32 * kXLoadWarps) {
-          const int r = i / kPer, c = kXPiece * p + kStep * (i % kPer);
-          const uint32_t to = dst + (uint32_t)(r * kXRow + kStep * (i % kPer));
-          const uint8_t* src = rows + (int64_t)r * D + c;
-          if constexpr (kBytes == 1) {
-            uint32_t v = 0;
+          for (int i = 0; i < XM; i += kRows, src += (int64_t)kRows * D, to += (uint32_t)(kRows * kXRow)) {
+            if constexpr (kBytes == 1) {
+              uint32_t v = 0;
 #pragma unroll
-            for (int b = 0; b < 4; ++b)
-              if (r < live && c + b < D) v |= (uint32_t)__ldg(src + b) << (8 * b);
-            asm volatile("st.shared.b32 [%0], %1;" ::"r"(to), "r"(v) : "memory");
-          } else {
-            const bool on = r < live && c < D;   // D is a multiple of kBytes
-            cp_async_or_zero<kBytes>(to, on ? src : x, on);
+              for (int b = 0; b < 4; ++b)
+                if (i < live && c + b < D) v |= (uint32_t)__ldg(src + b) << (8 * b);
+              asm volatile("st.shared.b32 [%0], %1;" ::"r"(to), "r"(v) : "memory");
+            } else {
+              const bool on = i < live && c < D;   // D is a multiple of kBytes
+              cp_async_or_zero<kBytes>(to, on ? src : x, on);
+            }
           }
         }
         if constexpr (kBytes == 1) mbar_arrive(&sh->piece_full[slot]);
         else cp_async_arrive(&sh->piece_full[slot]);
+        if (++slot == kXPieces) {
+          slot = 0;
+          ph ^= 1u;
+        }
       }
     }
     cp_async_wait_all();   // no copy outlives its thread
-  } else if (warp == kXMma && lane == 0) {
+  } else if (warp == kXMma) {
     // ---------------- MMA issuer ----------------
+    const bool lead = elect_one();
+    const uint32_t d = uniform(tmem);
+    const uint64_t bd0 = smem_desc(uniform(smem_u32(base)));
     const uint32_t idesc = idesc_f4(XM, nb);
-    uint32_t kc = 0, tile = 0;
+    uint32_t s = 0, ph = 0, dph = 1;
     bool ok = true;
 #pragma unroll 1
-    for (int64_t t = blockIdx.y; t < tiles && ok; t += gridDim.y, ++tile) {
-      if (tile > 0) ok = mbar_wait(&sh->drained, (tile - 1) & 1u, failed);
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    for (int64_t t = blockIdx.y; t < tiles && ok; t += gridDim.y) {
+      ok = __all_sync(0xffffffffu, mbar_wait(&sh->drained, dph, failed));
+      dph ^= 1u;
 #pragma unroll 1
-      for (int ch = 0; ch < nchunks && ok; ++ch, ++kc) {
-        const uint32_t s = kc % kXStages;
-        ok = mbar_wait(&sh->full[s], (kc / kXStages) & 1u, failed);
+      for (int ch = 0; ch < nchunks && ok; ++ch) {
+        ok = __all_sync(0xffffffffu, mbar_wait(&sh->full[s], ph, failed));
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint64_t bd = smem_desc(smem_u32(base + (ch >> 2) * nb * 128)) + 2 * (ch & 3);
-        const uint32_t ta = tmem + (uint32_t)kXStageCol + 32u * s;
+        const uint64_t bd = bd0 + (uint64_t)((uint32_t)(ch >> 2) * (uint32_t)(8 * nb) + 2u * (uint32_t)(ch & 3));
+        const uint32_t ta = d + (uint32_t)kXStageCol + 32u * s;
+        if (lead) {
 #pragma unroll
-        for (int p = 0; p < 4; ++p)
-          mma_f4_ts(tmem, ta + 8 * p, bd, idesc, tmem + kXSfA + 16 * p, tmem + kXSfB, (ch > 0 || p > 0) ? 1u : 0u);
-        mma_commit(&sh->empty[s]);
+          for (int p = 0; p < 4; ++p)
+            mma_f4_ts(d, ta + 8 * p, bd, idesc, d + kXSfA + 16 * p, d + kXSfB, (ch > 0 || p > 0) ? 1u : 0u);
+          mma_commit(&sh->empty[s]);
+        }
+        if (++s == kXStages) {
+          s = 0;
+          ph ^= 1u;
+        }
       }
-      if (ok) mma_commit(&sh->done);
+      if (ok && lead) mma_commit(&sh->done);
+      __syncwarp();
     }
   } else if (warp >= kXEpi0) {
     // ---------------- epilogue ----------------
@@ -403,16 +429,7 @@ __global__ void __launch_bounds__(kXTcThreads, 1)
       if (!__all_sync(0xffffffffu, mbar_wait(&sh->done, tile & 1u, failed))) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       uint32_t word[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-      for (int cb = 0; cb < 4; ++cb) {
-        if (cb >= words) break;
-        uint32_t v[32];
-        tmem_load32(v, tmem + ((uint32_t)(32 * sub) << 16) + (uint32_t)(32 * (half * words + cb)));
-        uint32_t acc = 0u;   // sign bits (0 for z = 0), column 0 first
-#pragma unroll
-        for (int j = 0; j < 32; ++j) acc = __funnelshift_l(v[j], acc, 1);
-        word[cb] = ~__brev(acc);
-      }
+      sign_words<4>(word, tmem + ((uint32_t)(32 * sub) << 16) + (uint32_t)(32 * half * words), words, 0.0f);
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(&sh->drained);

@@ -134,12 +134,8 @@ __device__ __forceinline__ uint32_t peer_addr(uint32_t local_addr, uint32_t rank
 // 16 accumulator columns of this warp's 32 lanes, as integers (exact).
 __device__ __forceinline__ void load_cols16(int (&z)[16], uint32_t taddr) {
   uint32_t v[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  tmem_load16(v, taddr);
+  tmem_wait_ld(v);
 #pragma unroll
   for (int j = 0; j < 16; ++j) z[j] = __float2int_rn(__uint_as_float(v[j]));
 }
@@ -310,28 +306,33 @@ __device__ __forceinline__ void run_tile(TileIn T, const Place& pl, int pat, boo
       __syncwarp();
       if (lane == 0) mbar_arrive(&sh->full[s]);
     }
-  } else if (lane == 0) {
+  } else {
     // ---------------- MMA issuer ----------------
-    const uint32_t idesc = idesc_f4(TN, 16 * nblk);
-    int s = 0;
-    uint32_t par = 0;
+    const bool lead = elect_one();
+    const uint32_t idesc = uniform(idesc_f4(TN, 16 * nblk));
+    const uint32_t d = uniform(tmem);
+    const uint64_t bd0 = smem_desc(uniform(smem_u32(stages)));
+    uint32_t s = 0, par = 0;
+    bool ok = true;
 #pragma unroll 1
-    for (int ks = ks0; ks < ks1; ++ks) {
-      if (!mbar_wait(&sh->full[s], par, failed)) break;
+    for (int ks = ks0; ks < ks1 && ok; ++ks) {
+      ok = __all_sync(kFull, mbar_wait(&sh->full[s], par, failed));
+      if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint64_t bd = smem_desc(smem_u32(stages + s * B_BYTES));
-      const uint32_t ta = tmem + (uint32_t)(kStageCol + 32 * s);
+      const uint64_t bd = bd0 + (uint64_t)(s * (uint32_t)(B_BYTES >> 4));
+      const uint32_t ta = d + (uint32_t)kStageCol + 32u * s;
+      if (lead) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e)   // K = 64 per MMA: 8 TMEM columns, 32 bytes of the stage rows
-        mma_f4_ts(tmem, ta + 8 * e, bd + 2 * e, idesc, tmem + kSfCol, tmem + kSfCol + 8,
-                  (ks > ks0 || e > 0) ? 1u : 0u);
-      mma_commit(&sh->empty[s]);
+        for (int e = 0; e < 4; ++e)   // K = 64 per MMA: 8 TMEM columns, 32 bytes of the stage rows
+          mma_f4_ts(d, ta + 8 * e, bd + 2 * e, idesc, d + kSfCol, d + kSfCol + 8, (ks > ks0 || e > 0) ? 1u : 0u);
+        mma_commit(&sh->empty[s]);
+      }
       if (++s == kStages) {
         s = 0;
         par ^= 1u;
       }
     }
-    if (np > 0 && !*failed) mma_commit(&sh->done);
+    if (np > 0 && ok && lead) mma_commit(&sh->done);
   }
   __syncwarp();
 

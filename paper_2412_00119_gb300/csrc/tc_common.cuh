@@ -52,6 +52,18 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t pari
   }
 }
 
+// One lane of the calling (converged) warp.  MMAs are issued by a whole warp with
+// this lane elected around the instruction alone: the operands are then computed
+// in uniform registers, where the instruction takes them from (under `lane == 0`
+// every operand is moved there one by one, 90 clocks per MMA).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+  return p != 0u;
+}
+// A value that is the same in every lane, into a uniform register.
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __reduce_max_sync(kFull, v); }
+
 // Shared-memory matrix descriptor: K-major, SWIZZLE_128B, 8-row groups 1024 B apart.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
   uint64_t d = 0;
@@ -197,18 +209,46 @@ __device__ __forceinline__ void tmem_store_row256(uint32_t taddr, const uint32_t
   }
 }
 
-// 32 TMEM columns of this warp's 32 lanes, waited for.
-__device__ __forceinline__ void tmem_load32(uint32_t (&v)[32], uint32_t taddr) {
+// 16 TMEM columns of this warp's 32 lanes; tmem_wait_ld before they are used.
+__device__ __forceinline__ void tmem_load16(uint32_t (&v)[16], uint32_t taddr) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-        "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-        "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]),
-        "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]),
-        "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
       : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+// v: loaded values that may be used after it.
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                 "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])
+               :: "memory");
+}
+
+// Sign words of 32 kWords accumulator columns from taddr on, for this lane's row:
+// bit j of word w is 1 where column 32 w + j minus npad is >= 0.  Each 16 columns
+// are in flight while the 16 before are shifted into their word.
+template <int kWords>
+__device__ __forceinline__ void sign_words(uint32_t (&word)[kWords], uint32_t taddr, int words, float npad) {
+  uint32_t v[2][16];
+  tmem_load16(v[0], taddr);
+  tmem_wait_ld(v[0]);
+#pragma unroll
+  for (int h = 0; h < 2 * kWords; ++h) {
+    if (h >= 2 * words) break;
+    if (h + 1 < 2 * words) tmem_load16(v[(h + 1) & 1], taddr + 16u * (uint32_t)(h + 1));
+    uint32_t acc = (h & 1) ? word[h >> 1] : 0u;   // column 0 first; its sign ends in bit 31
+    if (npad == 0.0f) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) acc = __funnelshift_l(v[h & 1][j], acc, 1);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+        acc = __funnelshift_l(__float_as_uint(__uint_as_float(v[h & 1][j]) - npad), acc, 1);
+    }
+    word[h >> 1] = (h & 1) ? ~__brev(acc) : acc;
+    if (h + 1 < 2 * words) tmem_wait_ld(v[(h + 1) & 1]);
+  }
 }
 
 }  // namespace tc
