@@ -343,7 +343,6 @@ int run_steps(bmlp_t* h, const uint64_t* xd, const int32_t* yd, int64_t n, cudaS
   const size_t head = offsetof(StepParams, x);
   CK(h, cudaMemcpyAsync(reinterpret_cast<char*>(h->dP) + head, reinterpret_cast<char*>(&h->hp) + head,
                         sizeof(StepParams) - head, cudaMemcpyHostToDevice, st));
-  CK(h, cudaMemsetAsync(&h->dCtrl->s, 0, sizeof(uint32_t), st));
   const int64_t steps = (n + h->bs - 1) / h->bs;
   if (h->profEvery != 1) {
     int rc = ensure_graph(h);

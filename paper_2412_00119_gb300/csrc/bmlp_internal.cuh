@@ -74,7 +74,6 @@ struct Ctrl {
   unsigned long long t;         // global mini-batch counter since creation
   unsigned long long err;       // last-layer 01-loss count since the last epoch end
   unsigned long long bad_labels;// labels outside 0..c-1 seen by the kernels
-  uint32_t s;                   // mini-batch index within the current train call
   uint32_t s_cur;               // the mini-batch in progress
   unsigned long long t_cur;
   uint32_t timeouts;            // bounded device waits that expired (BMLP_ETIMEOUT)
@@ -83,14 +82,6 @@ struct Ctrl {
   UpdStat stat[kStatSlots];
   unsigned long long layer_err[BMLP_MAX_LAYERS];  // local 01-loss count of each layer
 };
-
-// One thread of the first layer's forward pass, after its wait.
-__device__ __forceinline__ void begin_step(Ctrl* c, int L) {
-  c->s_cur = c->s;
-  c->t_cur = c->t;
-  c->upd_next = 0u;
-  for (int i = 0; i < L; ++i) c->any_mark[i] = 0u;
-}
 
 // Thresholds of the reinforcement sampler of one layer (Alg. 3 l.5-12): the
 // events of a neuron row are drawn per block of 64 inputs (the last block
@@ -111,6 +102,8 @@ struct StepParams {
   const uint64_t* x;            // packed inputs of the current train call
   const int32_t* y;             // labels of the current train call
   int64_t n;                    // patterns in the current train call
+  uint32_t s;                   // mini-batch index within the current train call (the update kernel
+                                // advances it; one copy to the device sets it with x, y and n)
   const RTables* rt;            // [L] reinforcement sampler thresholds
   int32_t nblk_max;             // max over layers of ceil(K_in / 64)
   Ctrl* ctrl;
@@ -157,6 +150,18 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 ctr, uint32_t k0, uint32_t 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// The mini-batch index (past the L1 cache: kernels that overlap this one write it).
+__device__ __forceinline__ uint32_t batch_index(const StepParams* P) { return __ldcg(&P->s); }
+
+// One thread of the first layer's forward pass, after its wait.
+__device__ __forceinline__ void begin_step(const StepParams* P) {
+  Ctrl* c = P->ctrl;
+  c->s_cur = batch_index(P);
+  c->t_cur = c->t;
+  c->upd_next = 0u;
+  for (int i = 0; i < P->L; ++i) c->any_mark[i] = 0u;
 }
 
 // Launch with or without the programmatic-stream-serialization attribute.
@@ -291,7 +296,7 @@ struct UpdLayer {
 };
 struct UpdArgs {
   UpdLayer layer[BMLP_MAX_LAYERS];
-  const StepParams* P;
+  StepParams* P;
   Ctrl* ctrl;
   const RTables* rt;
   int32_t L, bs, nw0, h_max;
@@ -307,7 +312,7 @@ cudaError_t launch_update_rows(int nplanes, unsigned grid, cudaStream_t st, bool
 // from DevLayer::EV.
 cudaError_t prepare_update_ws();
 cudaError_t launch_update_ws(int nplanes, int h_max, int bs, unsigned grid, cudaStream_t st, bool pdl,
-                             const StepParams* P);
+                             StepParams* P);
 // Attributes of the update kernel: fails when the library holds no sm_103a image.
 cudaError_t update_kernel_image(cudaFuncAttributes* fa);
 // Peak-rate kernel of one contraction engine (BMLP_FWD_*): launches it on

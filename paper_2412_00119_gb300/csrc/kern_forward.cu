@@ -139,8 +139,8 @@ dim3 eval_forward_block() { return dim3(NT); }
 __global__ void __launch_bounds__(NT) k_train_forward(const StepParams* __restrict__ P, int l) {
   __shared__ Stage st[2];
   const DevLayer& Ly = P->layer[l - 1];
-  if (l == 1 && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) begin_step(P->ctrl, P->L);
-  const int64_t start = (int64_t)P->ctrl->s * P->bs;
+  if (l == 1 && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) begin_step(P);
+  const int64_t start = (int64_t)batch_index(P) * P->bs;
   const int64_t rem = P->n - start;
   const int64_t bsz = rem < P->bs ? rem : P->bs;
   const uint64_t* A = (l == 1) ? P->x + start * P->nw0 : P->layer[l - 2].A;

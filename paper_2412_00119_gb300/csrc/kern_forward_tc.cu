@@ -22,7 +22,7 @@
 //   - the 256 producer threads copy a piece of the tile's 128 weight rows and of
 //     its pattern rows into shared memory with asynchronous copies of whole
 //     lines;
-//   - per k-step, weight warp q (of four) expands neuron rows 32 q .. + 31, a
+//   - two k-steps at a time (their latencies overlap), weight warp q (of four) expands neuron rows 32 q .. + 31, a
 //     lane per row, into 32 tensor-memory columns, and activation warp q expands
 //     pattern rows 32 q .. + 31 into a shared-memory stage, rows of 128 bytes
 //     with the 128B swizzle (16-byte chunk c of row r at chunk c ^ (r % 8));
@@ -37,10 +37,11 @@
 // The loops are kept rolled: a CTA runs through its code once or twice, and
 // with the k-steps of a piece unrolled the warps waited longer for instructions
 // (2.5 clocks per instruction issued) than for anything but memory.
-// Registers (<= 113), shared memory (103 KB) and tensor memory (256 columns)
-// are sized for two CTAs per SM: one expands while the other's MMAs run, and
-// the CTAs of the next layer, launched as programmatic dependents, set up
-// beside the running ones.
+// Shared memory (103 KB) and tensor memory (256 columns) are sized for two CTAs
+// per SM: one expands while the other's MMAs run, and the CTAs of the next layer,
+// launched as programmatic dependents, set up beside the running ones.  Registers
+// are held to 72, so that CTAs of the event draws and of the selection fit
+// beside two of these (a step of 8192-8192x4 154 us at 72, 156 at 96).
 //
 // What bounds it: latency, and L2 bandwidth for the widest layers.  At 100
 // patterns, launches back to back as programmatic dependents: 8192 -> 8192
@@ -264,8 +265,8 @@ __device__ __forceinline__ void run_tile(TileIn T, const Place& pl, int pat, boo
     const uint32_t srow = smem_u32(stages) + 128u * (uint32_t)r;
     bool ok = true;                              // (a failed wait leaves the loop's barriers matched)
 #pragma unroll 1
-    for (int ks = ks0; ks < ks1; ++ks) {
-      const int k = ks - ks0, s = k % kStages;
+    for (int ks = ks0; ks < ks1; ks += 2) {
+      const int k = ks - ks0;
       if (k % kSteps == 0) {
         if (k > 0) {
           producers_sync();                      // every warp has read the last piece
@@ -275,36 +276,56 @@ __device__ __forceinline__ void run_tile(TileIn T, const Place& pl, int pat, boo
         cp_async_wait_all();
         producers_sync();
       }
-      if (ok && k >= kStages)
-        ok = __all_sync(kFull, mbar_wait(&sh->empty[s], (uint32_t)((k / kStages - 1) & 1), failed));
+      const int s[2] = {k % kStages, (k + 1) % kStages};
+      const bool two = ks + 1 < ks1;
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        if (ok && k + i >= kStages && (i == 0 || two))
+          ok = __all_sync(kFull, mbar_wait(&sh->empty[s[i]], (uint32_t)(((k + i) / kStages - 1) & 1), failed));
       if (!ok) continue;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t src = brow + 32u * (uint32_t)(ks % kSteps);
-      const uint4 lo = lds128(src), hi = lds128(src + 16);
-      uint32_t x[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+      uint32_t x[2][8];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const uint4 lo = lds128(src + 32 * i), hi = lds128(src + 32 * i + 16);
+        x[i][0] = lo.x; x[i][1] = lo.y; x[i][2] = lo.z; x[i][3] = lo.w;
+        x[i][4] = hi.x; x[i][5] = hi.y; x[i][6] = hi.z; x[i][7] = hi.w;
+      }
       if (wwarp) {
         // rows past N hold whatever: their outputs are dropped (e2m1 has no NaN)
-        tmem_store_row256(tmem + lanes + (uint32_t)(kStageCol + 32 * s), x);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+          if (i == 0 || two) tmem_store_row256(tmem + lanes + (uint32_t)(kStageCol + 32 * s[i]), x[i]);
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       } else if (live) {
-        if (T.Kin - KF * ks < KF) {
+        const int valid = T.Kin - KF * ks;       // inputs from here on
+        if (valid < 2 * KF) {
           // pad bits, whatever the caller left in the rows' last word, count as +1
-          const int valid = T.Kin - KF * ks;
 #pragma unroll
-          for (int c = 0; c < 8; ++c)
-            x[c] &= valid >= 32 * c + 32 ? kFull : (valid <= 32 * c ? 0u : (1u << (valid - 32 * c)) - 1u);
+          for (int c = 0; c < 16; ++c)
+            x[c >> 3][c & 7] &= valid >= 32 * c + 32 ? kFull : (valid <= 32 * c ? 0u : (1u << (valid - 32 * c)) - 1u);
         }
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          uint32_t v[4];
-          e2m1_words(x[c], v);
-          sts128(srow + (uint32_t)(s * B_BYTES + 16 * (c ^ (r & 7))), v);
+        for (int i = 0; i < 2; ++i) {
+          const uint32_t row = (srow + (uint32_t)(s[i] * B_BYTES)) | (16u * (uint32_t)(r & 7));   // chunk c at row ^ 16 c
+          if (i == 0 || two) {
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+              uint32_t v[4];
+              e2m1_words(x[i][c], v);
+              sts128(row ^ (16u * c), v);
+            }
+          }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       }
       __syncwarp();
-      if (lane == 0) mbar_arrive(&sh->full[s]);
+      if (lane == 0) {
+        mbar_arrive(&sh->full[s[0]]);
+        if (two) mbar_arrive(&sh->full[s[1]]);
+      }
     }
   } else {
     // ---------------- MMA issuer ----------------
@@ -445,7 +466,7 @@ __device__ __forceinline__ void run_tile(TileIn T, const Place& pl, int pat, boo
 
 // One layer of the current training mini-batch.  Grid (S x neuron tiles,
 // pattern tiles of pat), clusters of S.
-__global__ void __launch_bounds__(THREADS, 2) k_train_forward_tc(const StepParams* __restrict__ P, int l,
+__global__ void __launch_bounds__(THREADS, 3) k_train_forward_tc(const StepParams* __restrict__ P, int l,
                                                                  int pat) {
   extern __shared__ uint8_t smem_raw[];
   const DevLayer& Ly = P->layer[l - 1];
@@ -461,11 +482,11 @@ __global__ void __launch_bounds__(THREADS, 2) k_train_forward_tc(const StepParam
   auto ready = [&](const uint64_t*& A, int64_t& M) {
     pdl_wait();
     pdl_trigger();
-    const int64_t start = (int64_t)P->ctrl->s * bs;
+    const int64_t start = (int64_t)batch_index(P) * bs;
     M = min((int64_t)bs, ncall - start);
     if (l == 1) {
       A = x + start * T.nw;
-      if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) begin_step(P->ctrl, P->L);
+      if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) begin_step(P);
     }
   };
   if (row_align(T.A, T.nw) == 16 && row_align(T.W, T.nw) == 16)

@@ -33,8 +33,8 @@ __device__ __forceinline__ int warp_sum(int v) {
 // waits before it lets the next kernel start, so a kernel two launches back
 // has always completed.
 // Bound: a chain of dependent L2 loads (batch index, label, rho) and two
-// barriers, so the model comes as a kernel parameter, z and rho are loaded
-// beside the classifier's words, and one warp finds the two largest scores
+// barriers, so the model comes as a kernel parameter, label, rho and classifier are
+// read before the wait and z beside the activations, and one warp finds the two largest scores
 // (with one thread walking over 100 classes the launch of 3072-4096x4 took 16.3 us,
 // now 12.3, 5 of them the two events around it).
 // ---------------------------------------------------------------------------
@@ -52,38 +52,59 @@ __device__ __forceinline__ uint16_t selection(uint32_t cand) {
   return cand == 0u ? kNoSel : (uint16_t)((key >> 1) | ((key & 1u) << 15));
 }
 
-__device__ __forceinline__ void cls_select_body(const ClsArgs& C, int li, int mu) {
+__device__ __forceinline__ void cls_select_body(const ClsArgs& C, int li, int mu, bool early) {
   const ClsLayer& Ly = C.layer[li];
   Ctrl* ctrl = C.ctrl;
   __shared__ int yh[BMLP_MAX_CLASSES];
   __shared__ int s_mark, s_timeout;
-  const int64_t start = (int64_t)ctrl->s * C.bs;
-  if (mu >= C.P->n - start) return;
+  const int64_t start = (int64_t)batch_index(C.P) * C.bs;
+  const bool in = mu < C.P->n - start;
   const int c = C.c;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  const int label = C.P->y[start + mu];
+  const int label = in ? C.P->y[start + mu] : 0;
   const int y = (label < 0 || label >= c) ? 0 : label;  // memory-safe stand-in; the host reports BMLP_EINVAL
-  // one read of the counter for the whole CTA (the last forward pass may be
-  // running beside an early CTA and could raise it meanwhile)
-  if (threadIdx.x == 0) s_timeout = ctrl->timeouts != 0u;
-  const int K = Ly.Kout, gamma = Ly.gamma;
+  const int K = Ly.Kout, gamma = Ly.gamma, nw = Ly.nw_out;
   const int16_t* z = Ly.Z + (int64_t)mu * K;
   const int8_t* rt = Ly.rhoT + (int64_t)y * K;
   // contiguous groups of 8, 16, .. 256 neurons: one thread per 8 neurons
   const int per = gamma >> 3;  // 8-neuron chunks per group
   const bool chunks = Ly.member == nullptr && (gamma & 7) == 0 && per <= 32 && (per & (per - 1)) == 0;
   const int nchunk = K >> 3;
-  uint4 zv = make_uint4(0, 0, 0, 0);
+  const bool mine = chunks && (int)threadIdx.x < nchunk;
+  // what no forward pass writes, before the wait: rho, and the classifier's
+  // words of this warp's first classes (rows of at most 32 words)
   uint2 rv = make_uint2(0, 0);
-  if (chunks && (int)threadIdx.x < nchunk) {
-    zv = *reinterpret_cast<const uint4*>(z + 8 * threadIdx.x);
-    rv = *reinterpret_cast<const uint2*>(rt + 8 * threadIdx.x);
+  if (mine) rv = *reinterpret_cast<const uint2*>(rt + 8 * threadIdx.x);
+  constexpr int kPre = 3;
+  uint64_t pre[kPre];
+#pragma unroll
+  for (int i = 0; i < kPre; ++i)
+    pre[i] = (warp + i * nwarps < c && lane < nw) ? Ly.PT[(int64_t)(warp + i * nwarps) * nw + lane] : 0ull;
+  if (!early) {
+    pdl_wait();
+    pdl_trigger();
   }
-  const uint64_t* a = Ly.A + (int64_t)mu * Ly.nw_out;
-  for (int j = warp; j < c; j += nwarps) {
-    const uint64_t* pt = Ly.PT + (int64_t)j * Ly.nw_out;
+  if (!in) return;
+  // one read of the counter for the whole CTA (the last forward pass may be
+  // running beside an early CTA and could raise it meanwhile)
+  if (threadIdx.x == 0) s_timeout = ctrl->timeouts != 0u;
+  uint4 zv = make_uint4(0, 0, 0, 0);
+  if (mine) zv = *reinterpret_cast<const uint4*>(z + 8 * threadIdx.x);
+  const uint64_t* a = Ly.A + (int64_t)mu * nw;
+  const uint64_t a0 = lane < nw ? a[lane] : 0ull;
+#pragma unroll
+  for (int i = 0; i < kPre; ++i) {
+    const int j = warp + i * nwarps;
+    if (j >= c) break;
+    int cnt = __popcll(a0 ^ pre[i]);
+    for (int w = lane + 32; w < nw; w += 32) cnt += __popcll(a[w] ^ Ly.PT[(int64_t)j * nw + w]);
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0) yh[j] = K - 2 * cnt;
+  }
+  for (int j = warp + kPre * nwarps; j < c; j += nwarps) {
+    const uint64_t* pt = Ly.PT + (int64_t)j * nw;
     int cnt = 0;
-    for (int w = lane; w < Ly.nw_out; w += 32) cnt += __popcll(a[w] ^ pt[w]);
+    for (int w = lane; w < nw; w += 32) cnt += __popcll(a[w] ^ pt[w]);
     cnt = __reduce_add_sync(0xffffffffu, cnt);
     if (lane == 0) yh[j] = K - 2 * cnt;
   }
@@ -165,15 +186,11 @@ __device__ __forceinline__ void cls_select_body(const ClsArgs& C, int li, int mu
   }
 }
 
-__global__ void __launch_bounds__(512) k_cls_select(const __grid_constant__ ClsArgs C) {
+__global__ void __launch_bounds__(512, 3) k_cls_select(const __grid_constant__ ClsArgs C) {
   const int li = blockIdx.y;
   const int mu = blockIdx.x;
   const bool early = C.early && li < C.L - 1;
-  if (!early) {
-    pdl_wait();
-    pdl_trigger();
-  }
-  cls_select_body(C, li, mu);
+  cls_select_body(C, li, mu, early);
   if (early) {
     pdl_wait();
     pdl_trigger();
@@ -209,7 +226,7 @@ __global__ void __launch_bounds__(kEvThreads) k_r_events(const StepParams* __res
   int li = 0;
   while (li + 1 < P->L && bid >= P->layer[li + 1].ev_cta_base) ++li;
   const DevLayer& Ly = P->layer[li];
-  load_tables(s_rt, P->rt[li]);
+  load_tables<kEvThreads>(s_rt, P->rt[li]);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int k = (bid - Ly.ev_cta_base) * kEvRowsPerCta + warp;

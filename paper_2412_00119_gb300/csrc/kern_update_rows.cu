@@ -19,8 +19,8 @@
 // the reinforcement sampler), a warp 32 consecutive blocks of a row, or the
 // blocks of several rows where rows are shorter; nothing is shared between
 // warps.  Before it waits for the selection kernel a warp draws its blocks'
-// reinforcement events (they depend on the step counter only) and loads its
-// planes; then it reads its rows' selections (DevLayer::sel of the row's
+// reinforcement events (they depend on the step counter only), loads its planes
+// and finds its mini-batch; then it reads its rows' selections (DevLayer::sel of the row's
 // group: the patterns whose entry is the row are its tuples), applies the
 // tuples in ascending mu, then the events, and writes planes and W.  A row
 // without tuple is written only where it has an event.  Layers with an empty
@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(kThreads) k_update_rows(const __grid_constant_
   const int n_in = Ly.Kin - 64 * b;                      // inputs of the block, 64 at most
   const bool live = k < Ly.Kout && n_in > 0;
   if (threadIdx.x == 0) stat[0] = stat[1] = 0ull;
-  load_tables(tab, U.rt[li]);
+  load_tables<kThreads>(tab, U.rt[li]);
   __syncthreads();
   // ---- before the wait: the block's events and planes ----
   uint64_t ev = 0ull;
@@ -82,23 +82,23 @@ __global__ void __launch_bounds__(kThreads) k_update_rows(const __grid_constant_
     load_planes<kP>(u[0], hrow);
     if (two) load_planes<kP>(u[1], hrow + kP);
   }
-  pdl_wait();
-  pdl_trigger();
   const uint32_t sidx = ctrl->s_cur;
   const int bs = U.bs;
   const int64_t start = (int64_t)sidx * bs;
   const int64_t rem = U.P->n - start;
   const int bsz = (int)(rem < bs ? rem : bs);
+  const uint64_t* a0 = li == 0 ? U.P->x + start * U.nw0 : Ly.aprev;
+  pdl_wait();
+  pdl_trigger();
+  const int gk = live ? (Ly.group_of ? (int)Ly.group_of[k] : k / Ly.gamma) : 0;
   // an expired bounded wait in this step's forward pass: no CP, no R (the
   // selection kernel marked nothing either); the counters still advance
   const bool skip = ctrl->timeouts != 0u || ctrl->any_mark[li] == 0u;
-  const uint64_t* a0 = li == 0 ? U.P->x + start * U.nw0 : Ly.aprev;
   const Sliced<kP, kOnes> S(U.h_max);
   bool hit_any = false;
   if (!skip) {
     const uint64_t* acol = a0 + b;
     const int nwa = Ly.nw_in;
-    const int gk = live ? (Ly.group_of ? (int)Ly.group_of[k] : k / Ly.gamma) : 0;
 #pragma unroll 1
     for (int m0 = 0; m0 < bsz; m0 += 128) {
       // tuples of this lane's row among patterns m0 .. m0 + 127: bit i of word q
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kThreads) k_update_rows(const __grid_constant_
     if (stat[1]) atomicAdd(&o.bytes, stat[1]);
     if (blockIdx.x == 0) {
       // the next step's counters (this kernel reads only the copies)
-      ctrl->s = sidx + 1;
+      U.P->s = sidx + 1;
       ctrl->t = ctrl->t_cur + 1;
     }
   }

@@ -416,7 +416,7 @@ __device__ __forceinline__ void ws_consumer(const StepParams* __restrict__ P, Ws
 }
 
 template <int kP, bool kOnes>
-__global__ void __launch_bounds__(kThreads, 1) k_update_ws(const StepParams* __restrict__ P) {
+__global__ void __launch_bounds__(kThreads, 1) k_update_ws(StepParams* P) {
   const Ring R = ring_of<kP>(P->bs);
   const int nslots = R.nslots;
   extern __shared__ uint8_t ws_raw[];
@@ -476,7 +476,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_ws(const StepParams* __r
     if (sh->failed) atomicAdd(&ctrl->timeouts, 1u);
     if (blockIdx.x == 0) {
       // the next step's counters (this kernel reads only the copies)
-      ctrl->s = sidx + 1;
+      P->s = sidx + 1;
       ctrl->t = ctrl->t_cur + 1;
     }
   }
@@ -489,7 +489,7 @@ cudaError_t set_smem() {
 }
 
 template <int kP, bool kOnes>
-cudaError_t launch_one(unsigned grid, size_t smem, cudaStream_t st, bool pdl, const StepParams* P) {
+cudaError_t launch_one(unsigned grid, size_t smem, cudaStream_t st, bool pdl, StepParams* P) {
   return launch_kernel(k_update_ws<kP, kOnes>, dim3(grid), dim3(kThreads), smem, st, pdl, P);
 }
 
@@ -516,7 +516,7 @@ cudaError_t prepare_update_ws() {
 }
 
 cudaError_t launch_update_ws(int nplanes, int h_max, int bs, unsigned grid, cudaStream_t st, bool pdl,
-                             const StepParams* P) {
+                             StepParams* P) {
   const bool ones = h_max == (1 << nplanes) - 1;
   const size_t smem = update_ws_smem(nplanes, bs);
   switch (nplanes) {

@@ -135,17 +135,19 @@ struct Tables {
   float inv;        // 1 / log2(1 - q)
 };
 
-// All threads of a CTA of at least kTableThreads.
-constexpr int kTableThreads = 195;
+// By all kThreads threads of a CTA.
+template <int kThreads>
 __device__ __forceinline__ void load_tables(Tables& tab, const RTables& R) {
-  const int i = threadIdx.x;
-  if (i < 128) tab.first[i >> 6][i & 63] = (uint32_t)(R.first[i >> 6][i & 63] - 1ull);
-  else if (i < 192) tab.gap[i - 128] = (uint32_t)(R.gap[i - 128] - 1ull);
-  else if (i < 194) {
-    tab.any[i - 192] = R.any[i - 192];
-    tab.scale[i - 192] = (float)R.any[i - 192] * 2.3283064365386963e-10f;
-  } else if (i == 194) {
-    tab.inv = 1.0f / __log2f(1.0f - (float)R.gap[0] * 2.3283064365386963e-10f);
+#pragma unroll
+  for (int i = threadIdx.x; i < 195; i += kThreads) {
+    if (i < 128) tab.first[i >> 6][i & 63] = (uint32_t)(R.first[i >> 6][i & 63] - 1ull);
+    else if (i < 192) tab.gap[i - 128] = (uint32_t)(R.gap[i - 128] - 1ull);
+    else if (i < 194) {
+      tab.any[i - 192] = R.any[i - 192];
+      tab.scale[i - 192] = (float)R.any[i - 192] * 2.3283064365386963e-10f;
+    } else {
+      tab.inv = 1.0f / __log2f(1.0f - (float)R.gap[0] * 2.3283064365386963e-10f);
+    }
   }
 }
 
