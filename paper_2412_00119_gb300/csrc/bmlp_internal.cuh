@@ -217,8 +217,8 @@ cudaError_t launch_group_order(int L, int max_K, bool redraw, cudaStream_t st, b
 // Reinforcement events of every neuron row of every layer for the current
 // step into DevLayer::EV (Alg. 3 l.5-12).
 void launch_r_events(unsigned grid, cudaStream_t st, const StepParams* P, uint32_t key0, uint32_t key1);
-constexpr int kEvRowsPerCta = 8;   // one warp per row
-constexpr int kEvThreads = 32 * kEvRowsPerCta;
+constexpr int kEvThreads = 128, kEvRowsPerWarp = 4;
+constexpr int kEvRowsPerCta = kEvThreads / 32 * kEvRowsPerWarp;
 // Generic forward for evaluation: A (M x nw_in) against W -> Aout (M x nw_out).
 __global__ void k_forward_eval(const uint64_t* __restrict__ A, int64_t M, int nw_in,
                                const uint64_t* __restrict__ W, int N, int Kin,

@@ -211,70 +211,66 @@ using namespace upd;
 
 }  // namespace
 
-// Reinforcement events of the current step (Alg. 3 l.5-12): warp per neuron
-// row; lane j draws the block draws of blocks 4j .. 4j+3 (one Philox call), the
-// blocks that hold an event are compacted into a per-warp list, and the lanes
-// share that list for the event draws (binary searches in the layer's
-// threshold tables, staged in shared memory); the row's bitmap goes to
-// DevLayer::EV.  It depends only on (seed, layer, neuron, step, p_r), so it
-// runs beside the forward passes.
+// Reinforcement events of the current step (Alg. 3 l.5-12): a warp takes
+// kEvRowsPerWarp neuron rows; lane j draws the block draws of blocks 4j .. 4j+3 of
+// each (one Philox call), the blocks that hold an event are listed per warp, and
+// the lanes share that list for the event draws; the rows' bitmaps go to
+// DevLayer::EV, zeros first.  It depends only on (seed, layer, neuron, step, p_r),
+// so it runs beside the forward passes.  Bound: instruction issue.  A list of
+// several rows leaves fewer lanes idle in its last round than one of a row (32
+// candidates of 128 blocks at 8192 inputs): 24.3 us for the four
+// layers of 8192 alone, 28.6 with a list per row, 31 with a CTA of eight rows.
 __global__ void __launch_bounds__(kEvThreads) k_r_events(const StepParams* __restrict__ P,
                                                          uint32_t key0, uint32_t key1) {
+  constexpr int kW = kEvThreads / 32;
   __shared__ Tables s_rt;
-  __shared__ uint16_t s_cand[kEvRowsPerCta][128];  // blocks with an event, per warp
+  __shared__ uint16_t s_cand[kW][128 * kEvRowsPerWarp];   // row * 128 + block
   const int bid = blockIdx.x;
   int li = 0;
   while (li + 1 < P->L && bid >= P->layer[li + 1].ev_cta_base) ++li;
   const DevLayer& Ly = P->layer[li];
   load_tables<kEvThreads>(s_rt, P->rt[li]);
-  __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int k = (bid - Ly.ev_cta_base) * kEvRowsPerCta + warp;
-  if (k >= Ly.Kout) return;
   const uint32_t l = (uint32_t)li + 1u;
   const uint32_t tt = (uint32_t)P->ctrl->t_cur;
-  const int Kin = Ly.Kin, nblk = Ly.nblk;
-  uint64_t* ev = Ly.EV + (int64_t)k * Ly.ev_stride;
+  const int Kin = Ly.Kin, nblk = Ly.nblk, stride = Ly.ev_stride;
   uint16_t* cand = s_cand[warp];
-  // rounds of 32 block groups (128 blocks): the block draws, one Philox call per
-  // lane; the blocks that hold an event are compacted into a list that the
-  // lanes then share, one block each, for the event draws
+  const int k0 = (bid - Ly.ev_cta_base) * kEvRowsPerCta + warp * kEvRowsPerWarp;
+  const int rows = min(kEvRowsPerWarp, Ly.Kout - k0);
+  uint64_t* ev0 = Ly.EV + (int64_t)k0 * stride;
+  const uint32_t below = (1u << lane) - 1u;
+  __syncthreads();
+  // rounds of 128 blocks
 #pragma unroll 1
-  for (int g0 = 0; 4 * g0 < nblk; g0 += 32) {
+  for (int g0 = 0; 4 * g0 < nblk && rows > 0; g0 += 32) {
     const int gq = g0 + lane;
-    uint32_t cmask = 0;
-    if (4 * gq < nblk) {
-      const uint4 u = philox4x32_10(make_uint4((uint32_t)gq, (uint32_t)k, (3u << 16) + l, tt), key0,
-                                    key1);
+    int total = 0;
+#pragma unroll 1
+    for (int r = 0; r < rows; ++r) {
+      uint4 u = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+      if (4 * gq < nblk) {
+        u = philox4x32_10(make_uint4((uint32_t)gq, (uint32_t)(k0 + r), (3u << 16) + l, tt), key0, key1);
+        // rows are 16-byte aligned and stride is even
+        uint4* z = reinterpret_cast<uint4*>(ev0 + (int64_t)r * stride + 4 * gq);
+        z[0] = make_uint4(0, 0, 0, 0);
+        if (4 * gq + 2 < stride) z[1] = make_uint4(0, 0, 0, 0);
+      }
 #pragma unroll
       for (int wq = 0; wq < 4; ++wq) {
         const int b = 4 * gq + wq;
-        if (b < nblk) {
-          const int x = (Kin - 64 * b >= 64) ? 0 : 1;
-          if ((unsigned long long)word_of(u, wq) < s_rt.any[x]) cmask |= 1u << wq;
-          else ev[b] = 0ull;
-        }
+        const bool in = b < nblk && (unsigned long long)word_of(u, wq) < s_rt.any[(Kin - 64 * b >= 64) ? 0 : 1];
+        const uint32_t bal = __ballot_sync(kFull, in);
+        if (in) cand[total + __popc(bal & below)] = (uint16_t)(128 * r + 4 * lane + wq);
+        total += __popc(bal);
       }
     }
-    // exclusive prefix of the candidate counts over the lanes
-    const int cnt = __popc(cmask);
-    int incl = cnt;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int v = __shfl_up_sync(kFull, incl, off);
-      if (lane >= off) incl += v;
-    }
-    const int total = __shfl_sync(kFull, incl, 31);
-    int pos = incl - cnt;
-#pragma unroll
-    for (int wq = 0; wq < 4; ++wq)
-      if ((cmask >> wq) & 1u) cand[pos++] = (uint16_t)(4 * gq + wq);
-    __syncwarp();
+    __syncwarp();   // the list and the zeros
 #pragma unroll 1
     for (int i = lane; i < total; i += 32) {
-      const int b = cand[i];
+      const int c = cand[i], b = 4 * g0 + (c & 127), r = c >> 7;
       const int n = min(64, Kin - 64 * b);
-      ev[b] = block_events(s_rt, (n == 64) ? 0 : 1, n, (uint32_t)b, (uint32_t)k, l, tt, key0, key1);
+      ev0[(int64_t)r * stride + b] = block_events(s_rt, (n == 64) ? 0 : 1, n, (uint32_t)b, (uint32_t)(k0 + r), l,
+                                                  tt, key0, key1);
     }
     __syncwarp();
   }
