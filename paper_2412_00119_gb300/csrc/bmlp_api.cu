@@ -395,18 +395,14 @@ int ensure_eval(bmlp_t* h, int64_t rows) {
 
 constexpr int64_t kEvalChunk = 65536;
 constexpr int64_t kStageRows = 65536;
-constexpr int64_t kTileRows = 512;
 
 // One layer of forward-only evaluation on the tensor-core engine.  pdl: the
-// launch before it in the stream is another call of this function whose
-// output it reads.
+// launch before it in the stream is another call of this function, or of
+// launch_predict_tile, on the same stream and handle.
 cudaError_t eval_layer_tc(bmlp_t* h, const DevLayer& D, const uint64_t* in, int64_t m, uint64_t* out,
                           cudaStream_t st, bool pdl) {
-  if (m <= kTileRows)
-    return launch_forward_tile(in, m, D.nw_in, D.W, D.Kout, D.Kin, out, D.nw_out, &h->dCtrl->timeouts, st,
-                               pdl);
-  launch_forward_eval_tc(in, m, D.nw_in, D.W, D.Kout, D.Kin, out, D.nw_out, &h->dCtrl->timeouts, st);
-  return cudaGetLastError();
+  return (forward_tiles_win(m, D.Kout, D.Kin) ? launch_forward_tile : launch_forward_eval_tc)(
+      in, m, D.nw_in, D.W, D.Kout, D.Kin, out, D.nw_out, &h->dCtrl->timeouts, st, pdl);
 }
 
 }  // namespace
@@ -765,7 +761,7 @@ int predict_impl(bmlp_t* h, const uint64_t* x, int64_t n, int32_t* out, void* cu
       prof_begin(h, kProfOut, st);
       if (h->tc && h->c <= kPredictTileClasses)
         CK(h, launch_predict_tile(in, m, D.nw_out, D.PT, h->c, D.Kout, o, &h->dCtrl->timeouts, st,
-                                  m <= kTileRows && !h->profiling));
+                                  !h->profiling));
       else
         k_predict_out<<<(unsigned)((m + 7) / 8), 256, 0, st>>>(in, m, D.nw_out, D.PT, h->c, D.Kout, o);
       prof_end(h, st);

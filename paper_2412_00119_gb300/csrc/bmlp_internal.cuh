@@ -248,6 +248,13 @@ cudaError_t launch_train_forward_tc(int bs, int Kout, int Kin, cudaStream_t st, 
 cudaError_t launch_forward_tile(const uint64_t* A, int64_t M, int nw_in, const uint64_t* W, int N, int Kin,
                                 uint64_t* Aout, int nw_out, unsigned int* timeouts, cudaStream_t st,
                                 bool pdl);
+// Whether these tiles or the pairs of launch_forward_eval_tc run an evaluation
+// layer faster.  One pattern tile always; else while the tiles fit the SMs once
+// and their 1,024-element pieces 1.6 times (tile against pair, us: 1000 -> 525 at
+// 2,000 / 4,096 patterns 5.9 / 7.2 and 7.7 / 7.3; 1024 -> 1024 at 2,000 / 4,096 5.8 /
+// 6.9 and 7.7 / 7.0; 3072 -> 2048 at 512 / 1,024 9.4 / 9.5 and 11.5 / 9.5; 4096 -> 4096
+// at 64 / 256 6.1 / 10.3 and 11.0 / 10.7).
+bool forward_tiles_win(int64_t M, int N, int Kin);
 // The evaluation output on the same tiles, for at most kPredictTileClasses
 // classes: labels[mu] = argmax_j of row mu of A against the c rows of PT (lowest
 // j on ties), K the width of the layer.
@@ -272,9 +279,9 @@ cudaError_t prepare_forward_eval_tc();
 // with arrive != 0; an expired wait adds one to *timeouts.
 void launch_wait_probe(unsigned int* timeouts, int arrive, unsigned long long limit_cycles,
                        cudaStream_t st);
-void launch_forward_eval_tc(const uint64_t* A, int64_t M, int nw_in, const uint64_t* W, int N,
+cudaError_t launch_forward_eval_tc(const uint64_t* A, int64_t M, int nw_in, const uint64_t* W, int N,
                             int Kin, uint64_t* Aout, int nw_out, unsigned int* timeouts,
-                            cudaStream_t st);
+                            cudaStream_t st, bool pdl);
 
 // One layer on the b1 mma.sync path (kern_forward_b1.cu): Aout (M x nw_out)
 // = packed sign(A W^T), sign(0) = +1, pad bits 0.

@@ -198,6 +198,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   pair_sync();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  // set up beside the tail of the layer before this one
+  pdl_wait();
+  pdl_trigger();
 
   if (warp < kProdWarps) {
     // ---------------- producers ----------------
@@ -427,19 +430,15 @@ cudaError_t prepare_forward_eval_tc() {
                               (int)kSmemBytes);
 }
 
-void launch_forward_eval_tc(const uint64_t* A, int64_t M, int nw_in, const uint64_t* W, int N, int Kin,
-                            uint64_t* Aout, int nw_out, unsigned int* timeouts, cudaStream_t st) {
+cudaError_t launch_forward_eval_tc(const uint64_t* A, int64_t M, int nw_in, const uint64_t* W, int N, int Kin,
+                                   uint64_t* Aout, int nw_out, unsigned int* timeouts, cudaStream_t st, bool pdl) {
   const int ntiles = (N + TN - 1) / TN;
   const int64_t tiles = (M + 2 * TM - 1) / (2 * TM) * ntiles;
   const int64_t pairs = sm_count() / 2 < tiles ? sm_count() / 2 : tiles;
   const bool wide = row_align(A, nw_in) == 16 && row_align(W, nw_in) == 16;
-  const unsigned grid = (unsigned)(2 * pairs);
-  if (wide)
-    k_forward_eval_tc<16><<<grid, THREADS, kSmemBytes, st>>>(A, M, nw_in, W, N, Kin, Aout, nw_out, ntiles, tiles,
-                                                             timeouts);
-  else
-    k_forward_eval_tc<8><<<grid, THREADS, kSmemBytes, st>>>(A, M, nw_in, W, N, Kin, Aout, nw_out, ntiles, tiles,
-                                                            timeouts);
+  return launch_kernel(wide ? k_forward_eval_tc<16> : k_forward_eval_tc<8>, dim3((unsigned)(2 * pairs)),
+                       dim3(THREADS), kSmemBytes, st, pdl, A, M, nw_in, W, N, Kin, Aout, nw_out, ntiles, tiles,
+                       timeouts);
 }
 
 }  // namespace bk

@@ -529,11 +529,13 @@ __global__ void __launch_bounds__(THREADS, 2)
 
 // Patterns per tile, pattern tiles and K split of M patterns on an N x Kin
 // layer.  The K range is split over up to kMaxSplit CTAs while every CTA keeps
-// a piece and all CTAs fit two per SM; then the patterns are dealt to more
-// tiles (of equal size, a multiple of 16) while all fit one per SM.  Measured at
-// 100 patterns, back to back: 8192 -> 8192 split 1 / 2 / 4 21.8 / 14.2 / 11.4 us;
-// 4096 -> 4096 split 2 / 4 7.7 / 6.1 us; 1024 -> 1024 (no split) pattern tiles of
-// 64 / 32 / 16 4.3 / 3.9 / 3.8 us.
+// a piece, all CTAs fit two per SM and the tiles alone fill at most half of the
+// SMs (3072-2048x3 at 512 patterns, 80 tiles: 717 us a call unsplit, 733 split);
+// then the patterns are dealt to more tiles (of equal size, a multiple of 16)
+// while all fit one per SM.  Measured at 100 patterns, back to back:
+// 8192 -> 8192 split 1 / 2 / 4 21.8 / 14.2 / 11.4 us; 4096 -> 4096 split 2 / 4
+// 7.7 / 6.1 us; 1024 -> 1024 (no split) pattern tiles of 64 / 32 / 16
+// 4.3 / 3.9 / 3.8 us.
 struct Shape {
   int pat, mtiles, ntiles, split;
 };
@@ -544,7 +546,7 @@ Shape shape_of(int64_t M, int N, int Kin, int sms) {
   const int npc = (Kin + KF * kSteps - 1) / (KF * kSteps);
   s.split = 1;
   for (int c = 2; c <= kMaxSplit; ++c)
-    if (npc >= c && s.ntiles * mt * c <= 2 * sms) s.split = c;
+    if (npc >= c && s.ntiles * mt * c <= 2 * sms && s.ntiles * mt * 2 <= sms) s.split = c;
   while (mt * s.ntiles * s.split * 2 <= sms && M > 16 * mt) mt *= 2;
   s.pat = (int)(((M + mt - 1) / mt + 15) / 16 * 16);
   s.mtiles = (int)((M + s.pat - 1) / s.pat);
@@ -599,6 +601,13 @@ cudaError_t launch_forward_tile(const uint64_t* A, int64_t M, int nw_in, const u
   const bool wide = row_align(A, nw_in) == 16 && row_align(W, nw_in) == 16;
   return launch_tiles(wide ? k_forward_tile<16> : k_forward_tile<8>, s, st, pdl, A, M, nw_in, W, N, Kin, Aout,
                       nw_out, timeouts, s.pat);
+}
+
+bool forward_tiles_win(int64_t M, int N, int Kin) {
+  if (M <= kMaxPat) return true;
+  const int64_t tiles = (M + kMaxPat - 1) / kMaxPat * ((N + TN - 1) / TN);
+  const int64_t npc = (Kin + KF * kSteps - 1) / (KF * kSteps);
+  return tiles <= sm_count() && 5 * tiles * npc <= 8 * sm_count();
 }
 
 cudaError_t launch_predict_tile(const uint64_t* A, int64_t M, int nw, const uint64_t* PT, int c, int K,
