@@ -396,13 +396,18 @@ int ensure_eval(bmlp_t* h, int64_t rows) {
 constexpr int64_t kEvalChunk = 65536;
 constexpr int64_t kStageRows = 65536;
 
-// One layer of forward-only evaluation on the tensor-core engine.  pdl: the
-// launch before it in the stream is another call of this function, or of
-// launch_predict_tile, on the same stream and handle.
+// One layer of forward-only evaluation on the tensor-core engine, as a
+// programmatic dependent of whatever runs before it in the stream (it reads and
+// writes nothing before that has completed, but for the weights with w_early:
+// the launch before it is another call of this function, or of
+// launch_predict_tile, for the same handle).
 cudaError_t eval_layer_tc(bmlp_t* h, const DevLayer& D, const uint64_t* in, int64_t m, uint64_t* out,
-                          cudaStream_t st, bool pdl) {
-  return (forward_tiles_win(m, D.Kout, D.Kin) ? launch_forward_tile : launch_forward_eval_tc)(
-      in, m, D.nw_in, D.W, D.Kout, D.Kin, out, D.nw_out, &h->dCtrl->timeouts, st, pdl);
+                          cudaStream_t st, bool w_early) {
+  const bool pdl = !h->profiling;
+  if (forward_tiles_win(m, D.Kout, D.Kin))
+    return launch_forward_tile(in, m, D.nw_in, D.W, D.Kout, D.Kin, out, D.nw_out, &h->dCtrl->timeouts, st, pdl,
+                               w_early);
+  return launch_forward_eval_tc(in, m, D.nw_in, D.W, D.Kout, D.Kin, out, D.nw_out, &h->dCtrl->timeouts, st, pdl);
 }
 
 }  // namespace
@@ -747,7 +752,7 @@ int predict_impl(bmlp_t* h, const uint64_t* x, int64_t n, int32_t* out, void* cu
       const DevLayer& D = h->hp.layer[l - 1];
       prof_begin(h, kProfEvalFwd, st);
       if (h->tc)
-        CK(h, eval_layer_tc(h, D, in, m, h->evA[cur], st, l > 1 && !h->profiling));
+        CK(h, eval_layer_tc(h, D, in, m, h->evA[cur], st, l > 1));
       else
         k_forward_eval<<<eval_forward_grid(m, D.Kout), eval_forward_block(), 0, st>>>(
             in, m, D.nw_in, D.W, D.Kout, D.Kin, h->evA[cur], D.nw_out);

@@ -244,10 +244,10 @@ cudaError_t launch_train_forward_tc(int bs, int Kout, int Kin, cudaStream_t st, 
                                     const StepParams* P, int l);
 // The same tiles for one layer of forward-only evaluation on a small batch: A
 // (M x nw_in) against W -> Aout (M x nw_out); an expired bounded wait adds one
-// to *timeouts.
+// to *timeouts.  w_early: with pdl, the launch before it does not write W.
 cudaError_t launch_forward_tile(const uint64_t* A, int64_t M, int nw_in, const uint64_t* W, int N, int Kin,
                                 uint64_t* Aout, int nw_out, unsigned int* timeouts, cudaStream_t st,
-                                bool pdl);
+                                bool pdl, bool w_early);
 // Whether these tiles or the pairs of launch_forward_eval_tc run an evaluation
 // layer faster.  One pattern tile always; else while the tiles fit the SMs once
 // and their 1,024-element pieces 1.6 times (tile against pair, us: 1000 -> 525 at

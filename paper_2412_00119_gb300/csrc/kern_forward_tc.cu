@@ -495,12 +495,13 @@ __global__ void __launch_bounds__(THREADS, 3) k_train_forward_tc(const StepParam
     run_tile<8>(T, place(smem_raw), pat, l > 1, ready, &P->ctrl->timeouts);
 }
 
-// One layer of forward-only evaluation on a small batch.
+// One layer of forward-only evaluation on a small batch.  w_early: no kernel that
+// may still run beside this one writes the weights.
 template <int kAlign>
 __global__ void __launch_bounds__(THREADS, 2)
     k_forward_tile(const uint64_t* __restrict__ A, int64_t M, int nw, const uint64_t* __restrict__ W, int N,
                    int Kin, uint64_t* __restrict__ Aout, int nw_out, unsigned int* __restrict__ timeouts,
-                   int pat) {
+                   int pat, bool w_early) {
   extern __shared__ uint8_t smem_raw[];
   const TileIn T{A, W, nw, N, Kin, nullptr, Aout, nw_out, nullptr};
   auto ready = [&](const uint64_t*&, int64_t& m) {
@@ -508,7 +509,7 @@ __global__ void __launch_bounds__(THREADS, 2)
     pdl_trigger();
     m = M;
   };
-  run_tile<kAlign>(T, place(smem_raw), pat, true, ready, timeouts);
+  run_tile<kAlign>(T, place(smem_raw), pat, w_early, ready, timeouts);
 }
 
 // Evaluation output on at most 128 classes: labels = argmax_j (A PT^T)_j, lowest j
@@ -596,11 +597,11 @@ cudaError_t launch_train_forward_tc(int bs, int Kout, int Kin, cudaStream_t st, 
 
 cudaError_t launch_forward_tile(const uint64_t* A, int64_t M, int nw_in, const uint64_t* W, int N, int Kin,
                                 uint64_t* Aout, int nw_out, unsigned int* timeouts, cudaStream_t st,
-                                bool pdl) {
+                                bool pdl, bool w_early) {
   const Shape s = shape_of(M, N, Kin, sm_count());
   const bool wide = row_align(A, nw_in) == 16 && row_align(W, nw_in) == 16;
   return launch_tiles(wide ? k_forward_tile<16> : k_forward_tile<8>, s, st, pdl, A, M, nw_in, W, N, Kin, Aout,
-                      nw_out, timeouts, s.pat);
+                      nw_out, timeouts, s.pat, w_early);
 }
 
 bool forward_tiles_win(int64_t M, int N, int Kin) {
