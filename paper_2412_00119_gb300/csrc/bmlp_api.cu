@@ -250,10 +250,18 @@ constexpr int kGraphSteps = 8;
 // (3072-2048x3) the ring alone, without the draws, 36.7 / 35.5.
 constexpr int64_t kRowsWeights = 20ll << 20;
 
-// One mini-batch step.  fork: the graph form (event draws on a branch,
-// programmatic dependent launches); chained: the step follows another step in
-// the same graph, so its first forward is a dependent of that step's update.
-int enqueue_step(bmlp_t* h, cudaStream_t st, bool fork, bool chained = false) {
+// One mini-batch step.  How it is launched:
+//   kStepPlain    kernel by kernel with full dependencies (sampled mini-batches);
+//   kStepDirect   kernel by kernel as programmatic dependents, with the call's
+//                 inputs as kernel parameters (a call of one mini-batch);
+//   kStepGraph    captured: programmatic dependents, the event draws of large
+//                 models on a branch;
+//   kStepChained  the same after another step of the graph, so that its first
+//                 forward pass is a dependent of that step's update.
+enum StepForm { kStepPlain, kStepDirect, kStepGraph, kStepChained };
+
+int enqueue_step(bmlp_t* h, cudaStream_t st, StepForm form, const OneBatch& one = OneBatch{}) {
+  const bool fork = form == kStepGraph || form == kStepChained, pdl = form != kStepPlain;
   for (int l = 1; l <= h->L; ++l) {
     if (fork && h->updRing && l == 2) {
       // the events are drawn on a branch beside the other layers' passes
@@ -264,20 +272,22 @@ int enqueue_step(bmlp_t* h, cudaStream_t st, bool fork, bool chained = false) {
     }
     prof_begin(h, kProfTrainFwd, st);
     if (h->tc)
-      CK(h, launch_train_forward_tc(h->bs, h->K[l], h->K[l - 1], st, fork && (l > 1 || chained), h->dP, l));
+      CK(h, launch_train_forward_tc(h->bs, h->K[l], h->K[l - 1], st, pdl && (l > 1 || form != kStepGraph), h->dP, l,
+                                    one));
     else
       k_train_forward<<<train_forward_grid(h->bs, h->K[l]), train_forward_block(), 0, st>>>(h->dP, l);
     prof_end(h, st);
   }
   if (h->group_mode == BMLP_GROUPS_RESHUFFLED) {
     // this step's partition (keyed by the step counter) before the selection
-    CK(h, launch_group_order(h->L, h->max_K, true, st, fork && h->tc, h->dP));
+    CK(h, launch_group_order(h->L, h->max_K, true, st, pdl && h->tc, h->dP));
   }
   prof_begin(h, kProfCls, st);
   // inside the step graph each kernel after the first is launched as a
   // programmatic dependent of the one before it (launch and prologue overlap
   // the previous kernel's tail); the event-draw branch joins with a full edge
-  CK(h, launch_cls_select(h->cls, h->max_K, st, fork && h->tc));
+  h->cls.one = one;
+  CK(h, launch_cls_select(h->cls, h->max_K, st, pdl && h->tc));
   prof_end(h, st);
   if (fork && h->updRing && h->L > 1) CK(h, cudaStreamWaitEvent(st, h->evJoin, 0));
   if (h->updRing && (!fork || h->L == 1)) {
@@ -287,9 +297,11 @@ int enqueue_step(bmlp_t* h, cudaStream_t st, bool fork, bool chained = false) {
   }
   prof_begin(h, kProfUpd, st);
   if (h->updRing)
-    CK(h, launch_update_ws(h->hp.nplanes, h->h_max, h->bs, (unsigned)sm_count(), st, fork, h->dP));
-  else
-    CK(h, launch_update_rows(h->hp.nplanes, h->updCtas, st, fork, h->upd));
+    CK(h, launch_update_ws(h->hp.nplanes, h->h_max, h->bs, (unsigned)sm_count(), st, pdl, h->dP, one));
+  else {
+    h->upd.one = one;
+    CK(h, launch_update_rows(h->hp.nplanes, h->updCtas, st, pdl, h->upd));
+  }
   prof_end(h, st);
   CK(h, cudaGetLastError());
   return BMLP_OK;
@@ -302,7 +314,7 @@ int capture_steps(bmlp_t* h, int steps, cudaGraphExec_t* exec) {
   const bool prof = h->profiling;
   h->profiling = false;
   int rc = BMLP_OK;
-  for (int i = 0; i < steps && rc == BMLP_OK; ++i) rc = enqueue_step(h, h->capStream, true, i > 0);
+  for (int i = 0; i < steps && rc == BMLP_OK; ++i) rc = enqueue_step(h, h->capStream, i > 0 ? kStepChained : kStepGraph);
   h->profiling = prof;
   cudaError_t e = cudaStreamEndCapture(h->capStream, &g);
   if (rc != BMLP_OK) {
@@ -337,13 +349,20 @@ int ensure_graph(bmlp_t* h) {
 
 // Train on n device-resident patterns.
 int run_steps(bmlp_t* h, const uint64_t* xd, const int32_t* yd, int64_t n, cudaStream_t st) {
+  const int64_t steps = (n + h->bs - 1) / h->bs;
+  h->launches += steps * (h->L + 2 + (h->updRing ? 1 : 0) + (h->group_mode == BMLP_GROUPS_RESHUFFLED ? 1 : 0));
+  if (steps == 1 && h->tc && h->profEvery == 0) {
+    // one mini-batch: launched directly, its inputs as kernel parameters
+    const int rc = enqueue_step(h, st, kStepDirect, OneBatch{xd, yd, n});
+    h->t_host += 1;
+    return rc;
+  }
   h->hp.x = xd;
   h->hp.y = yd;
   h->hp.n = n;
   const size_t head = offsetof(StepParams, x);
   CK(h, cudaMemcpyAsync(reinterpret_cast<char*>(h->dP) + head, reinterpret_cast<char*>(&h->hp) + head,
                         sizeof(StepParams) - head, cudaMemcpyHostToDevice, st));
-  const int64_t steps = (n + h->bs - 1) / h->bs;
   if (h->profEvery != 1) {
     int rc = ensure_graph(h);
     if (rc != BMLP_OK) return rc;
@@ -356,7 +375,7 @@ int run_steps(bmlp_t* h, const uint64_t* xd, const int32_t* yd, int64_t n, cudaS
     // the others as graphs of kGraphSteps steps, or of one step
     h->profiling = sampled(s);
     if (h->profiling) {
-      int rc = enqueue_step(h, st, false);
+      int rc = enqueue_step(h, st, kStepPlain);
       if (rc != BMLP_OK) return rc;
       ++s;
       continue;
@@ -367,7 +386,6 @@ int run_steps(bmlp_t* h, const uint64_t* xd, const int32_t* yd, int64_t n, cudaS
     s += multi ? kGraphSteps : 1;
   }
   h->profiling = h->profEvery > 0;
-  h->launches += steps * (h->L + 2 + (h->updRing ? 1 : 0) + (h->group_mode == BMLP_GROUPS_RESHUFFLED ? 1 : 0));
   h->t_host += steps;
   return BMLP_OK;
 }

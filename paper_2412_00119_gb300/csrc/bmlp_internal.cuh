@@ -152,6 +152,14 @@ __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// The inputs of a call of one mini-batch, passed to its kernels by value (no copy
+// to StepParams and no graph); x null: they are in StepParams.
+struct OneBatch {
+  const uint64_t* x;
+  const int32_t* y;
+  int64_t n;
+};
+
 // The mini-batch index (past the L1 cache: kernels that overlap this one write it).
 __device__ __forceinline__ uint32_t batch_index(const StepParams* P) { return __ldcg(&P->s); }
 
@@ -208,6 +216,7 @@ struct ClsArgs {
   Ctrl* ctrl;
   int32_t L, c, bs, r_num, r_den;
   int32_t early;   // the CTAs of the layers below the last work before they wait
+  OneBatch one;
 };
 cudaError_t launch_cls_select(const ClsArgs& C, int max_K, cudaStream_t st, bool pdl);
 // Group order of every layer with a random partition (DevLayer::member /
@@ -241,7 +250,7 @@ __global__ void k_repack_w(const uint32_t* H, uint64_t* W, int Kin, int Kout, in
 // bits.  pdl: launched with the programmatic-stream-serialization attribute.
 cudaError_t prepare_train_forward_tc();
 cudaError_t launch_train_forward_tc(int bs, int Kout, int Kin, cudaStream_t st, bool pdl,
-                                    const StepParams* P, int l);
+                                    const StepParams* P, int l, const OneBatch& one);
 // The same tiles for one layer of forward-only evaluation on a small batch: A
 // (M x nw_in) against W -> Aout (M x nw_out); an expired bounded wait adds one
 // to *timeouts.  w_early: with pdl, the launch before it does not write W.
@@ -308,6 +317,7 @@ struct UpdArgs {
   const RTables* rt;
   int32_t L, bs, nw0, h_max;
   uint32_t key0, key1;
+  OneBatch one;
 };
 // Sets lanes, upr and cta_base of a layer (Kin and Kout given); returns the first
 // CTA of the next one.
@@ -319,7 +329,7 @@ cudaError_t launch_update_rows(int nplanes, unsigned grid, cudaStream_t st, bool
 // from DevLayer::EV.
 cudaError_t prepare_update_ws();
 cudaError_t launch_update_ws(int nplanes, int h_max, int bs, unsigned grid, cudaStream_t st, bool pdl,
-                             StepParams* P);
+                             StepParams* P, const OneBatch& one);
 // Attributes of the update kernel: fails when the library holds no sm_103a image.
 cudaError_t update_kernel_image(cudaFuncAttributes* fa);
 // Peak-rate kernel of one contraction engine (BMLP_FWD_*): launches it on

@@ -467,12 +467,12 @@ __device__ __forceinline__ void run_tile(TileIn T, const Place& pl, int pat, boo
 // One layer of the current training mini-batch.  Grid (S x neuron tiles,
 // pattern tiles of pat), clusters of S.
 __global__ void __launch_bounds__(THREADS, 3) k_train_forward_tc(const StepParams* __restrict__ P, int l,
-                                                                 int pat) {
+                                                                 int pat, const OneBatch one) {
   extern __shared__ uint8_t smem_raw[];
   const DevLayer& Ly = P->layer[l - 1];
-  const uint64_t* x = l == 1 ? P->x : P->layer[l - 2].A;
+  const uint64_t* x = l > 1 ? P->layer[l - 2].A : (one.x ? one.x : P->x);
   const TileIn T{x, Ly.W, Ly.nw_in, Ly.Kout, Ly.Kin, Ly.Z, Ly.A, Ly.nw_out, nullptr};
-  const int64_t ncall = P->n;
+  const int64_t ncall = one.x ? one.n : P->n;
   const int bs = P->bs;
   // Layers >= 2: the weights (the previous step's update), the batch index
   // and every pointer were written two or more launches back, so the weights
@@ -482,7 +482,7 @@ __global__ void __launch_bounds__(THREADS, 3) k_train_forward_tc(const StepParam
   auto ready = [&](const uint64_t*& A, int64_t& M) {
     pdl_wait();
     pdl_trigger();
-    const int64_t start = (int64_t)batch_index(P) * bs;
+    const int64_t start = one.x ? 0 : (int64_t)batch_index(P) * bs;
     M = min((int64_t)bs, ncall - start);
     if (l == 1) {
       A = x + start * T.nw;
@@ -590,9 +590,9 @@ cudaError_t prepare_train_forward_tc() {
 }
 
 cudaError_t launch_train_forward_tc(int bs, int Kout, int Kin, cudaStream_t st, bool pdl,
-                                    const StepParams* P, int l) {
+                                    const StepParams* P, int l, const OneBatch& one) {
   const Shape s = shape_of(bs, Kout, Kin, sm_count());
-  return launch_tiles(k_train_forward_tc, s, st, pdl, P, l, s.pat);
+  return launch_tiles(k_train_forward_tc, s, st, pdl, P, l, s.pat, one);
 }
 
 cudaError_t launch_forward_tile(const uint64_t* A, int64_t M, int nw_in, const uint64_t* W, int N, int Kin,

@@ -57,11 +57,11 @@ __device__ __forceinline__ void cls_select_body(const ClsArgs& C, int li, int mu
   Ctrl* ctrl = C.ctrl;
   __shared__ int yh[BMLP_MAX_CLASSES];
   __shared__ int s_mark, s_timeout;
-  const int64_t start = (int64_t)batch_index(C.P) * C.bs;
-  const bool in = mu < C.P->n - start;
+  const int64_t start = C.one.x ? 0 : (int64_t)batch_index(C.P) * C.bs;
+  const bool in = mu < (C.one.x ? C.one.n : C.P->n) - start;
   const int c = C.c;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  const int label = in ? C.P->y[start + mu] : 0;
+  const int label = in ? (C.one.x ? C.one.y : C.P->y)[start + mu] : 0;
   const int y = (label < 0 || label >= c) ? 0 : label;  // memory-safe stand-in; the host reports BMLP_EINVAL
   const int K = Ly.Kout, gamma = Ly.gamma, nw = Ly.nw_out;
   const int16_t* z = Ly.Z + (int64_t)mu * K;

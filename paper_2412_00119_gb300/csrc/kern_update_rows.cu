@@ -84,10 +84,10 @@ __global__ void __launch_bounds__(kThreads) k_update_rows(const __grid_constant_
   }
   const uint32_t sidx = ctrl->s_cur;
   const int bs = U.bs;
-  const int64_t start = (int64_t)sidx * bs;
-  const int64_t rem = U.P->n - start;
+  const int64_t start = U.one.x ? 0 : (int64_t)sidx * bs;
+  const int64_t rem = (U.one.x ? U.one.n : U.P->n) - start;
   const int bsz = (int)(rem < bs ? rem : bs);
-  const uint64_t* a0 = li == 0 ? U.P->x + start * U.nw0 : Ly.aprev;
+  const uint64_t* a0 = li == 0 ? (U.one.x ? U.one.x : U.P->x + start * U.nw0) : Ly.aprev;
   pdl_wait();
   pdl_trigger();
   const int gk = live ? (Ly.group_of ? (int)Ly.group_of[k] : k / Ly.gamma) : 0;

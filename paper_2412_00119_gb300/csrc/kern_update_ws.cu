@@ -416,7 +416,7 @@ __device__ __forceinline__ void ws_consumer(const StepParams* __restrict__ P, Ws
 }
 
 template <int kP, bool kOnes>
-__global__ void __launch_bounds__(kThreads, 1) k_update_ws(StepParams* P) {
+__global__ void __launch_bounds__(kThreads, 1) k_update_ws(StepParams* P, const OneBatch one) {
   const Ring R = ring_of<kP>(P->bs);
   const int nslots = R.nslots;
   extern __shared__ uint8_t ws_raw[];
@@ -439,8 +439,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_ws(StepParams* P) {
   pdl_wait();
   pdl_trigger();
   const uint32_t sidx = ctrl->s_cur;
-  const int64_t start = (int64_t)sidx * P->bs;
-  const int64_t rem = P->n - start;
+  const int64_t start = one.x ? 0 : (int64_t)sidx * P->bs;
+  const int64_t rem = (one.x ? one.n : P->n) - start;
   const int bsz = (int)(rem < P->bs ? rem : P->bs);
   // an expired bounded wait in this step's forward pass: no CP, no R (the
   // selection kernel marked nothing either); the counters still advance
@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_ws(StepParams* P) {
     const DevLayer& D = P->layer[li];
     LayerSh& o = sh->lay[li];
     o.H = D.H; o.W = D.W; o.EV = D.EV; o.sel = D.sel; o.group_of = D.group_of;
-    o.aprev = li == 0 ? reinterpret_cast<const uint32_t*>(P->x + start * P->nw0)
+    o.aprev = li == 0 ? reinterpret_cast<const uint32_t*>(one.x ? one.x : P->x + start * P->nw0)
                       : reinterpret_cast<const uint32_t*>(P->layer[li - 1].A);
     o.row_base = D.row_base; o.gamma = D.gamma; o.ngrp = D.ngrp; o.ldh = D.ldh; o.nw_in = D.nw_in;
     o.ev_stride = D.ev_stride; o.Kin = D.Kin; o.pad = 0;
@@ -489,8 +489,8 @@ cudaError_t set_smem() {
 }
 
 template <int kP, bool kOnes>
-cudaError_t launch_one(unsigned grid, size_t smem, cudaStream_t st, bool pdl, StepParams* P) {
-  return launch_kernel(k_update_ws<kP, kOnes>, dim3(grid), dim3(kThreads), smem, st, pdl, P);
+cudaError_t launch_one(unsigned grid, size_t smem, cudaStream_t st, bool pdl, StepParams* P, const OneBatch& one) {
+  return launch_kernel(k_update_ws<kP, kOnes>, dim3(grid), dim3(kThreads), smem, st, pdl, P, one);
 }
 
 }  // namespace
@@ -516,17 +516,17 @@ cudaError_t prepare_update_ws() {
 }
 
 cudaError_t launch_update_ws(int nplanes, int h_max, int bs, unsigned grid, cudaStream_t st, bool pdl,
-                             StepParams* P) {
+                             StepParams* P, const OneBatch& one) {
   const bool ones = h_max == (1 << nplanes) - 1;
   const size_t smem = update_ws_smem(nplanes, bs);
   switch (nplanes) {
-    case 1: return launch_one<1, true>(grid, smem, st, pdl, P);
-    case 2: return launch_one<2, true>(grid, smem, st, pdl, P);
-    case 4: return ones ? launch_one<4, true>(grid, smem, st, pdl, P)
-                        : launch_one<4, false>(grid, smem, st, pdl, P);
-    case 8: return ones ? launch_one<8, true>(grid, smem, st, pdl, P)
-                        : launch_one<8, false>(grid, smem, st, pdl, P);
-    case 16: return launch_one<16, false>(grid, smem, st, pdl, P);
+    case 1: return launch_one<1, true>(grid, smem, st, pdl, P, one);
+    case 2: return launch_one<2, true>(grid, smem, st, pdl, P, one);
+    case 4: return ones ? launch_one<4, true>(grid, smem, st, pdl, P, one)
+                        : launch_one<4, false>(grid, smem, st, pdl, P, one);
+    case 8: return ones ? launch_one<8, true>(grid, smem, st, pdl, P, one)
+                        : launch_one<8, false>(grid, smem, st, pdl, P, one);
+    case 16: return launch_one<16, false>(grid, smem, st, pdl, P, one);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -61,3 +61,32 @@ def test_rows_kernel_batches(bs):
                                           (1001, (2100, 10010))])
 def test_ring_kernel(h_max, widths):
     check(widths, h_max, 60, 20)
+
+
+# calls of one mini-batch (their kernels get the inputs as parameters), whole and
+# short ones, mixed with a longer call and an evaluation
+@pytest.mark.parametrize("widths,group_mode,bs", [((70, 40), 0, 16), ((200, 96, 130), 2, 30), ((130, 64, 64, 64), 1, 100),
+                                                  ((5000, 4500), 0, 20), ((3000, 4096, 4096), 2, 150)])
+def test_calls_of_one_batch(widths, group_mode, bs):
+    gpu = B.BMLP(widths, 5, seed=3, bs=bs, group_mode=group_mode)
+    ref = O.OracleModel(list(widths), 5, seed=3, bs=bs)
+    ref.set_group_mode(group_mode)
+    sizes = [bs, bs, max(1, bs // 2), 2 * bs + 1, 1, bs] if widths[0] < 1000 else [bs, 2 * bs, 3]
+    n = sum(sizes)
+    xp = W.random_packed(5, n, widths[0])
+    y = np.random.default_rng(5).integers(0, 5, n).astype(np.int32)
+    x, yd, xpm = torch.from_numpy(xp.view(np.int64)).to(DEV), torch.from_numpy(y).to(DEV), W.unpack(xp, widths[0])
+    out = torch.empty(n, dtype=torch.int32, device=DEV)
+    a = 0
+    for m in sizes:
+        gpu.train(x[a:a + m], yd[a:a + m])
+        gpu.predict(x, out)
+        ref.train(xpm[a:a + m], y[a:a + m])
+        a += m
+    assert np.array_equal(out.cpu().numpy(), ref.predict(xpm))
+    for l in range(1, len(widths)):
+        H, Wb, _, _, step = gpu.state(l)
+        assert np.array_equal(H.astype(np.int32), ref.H(l).T)
+        assert np.array_equal(Wb, W.pack(np.where(ref.H(l).T > 0, 1, -1)))
+        assert step == ref.step
+    gpu.close()
