@@ -7,14 +7,14 @@
 // packed as bits (bit i % 64 of word i / 64 = 1 <-> +1, pad bits 0), the input
 // format of bmlp_train / bmlp_predict.
 //
-// k_binarize_regs (K <= kRegMax): a warp, or four warps, per pattern, with the
+// k_binarize_regs (K <= kRegMax): a warp, or two, per pattern, with the
 // pattern's values in registers as order-preserving 32-bit keys (bits ^
 // 0x80000000 for a clear sign bit, ~bits for a set one), so that memory is read
 // once.  The median is the key p with #{key < p} <= rank < #{key <= p}.  It is
 // bracketed: the median lies in [lo, hi], with #{key < lo} and #{key <= hi}
 // known.  The smallest value is tried first (the median of image-like data, which
-// is mostly zeros), then keys inside the bracket, interpolated linearly between
-// its ends by the counts (from the sixth round on in turn with the middle of the
+// is mostly zeros), then two of a sample of 32, then keys inside the bracket,
+// interpolated linearly between its ends by the counts (from the sixth round on in turn with the middle of the
 // key range, which alone ends after 32 rounds).  A round is one comparison per
 // value and a warp sum.  Once at most 32 candidates are left a warp lists them,
 // one per lane, and ranks each against the others; with many equal values the
@@ -22,7 +22,7 @@
 // the median as floats, so -0 and +0 are equal as they are in fp32, and one
 // ballot packs 32 of them.
 // Bound: memory, then instructions (about 8 per value).  60,000 x 784 of
-// grey levels: 52.4 us = 3.7 TB/s (the radix select 299 us).
+// grey levels: 36 us = 5.4 TB/s (the radix select 299 us), of normal values 82 (290).
 //
 // k_binarize_median (larger K): one CTA per pattern.  The median is found
 // exactly by a radix select over the same keys: four passes of 8-bit digits,
@@ -46,19 +46,19 @@ __device__ __forceinline__ float key_float(uint32_t k) {
   return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
 }
 
-constexpr int kRegWarps = 4;        // warps of a CTA
-constexpr int kRegMax = 32 * kRegWarps * 32;
+constexpr int kRegMax = 64 * 64;
 
-// kWarps warps per pattern (1 or kRegWarps), kR values per lane: K <= 32 kWarps kR.
-// Value j of lane l of the pattern's warp w is x[32 (w + kWarps j) + l].
-template <int kWarps, int kR>
-__global__ void __launch_bounds__(32 * kRegWarps)
+// kWarps warps per pattern (1, four patterns per CTA, or 2, a CTA), kR values per lane: K <= 32 kWarps kR;
+// K >= 32 kWarps kFull, so the first kFull values of every lane are inside the
+// pattern.  Value j of lane l of the pattern's warp w is x[32 (w + kWarps j) + l].
+template <int kWarps, int kR, int kFull>
+__global__ void __launch_bounds__(kWarps == 1 ? 128 : 32 * kWarps)
     k_binarize_regs(const float* __restrict__ x, int64_t n, int K, int nw, uint64_t* __restrict__ out) {
-  __shared__ uint32_t red[2][kRegWarps];
-  __shared__ uint32_t cand[kWarps == 1 ? kRegWarps : 1][32];
+  constexpr int kPats = kWarps == 1 ? 4 : 1;     // patterns per CTA
+  __shared__ uint32_t red[2][kWarps];
+  __shared__ uint32_t cand[kPats][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int w = kWarps == 1 ? 0 : warp;
-  constexpr int kPats = kRegWarps / kWarps;     // patterns per CTA
   const uint32_t rank = (uint32_t)((K + 1) / 2 - 1);   // 0-based rank of the lower median
   int flip = 0;
   // a sum (or minimum / maximum) over the pattern's warps
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(32 * kRegWarps)
     __syncthreads();
     uint32_t t = red[flip][0];
 #pragma unroll
-    for (int i = 1; i < kRegWarps; ++i)
+    for (int i = 1; i < kWarps; ++i)
       t = op == 0 ? t + red[flip][i] : (op == 1 ? min(t, red[flip][i]) : max(t, red[flip][i]));
     flip ^= 1;   // the next round writes the other buffer: no second barrier
     return t;
@@ -79,19 +79,17 @@ __global__ void __launch_bounds__(32 * kRegWarps)
        mu += (int64_t)gridDim.x * kPats) {
     const float* row = x + mu * (int64_t)K;
     uint32_t key[kR];   // values past K: the largest key, never below a pivot
+    auto inside = [&](int j) { return j < kFull || 32 * (w + kWarps * j) + lane < K; };
 #pragma unroll
-    for (int j = 0; j < kR; ++j) {
-      const int i = 32 * (w + kWarps * j) + lane;
-      key[j] = i < K ? __float_as_uint(__ldcs(row + i)) : 0x7FFFFFFFu;
-    }
-    uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
+    for (int j = 0; j < kR; ++j)
+      key[j] = inside(j) ? __float_as_uint(__ldcs(row + 32 * (w + kWarps * j) + lane)) : 0x7FFFFFFFu;
+    uint32_t kmin = 0xFFFFFFFFu;
 #pragma unroll
     for (int j = 0; j < kR; ++j) {
       key[j] ^= (uint32_t)((int32_t)key[j] >> 31) | 0x80000000u;
       kmin = min(kmin, key[j]);
-      if (32 * (w + kWarps * j) + lane < K) kmax = max(kmax, key[j]);
     }
-    uint32_t lo = all_warps(kmin, 1), hi = all_warps(kmax, 2);
+    uint32_t lo = all_warps(kmin, 1), hi = 0xFFFFFFFFu;
     uint32_t clo = 0u, chi = (uint32_t)K;   // #{key < lo}, #{key <= hi}
     uint32_t p = lo;
 #pragma unroll 1
@@ -108,36 +106,91 @@ __global__ void __launch_bounds__(32 * kRegWarps)
         clo = c;
       }
       if (lo >= hi) break;
-      if (kWarps == 1 && chi - clo <= 32u && hi != 0xFFFFFFFFu) {
+      if (it == 0) {
+        // not the smallest value: bracket between the 12th and the 21st of 32 values
+        // from four places of the pattern, in key order (a bitonic sort over the lanes)
+        uint32_t v = (lane & 2) ? ((lane & 1) ? key[7 * kR / 8] : key[5 * kR / 8])
+                                : ((lane & 1) ? key[3 * kR / 8] : key[kR / 8]);
+        if constexpr (kWarps > 1) {
+          if (lane < 32 / kWarps) cand[0][32 / kWarps * warp + lane] = v;
+          __syncthreads();
+          v = cand[0][lane];
+        }
+#pragma unroll
+        for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+          for (int j = k >> 1; j > 0; j >>= 1) {
+            const uint32_t o = __shfl_xor_sync(0xffffffffu, v, j);
+            v = ((lane & j) == 0) == ((lane & k) == 0) ? min(v, o) : max(v, o);
+          }
+        const uint32_t a = max(__shfl_sync(0xffffffffu, v, 11), lo), z = __shfl_sync(0xffffffffu, v, 20);
+        uint32_t ca = 0u, cz = 0u;   // #{key < a}, #{key <= z}; z is a value or the padding
+#pragma unroll
+        for (int j = 0; j < kR; ++j) {
+          ca += key[j] < a ? 1u : 0u;
+          cz += key[j] <= z ? 1u : 0u;
+        }
+        ca = all_warps(ca, 0);
+        cz = z == 0xFFFFFFFFu ? (uint32_t)K : all_warps(cz, 0);
+        if (rank < ca) {
+          hi = a - 1u;
+          chi = ca;
+        } else {
+          lo = a;
+          clo = ca;
+          if (rank < cz) {
+            hi = z;
+            chi = cz;
+          } else {
+            lo = z + 1u;
+            clo = cz;
+          }
+        }
+        if (lo >= hi) break;
+      }
+      if (chi - clo <= 32u && hi != 0xFFFFFFFFu) {
         // at most a warp of candidates: one per lane, ranked against the others
-        uint32_t* list = cand[warp];
-        uint32_t cnt = 0u;
+        uint32_t* list = cand[kWarps == 1 ? warp : 0];
+        uint32_t at = 0u;   // where this warp's candidates go
+        if constexpr (kWarps > 1) {
+          uint32_t mine = 0u;
+#pragma unroll
+          for (int j = 0; j < kR; ++j) mine += (key[j] >= lo && key[j] <= hi) ? 1u : 0u;
+          mine = __reduce_add_sync(0xffffffffu, mine);
+          if (lane == 0) red[flip][warp] = mine;
+          __syncthreads();
+          for (int i = 0; i < warp; ++i) at += red[flip][i];
+          flip ^= 1;
+        }
 #pragma unroll
         for (int j = 0; j < kR; ++j) {
           const bool in = key[j] >= lo && key[j] <= hi;
           const unsigned b = __ballot_sync(0xffffffffu, in);
-          if (in) list[cnt + __popc(b & ((1u << lane) - 1u))] = key[j];
-          cnt += __popc(b);
+          if (in) list[at + __popc(b & ((1u << lane) - 1u))] = key[j];
+          at += __popc(b);
         }
-        __syncwarp();
+        if constexpr (kWarps > 1) __syncthreads();
+        else __syncwarp();
+        const uint32_t cnt = chi - clo;
         const uint32_t mine = (uint32_t)lane < cnt ? list[lane] : 0xFFFFFFFFu;
         uint32_t below = 0u;
         for (uint32_t i = 0; i < cnt; ++i) {
           const uint32_t o = list[i];
           below += (o < mine || (o == mine && i < (uint32_t)lane)) ? 1u : 0u;
         }
-        const unsigned at = __ballot_sync(0xffffffffu, (uint32_t)lane < cnt && below == rank - clo);
-        hi = __shfl_sync(0xffffffffu, mine, __ffs(at) - 1);
-        __syncwarp();
+        const unsigned who = __ballot_sync(0xffffffffu, (uint32_t)lane < cnt && below == rank - clo);
+        hi = __shfl_sync(0xffffffffu, mine, __ffs(who) - 1);
+        if constexpr (kWarps > 1) __syncthreads();   // the list is the next pattern's
+        else __syncwarp();
         break;
       }
-      if (it >= 3 || chi - clo == 1u) {
+      if (it >= 3 || chi - clo == 1u || hi == 0xFFFFFFFFu) {
         // the bracket's ends onto values (many equal ones, or one candidate)
         uint32_t a = 0xFFFFFFFFu, z = 0u;
 #pragma unroll
         for (int j = 0; j < kR; ++j) {
           if (key[j] >= lo) a = min(a, key[j]);
-          if (key[j] <= hi) z = max(z, key[j]);
+          if (key[j] <= hi && inside(j)) z = max(z, key[j]);
         }
         lo = all_warps(a, 1);
         hi = all_warps(z, 2);
@@ -146,22 +199,32 @@ __global__ void __launch_bounds__(32 * kRegWarps)
       p = lo + ((hi - lo) >> 1);
       if (it < 6 || (it & 1) == 0) {
         const float flo = key_float(lo), fhi = key_float(hi);
-        const float f = flo + (fhi - flo) * (((float)(rank - clo) + 0.5f) / (float)(chi - clo));
+        // eight values past the median, towards the farther end: the bracket then
+        // closes from both sides, and soon holds at most a warp of candidates
+        const float t = (float)(rank - clo) + 0.5f, na = (float)(chi - clo);
+        const float to = 2.0f * t < na ? fminf(t + 8.0f, na - 0.5f) : fmaxf(t - 8.0f, 0.5f);
+        const float f = flo + (fhi - flo) * (to / na);
         const uint32_t kf = float_key(f);
         if (kf >= lo && kf < hi) p = kf;   // (a NaN's or an infinity's key: the middle)
       }
     }
+    // x > m as floats, on keys: none for a NaN m; m = -0 compares like +0; a NaN x
+    // (keys above +infinity's; the padding is one) compares false
     const float m = key_float(hi);
-    uint32_t mine = 0u;
+    const uint32_t above = m == 0.0f ? 0x80000001u : (m == m ? hi + 1u : 0xFFFFFFFFu);
+    const uint32_t width = above <= 0xFF800000u ? 0xFF800001u - above : 0u;
+    // lane l holds words w + kWarps l and, beyond 32, w + kWarps (l + 32) of the row
+    uint32_t mine[2] = {0u, 0u};
 #pragma unroll
     for (int j = 0; j < kR; ++j) {
-      const int i = 32 * (w + kWarps * j) + lane;
-      const unsigned bits = __ballot_sync(0xffffffffu, i < K && key_float(key[j]) > m);
-      if (lane == j) mine = bits;
+      const unsigned bits = __ballot_sync(0xffffffffu, key[j] - above < width);
+      if (lane == (j & 31)) mine[j >> 5] = bits;
     }
-    // lane j holds word w + kWarps j of the row
-    const int word = w + kWarps * lane;
-    if (word < 2 * nw) reinterpret_cast<uint32_t*>(out + mu * (int64_t)nw)[word] = mine;
+#pragma unroll
+    for (int h = 0; h < (kR > 32 ? 2 : 1); ++h) {
+      const int word = w + kWarps * (lane + 32 * h);
+      if (word < 2 * nw) reinterpret_cast<uint32_t*>(out + mu * (int64_t)nw)[word] = mine[h];
+    }
   }
 }
 
@@ -227,16 +290,21 @@ __global__ void __launch_bounds__(kBinThreads)
 void launch_binarize_median(const float* x, int64_t n, int K, int nw, uint64_t* out,
                             cudaStream_t st) {
   const int64_t grid = n < (int64_t)1 << 20 ? n : (int64_t)1 << 20;
-  auto regs = [&](auto kern, int pats) {
+  // the fewest registers that hold the pattern; one warp as long as it can (a
+  // round of two or more warps costs a barrier: 20,000 x 1200 normal values 107 us
+  // with four warps a pattern)
+  auto regs = [&](auto kern, int pats, int threads) {
     const int64_t ctas = (n + pats - 1) / pats;
-    kern<<<(unsigned)(ctas < grid ? ctas : grid), 32 * kRegWarps, 0, st>>>(x, n, K, nw, out);
+    kern<<<(unsigned)(ctas < grid ? ctas : grid), threads, 0, st>>>(x, n, K, nw, out);
   };
-  if (K <= 32 * 8) regs(k_binarize_regs<1, 8>, kRegWarps);
-  else if (K <= 32 * 16) regs(k_binarize_regs<1, 16>, kRegWarps);
-  else if (K <= 32 * 25) regs(k_binarize_regs<1, 25>, kRegWarps);
-  else if (K <= 32 * 32) regs(k_binarize_regs<1, 32>, kRegWarps);
-  else if (K <= kRegMax / 2) regs(k_binarize_regs<kRegWarps, 16>, 1);
-  else if (K <= kRegMax) regs(k_binarize_regs<kRegWarps, 32>, 1);
+  if (K <= 32 * 8) regs(k_binarize_regs<1, 8, 0>, 4, 128);
+  else if (K <= 32 * 16) regs(k_binarize_regs<1, 16, 8>, 4, 128);
+  else if (K <= 32 * 25) regs(k_binarize_regs<1, 25, 16>, 4, 128);
+  else if (K <= 32 * 32) regs(k_binarize_regs<1, 32, 25>, 4, 128);
+  else if (K <= 32 * 48) regs(k_binarize_regs<1, 48, 32>, 4, 128);
+  else if (K <= 32 * 64) regs(k_binarize_regs<1, 64, 48>, 4, 128);
+  else if (K <= 64 * 48) regs(k_binarize_regs<2, 48, 32>, 1, 64);
+  else if (K <= kRegMax) regs(k_binarize_regs<2, 64, 48>, 1, 64);
   else k_binarize_median<<<(unsigned)grid, kBinThreads, 0, st>>>(x, n, K, nw, out);
 }
 

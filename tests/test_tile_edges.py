@@ -117,7 +117,8 @@ def test_expand_edges(n, D, K, kind):
 
 
 # widths at every change of registers per lane and warps per pattern
-@pytest.mark.parametrize("K", [1, 2, 31, 33, 256, 257, 512, 513, 799, 800, 801, 1024, 1025, 2048, 2049, 4096, 4097])
+@pytest.mark.parametrize("K", [1, 2, 31, 33, 256, 257, 512, 513, 800, 801, 1024, 1025, 1536, 1537, 2048, 2049, 3072, 3073,
+                               4096, 4097])
 @pytest.mark.parametrize("kind", ["pixels", "gauss", "ties", "wide"])
 def test_binarize_edges(K, kind):
     n = 37
@@ -127,6 +128,7 @@ def test_binarize_edges(K, kind):
         x[0] = 3.0
         x[1, ::2], x[1, 1::2] = np.float32(np.inf), np.float32(-np.inf)
         x[2, : K // 2] = np.float32(-0.0)
+        x[3, : K // 2 + 1], x[3, K // 2 + 1:] = np.float32(-0.0), np.float32(0.0)   # median -0
     else:
         x = W.real_patterns(K, n, K, kind)
     out = torch.full((n, W.words(K)), -1, dtype=torch.int64, device=DEV)
