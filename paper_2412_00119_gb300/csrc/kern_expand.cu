@@ -11,7 +11,7 @@
 // k % 64 of word k / 64, pad bits 0), i.e. bmlp_train / bmlp_predict input
 // for K_0 = K.
 //
-// k_expand_tc (D <= kTcMaxD): the product on the tensor cores, exact in 4-bit
+// k_expand_tc (D <= kTcMaxD, x aligned to 4 bytes): the product on the tensor cores, exact in 4-bit
 // operands.  A byte is four base-4 digits, x = d0 + 4 d1 + 16 d2 + 64 d3, and 0,
 // 1, 2, 3 and +-1 are e2m1 values, so z is the sum of four e2m1 x e2m1 products
 // with block scales 1, 4, 16 and 64 (UE8M0 holds powers of two); every product
@@ -33,7 +33,7 @@
 // Every mbarrier wait is bounded like all others of the library; this entry
 // point has no handle, so an expiry leaves its tiles unwritten.
 //
-// k_expand_sign (larger D): a 128-pattern x 128-neuron tile per CTA of 256 threads, the
+// k_expand_sign (the rest): a 128-pattern x 128-neuron tile per CTA of 256 threads, the
 // inputs in chunks of 64 (one word of E per neuron): the chunk's bytes of x
 // and the chunk's E bits, expanded to +-1 bytes, are staged in shared memory
 // (rows padded to 17 words: conflict-free reads; the next chunk's raw words
@@ -221,7 +221,11 @@ __device__ __forceinline__ uint32_t weight_nibbles(uint32_t byte) {
   return 0x22222222u | even | (odd << 4);
 }
 
-// kBytes: 16 or 4, the copies that every row of x allows, or 1.
+// kBytes: 16 or 4, the copies that every row of x allows, or 1: rows that start at
+// any byte of an x aligned to words.  Those are copied as the words that hold
+// them, zeros past the row's end, and shifted by the producers: 600 x 70 -> 1024
+// 7.3 us, 20,000 x 785 -> 1024 53 (byte loads in the loaders 16.5 and 100, the dp4a
+// kernel 12.4 and 357).
 template <int kBytes>
 __global__ void __launch_bounds__(kXTcThreads, 1)
     k_expand_tc(const uint8_t* __restrict__ x, int64_t n, int D, const uint64_t* __restrict__ E, int K, int nwD,
@@ -299,6 +303,9 @@ __global__ void __launch_bounds__(kXTcThreads, 1)
     bool ok = true;
 #pragma unroll 1
     for (int64_t t = blockIdx.y; t < tiles && ok; t += gridDim.y, ch -= nchunks) {
+      // bits before the row's first byte in its words
+      const uint32_t skew =
+          kBytes == 1 ? 8u * (uint32_t)((reinterpret_cast<uintptr_t>(x) + (t * XM + 32 * q + lane) * D) & 3) : 0u;
 #pragma unroll 1
       for (int p = 0; p < npc && ok; ++p) {
         ok = __all_sync(0xffffffffu, mbar_wait(&sh->piece_full[slot], pph, failed));
@@ -311,6 +318,12 @@ __global__ void __launch_bounds__(kXTcThreads, 1)
           for (int i = 0; i < 4; ++i) {
             const uint4 v = lds128(src + 16u * i);
             w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+          }
+          if constexpr (kBytes == 1) {
+            uint32_t next;
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(next) : "r"(src + 64u) : "memory");
+#pragma unroll
+            for (int i = 0; i < 16; ++i) w[i] = __funnelshift_r(w[i], i < 15 ? w[i + 1] : next, skew);
           }
           ok = __all_sync(0xffffffffu, mbar_wait(&sh->empty[s], eph, failed));
           if (!ok) break;
@@ -351,34 +364,45 @@ __global__ void __launch_bounds__(kXTcThreads, 1)
     bool ok = true;
 #pragma unroll 1
     for (int64_t t = blockIdx.y; t < tiles && ok; t += gridDim.y) {
-      const uint8_t* rows = x + (t * XM + r0) * D + c0;
+      const uint8_t* rows = x + (t * XM + r0) * D + (kBytes == 1 ? 0 : c0);
+      // rows past n keep what is there: their outputs are dropped (e2m1 has no NaN)
       const int live = (int)min((int64_t)XM, n - t * XM) - r0;
 #pragma unroll 1
       for (int p = 0; p < npc && ok; ++p) {
         ok = mbar_wait(&sh->piece_empty[slot], ph, failed);
         if (!ok) break;
+        if constexpr (kBytes == 1) {
+          // the aligned word that is c past the first of a row, its bytes of the row
+          auto copy = [&](const uint8_t* row, uint32_t to, int c) {
+            const int skew = (int)(reinterpret_cast<uintptr_t>(row) & 3);
+            const int size = min(4, max(0, D + skew - c));
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
+                         ::"r"(to), "l"(size > 0 ? row + (c - skew) : x), "r"(size) : "memory");
+          };
+          const uint32_t to0 = smem_u32(pieces) + slot * (uint32_t)kXPieceBytes;
+          const uint8_t* row = rows;
+          uint32_t to = to0 + (uint32_t)(r0 * kXRow + c0);
+#pragma unroll 8
+          for (int i = 0; i < live; i += kRows, row += kRows * D, to += (uint32_t)(kRows * kXRow))
+            copy(row, to, kXPiece * p + c0);
+          static_assert(32 * kXLoadWarps == XM, "a row's last word by a thread each");
+          if (t * XM + tid < n)
+            copy(x + (t * XM + tid) * D, to0 + (uint32_t)(tid * kXRow + kXPiece), kXPiece * (p + 1));
+        } else {
 #pragma unroll 1
-        for (int e = 0; e < kCols; ++e) {
-          const int c = kXPiece * p + c0 + e * 32 * kXLoadWarps * kStep;   // the copy's first input
-          const uint8_t* src = rows + kXPiece * p + e * 32 * kXLoadWarps * kStep;
-          uint32_t to = smem_u32(pieces) + slot * (uint32_t)kXPieceBytes +
-                        (uint32_t)(r0 * kXRow + c0 + e * 32 * kXLoadWarps * kStep);
+          for (int e = 0; e < kCols; ++e) {
+            const int c = kXPiece * p + c0 + e * 32 * kXLoadWarps * kStep;   // the copy's first input
+            const uint8_t* src = rows + kXPiece * p + e * 32 * kXLoadWarps * kStep;
+            uint32_t to = smem_u32(pieces) + slot * (uint32_t)kXPieceBytes +
+                          (uint32_t)(r0 * kXRow + c0 + e * 32 * kXLoadWarps * kStep);
 #pragma unroll 4
-          for (int i = 0; i < XM; i += kRows, src += (int64_t)kRows * D, to += (uint32_t)(kRows * kXRow)) {
-            if constexpr (kBytes == 1) {
-              uint32_t v = 0;
-#pragma unroll
-              for (int b = 0; b < 4; ++b)
-                if (i < live && c + b < D) v |= (uint32_t)__ldg(src + b) << (8 * b);
-              asm volatile("st.shared.b32 [%0], %1;" ::"r"(to), "r"(v) : "memory");
-            } else {
-              const bool on = i < live && c < D;   // D is a multiple of kBytes
+            for (int i = 0; i < live; i += kRows, src += kRows * D, to += (uint32_t)(kRows * kXRow)) {
+              const bool on = c < D;   // D is a multiple of kBytes
               cp_async_or_zero<kBytes>(to, on ? src : x, on);
             }
           }
         }
-        if constexpr (kBytes == 1) mbar_arrive(&sh->piece_full[slot]);
-        else cp_async_arrive(&sh->piece_full[slot]);
+        cp_async_arrive(&sh->piece_full[slot]);
         if (++slot == kXPieces) {
           slot = 0;
           ph ^= 1u;
@@ -509,7 +533,7 @@ void launch_expand_weights(uint64_t seed, int K, int D, uint64_t* E, cudaStream_
 cudaError_t launch_expand_sign(const uint8_t* x, int64_t n, int D, const uint64_t* E, int K, uint64_t* out,
                                cudaStream_t st) {
   const int nwD = (D + 63) / 64, nwK = (K + 63) / 64;
-  if (D <= kTcMaxD) {
+  if (D <= kTcMaxD && reinterpret_cast<uintptr_t>(x) % 4 == 0) {
     const uintptr_t a = reinterpret_cast<uintptr_t>(x) | (uintptr_t)(uint32_t)D;
     return (a & 15) == 0 ? launch_expand_tc<16>(x, n, D, E, K, out, st)
                          : ((a & 3) == 0 ? launch_expand_tc<4>(x, n, D, E, K, out, st)

@@ -116,6 +116,24 @@ def test_expand_edges(n, D, K, kind):
     assert np.array_equal(out.cpu().numpy().view(np.uint64), W.pack(O.expand_sign(x, e)))
 
 
+# rows that start at any byte of a 32-bit word, also the first; other bytes all
+# around them
+@pytest.mark.parametrize("off", [0, 1, 2, 3])
+@pytest.mark.parametrize("n,D,K", [(1, 1, 1), (5, 3, 70), (129, 70, 64), (300, 254, 130), (140, 255, 65), (131, 513, 257),
+                                   (127, 256, 64), (50, 4607, 64)])
+def test_expand_unaligned(n, D, K, off):
+    x = W.pixel_bytes(n + D + off, n, D, "pixels")
+    x[-1, -1] = x[0, 0] = 255
+    buf = torch.full((n * D + 16,), 255, dtype=torch.uint8, device=DEV)
+    buf[off:off + n * D] = torch.from_numpy(x).to(DEV).view(-1)
+    e = O.expand_weights(5 + K, K, D)
+    E = torch.empty((K, W.words(D)), dtype=torch.int64, device=DEV)
+    B.bmlp_expand_weights(5 + K, K, D, E)
+    out = torch.full((n, W.words(K)), -1, dtype=torch.int64, device=DEV)
+    B.bmlp_expand_sign(buf[off:off + n * D].view(n, D), E, K, out)
+    assert np.array_equal(out.cpu().numpy().view(np.uint64), W.pack(O.expand_sign(x, e)))
+
+
 # widths at every change of registers per lane and warps per pattern
 @pytest.mark.parametrize("K", [1, 2, 31, 33, 256, 257, 512, 513, 800, 801, 1024, 1025, 1536, 1537, 2048, 2049, 3072, 3073,
                                4096, 4097])
