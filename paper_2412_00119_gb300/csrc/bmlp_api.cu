@@ -1,10 +1,12 @@
 // bmlp_api.cu -- host side of the C-ABI declared in include/bmlp.h.
 //
-// One training mini-batch is one event-draw launch, L forward launches, one
-// local-classifier + selection launch and one update launch.  All of them read
-// the batch index s and the step counter t from a device-resident control block
-// that the update kernel advances, so captured CUDA graphs (of eight steps, or
-// one) replay step after step with no host work between steps.  Batch pointers
+// One training mini-batch is L forward launches, one local-classifier +
+// selection launch and one update launch (which draws the reinforcement events
+// itself up to kRowsWeights hidden weights; above, a launch of its own draws them
+// on a branch of the graph).  All of them read the batch index s and the step
+// counter t from a device-resident control block that the update kernel
+// advances, so captured CUDA graphs (of eight steps, or one) replay step after
+// step with no host work between steps.  Batch pointers
 // live in a device-resident parameter block that a stream-ordered copy
 // refreshes at the start of a call.  Each entry point that launches work opens
 // an NVTX range named after it (header-only NVTX v3: a no-op unless a tracing
@@ -94,6 +96,7 @@ struct bmlp {
   ClsArgs cls{};
   unsigned updCtas = 0, evCtas = 0;
   bool updRing = false;   // the update streams through a shared-memory ring (large models)
+  int evLayer = 0;        // its graphs draw events beside the passes from this layer on
   // profiling
   bool profiling = false;       // events around the kernels being enqueued now
   int32_t profEvery = 0;        // 0 off, 1 every mini-batch, S every S-th mini-batch
@@ -234,11 +237,6 @@ int prof_collect(bmlp_t* h, cudaStream_t st) {
   return BMLP_OK;
 }
 
-// Enqueue the kernels of one training mini-batch on `st`.  The reinforcement
-// events depend only on (seed, layer, neuron, step, p_r): when `fork` is set
-// (graph capture) their kernel runs on a side stream next to the forward
-// passes, which leave most of every SM idle, and joins before the update;
-// otherwise it runs first on `st`.
 // Mini-batch steps per captured training graph (a shorter run, or one that
 // has sampled steps in the way, uses the one-step graph).
 constexpr int kGraphSteps = 8;
@@ -249,6 +247,15 @@ constexpr int kGraphSteps = 8;
 // 113.6, 268 M (8192x4) 152.7 / 198.7; 2.9 M (784-1024x3) 41.3 / 30.0, and at 15 M
 // (3072-2048x3) the ring alone, without the draws, 36.7 / 35.5.
 constexpr int64_t kRowsWeights = 20ll << 20;
+// Where the draws of the ring's models branch off (they read only the step counter
+// and the tables): before the first pass with one layer, or with a layer of this
+// many weights at up to 128 patterns, else after it.  Step time (us), before the
+// first pass / after it (with one layer: after the selection, no branch):
+// 5120-5120 35.4 / 43.2, 8192-8192 45.9 / 52.0, 3072-8192x2 69.1 / 73.2,
+// 8192x4 138.9 / 146.4; 3072-4096x4 66.8 / 63.6, 6144x2 60.0 / 59.1,
+// 6144-8192-6144 70.9 / 70.6, 7168x4 128.6 / 127.6, 8192x4 at 300 patterns
+// 236.9 / 235.5.
+constexpr int64_t kEarlyDrawWeights = 56ll << 20;
 
 // One mini-batch step.  How it is launched:
 //   kStepPlain    kernel by kernel with full dependencies (sampled mini-batches);
@@ -263,8 +270,8 @@ enum StepForm { kStepPlain, kStepDirect, kStepGraph, kStepChained };
 int enqueue_step(bmlp_t* h, cudaStream_t st, StepForm form, const OneBatch& one = OneBatch{}) {
   const bool fork = form == kStepGraph || form == kStepChained, pdl = form != kStepPlain;
   for (int l = 1; l <= h->L; ++l) {
-    if (fork && h->updRing && l == 2) {
-      // the events are drawn on a branch beside the other layers' passes
+    if (fork && l == h->evLayer) {
+      // the events are drawn on a branch beside the passes from this one on
       CK(h, cudaEventRecord(h->evFork, st));
       CK(h, cudaStreamWaitEvent(h->sideStream, h->evFork, 0));
       launch_r_events(h->evCtas, h->sideStream, h->dP, h->hp.key0, h->hp.key1);
@@ -289,8 +296,8 @@ int enqueue_step(bmlp_t* h, cudaStream_t st, StepForm form, const OneBatch& one 
   h->cls.one = one;
   CK(h, launch_cls_select(h->cls, h->max_K, st, pdl && h->tc));
   prof_end(h, st);
-  if (fork && h->updRing && h->L > 1) CK(h, cudaStreamWaitEvent(st, h->evJoin, 0));
-  if (h->updRing && (!fork || h->L == 1)) {
+  if (fork && h->updRing) CK(h, cudaStreamWaitEvent(st, h->evJoin, 0));
+  if (h->updRing && !fork) {
     prof_begin(h, kProfEvents, st);
     launch_r_events(h->evCtas, st, h->dP, h->hp.key0, h->hp.key1);
     prof_end(h, st);
@@ -543,7 +550,7 @@ int bmlp_create(const int32_t* widths, int32_t n_widths, int32_t classes, int16_
   P.key1 = (uint32_t)(seed >> 32);
   UpdArgs& U = h->upd;
   int upd_cta = 0, ev_cta = 0;
-  int64_t weights = 0;
+  int64_t weights = 0, largest = 0;   // hidden weights of the model, of its largest layer
   for (int l = 1; l <= L; ++l) {
     DevLayer& D = P.layer[l - 1];
     D.Kin = h->K[l - 1]; D.Kout = h->K[l];
@@ -585,6 +592,7 @@ int bmlp_create(const int32_t* widths, int32_t n_widths, int32_t classes, int16_
     UpdLayer& o = U.layer[l - 1];
     o.H = D.H; o.W = D.W; o.sel = D.sel; o.group_of = D.group_of;
     weights += (int64_t)D.Kin * D.Kout;
+    largest = std::max(largest, (int64_t)D.Kin * D.Kout);
     o.aprev = l == 1 ? nullptr : P.layer[l - 2].A;
     o.Kin = D.Kin; o.Kout = D.Kout; o.gamma = D.gamma; o.ldh = D.ldh; o.nw_in = D.nw_in;
     upd_cta = update_rows_layout(o, upd_cta);
@@ -602,6 +610,7 @@ int bmlp_create(const int32_t* widths, int32_t n_widths, int32_t classes, int16_
   h->evCtas = (unsigned)ev_cta;
   h->updRing = weights > kRowsWeights;
   if (h->updRing) {
+    h->evLayer = L == 1 || (largest >= kEarlyDrawWeights && bs <= 128) ? 1 : 2;
     const cudaError_t ea = prepare_update_ws();
     if (ea != cudaSuccess) return bail(cuda_fail(h, ea, "update kernel shared memory attribute"));
   }

@@ -219,9 +219,10 @@ using namespace upd;
 // so it runs beside the forward passes.  Bound: instruction issue.  A list of
 // several rows leaves fewer lanes idle in its last round than one of a row (32
 // candidates of 128 blocks at 8192 inputs): 24.3 us for the four
-// layers of 8192 alone, 28.6 with a list per row, 31 with a CTA of eight rows.
-__global__ void __launch_bounds__(kEvThreads) k_r_events(const StepParams* __restrict__ P,
-                                                         uint32_t key0, uint32_t key1) {
+// layers of 8192 alone, 28.6 with a list per row, 31 with a CTA of eight rows.  Registers are
+// held to twelve CTAs per SM, so that they fit beside the CTAs of a forward pass.
+__global__ void __launch_bounds__(kEvThreads, 12) k_r_events(const StepParams* __restrict__ P,
+                                                             uint32_t key0, uint32_t key1) {
   constexpr int kW = kEvThreads / 32;
   __shared__ Tables s_rt;
   __shared__ uint16_t s_cand[kW][128 * kEvRowsPerWarp];   // row * 128 + block
@@ -232,7 +233,7 @@ __global__ void __launch_bounds__(kEvThreads) k_r_events(const StepParams* __res
   load_tables<kEvThreads>(s_rt, P->rt[li]);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t l = (uint32_t)li + 1u;
-  const uint32_t tt = (uint32_t)P->ctrl->t_cur;
+  const uint32_t tt = (uint32_t)P->ctrl->t;   // the first pass may not have copied it yet
   const int Kin = Ly.Kin, nblk = Ly.nblk, stride = Ly.ev_stride;
   uint16_t* cand = s_cand[warp];
   const int k0 = (bid - Ly.ev_cta_base) * kEvRowsPerCta + warp * kEvRowsPerWarp;

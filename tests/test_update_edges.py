@@ -63,6 +63,12 @@ def test_ring_kernel(h_max, widths):
     check(widths, h_max, 60, 20)
 
 
+# steps in a row: the events are drawn beside the first pass or the second
+@pytest.mark.parametrize("widths", [(5000, 4500), (4600, 4600, 300)])
+def test_ring_kernel_steps(widths):
+    check(widths, 255, 18 * 10, 10)
+
+
 # calls of one mini-batch (their kernels get the inputs as parameters), whole and
 # short ones, mixed with a longer call and an evaluation
 @pytest.mark.parametrize("widths,group_mode,bs", [((70, 40), 0, 16), ((200, 96, 130), 2, 30), ((130, 64, 64, 64), 1, 100),
