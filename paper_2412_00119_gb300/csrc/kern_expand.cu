@@ -46,6 +46,8 @@
 // k_expand_weights: E from the Philox stream of the expansion weights,
 // e_k,i = +1 iff bit 31 of word i%4 of Philox (i/4, k, 33*2^16, 0) (the
 // library's stream layout is listed in bmlp_internal.cuh); pad bits 0.
+#include <algorithm>
+
 #include "tc_common.cuh"
 
 namespace bk {
@@ -446,14 +448,15 @@ __global__ void __launch_bounds__(kXTcThreads, 1)
   } else if (warp >= kXEpi0) {
     // ---------------- epilogue ----------------
     const int sub = warp & 3, half = (warp - kXEpi0) >> 2;
-    const int words = nb / 64;   // 32-neuron words of this warp: half words half, ..
+    // this warp's words of 32 neurons
+    const int first = half * ((nb / 32 + 1) / 2), words = (nb / 32 + 1 - half) / 2;
     uint32_t tile = 0;
 #pragma unroll 1
     for (int64_t t = blockIdx.y; t < tiles; t += gridDim.y, ++tile) {
       if (!__all_sync(0xffffffffu, mbar_wait(&sh->done, tile & 1u, failed))) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       uint32_t word[4] = {0u, 0u, 0u, 0u};
-      sign_words<4>(word, tmem + ((uint32_t)(32 * sub) << 16) + (uint32_t)(32 * half * words), words, 0.0f);
+      sign_words<4>(word, tmem + ((uint32_t)(32 * sub) << 16) + (uint32_t)(32 * first), words, 0.0f);
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(&sh->drained);
@@ -462,7 +465,7 @@ __global__ void __launch_bounds__(kXTcThreads, 1)
         uint32_t* row = reinterpret_cast<uint32_t*>(out + m * nwK);
 #pragma unroll
         for (int cb = 0; cb < 4; ++cb) {
-          const int nn = n0 + 32 * (half * words + cb), valid = K - nn;
+          const int nn = n0 + 32 * (first + cb), valid = K - nn;
           const uint32_t keep = valid >= 32 ? 0xffffffffu : (valid <= 0 ? 0u : (1u << valid) - 1u);
           // words wholly past K (inside the row's last 64-bit word) are written 0
           if (cb < words && (nn >> 5) < 2 * nwK) row[nn >> 5] = word[cb] & keep;
@@ -484,13 +487,23 @@ cudaError_t launch_expand_tc(const uint8_t* x, int64_t n, int D, const uint64_t*
   const int blocks = (D + kXPiece - 1) / kXPiece;   // of 256 inputs
   const int64_t tiles = (n + XM - 1) / XM;
   const int sms = sm_count();
-  // the widest neuron tile whose weights fit; narrower ones while all tiles
-  // together leave SMs idle
-  int nb = 256;
-  while (nb > 64 && (nb * 128 * blocks > 18 * 64 * 128 || nb / 2 >= K || tiles * ((K + nb - 1) / nb) < sms)) nb /= 2;
-  const unsigned nt = (unsigned)((K + nb - 1) / nb);
-  int64_t gy = sms / (int)nt > 0 ? sms / (int)nt : 1;
-  if (gy > tiles) gy = tiles;
+  // Neurons per CTA: a chunk takes 560 to 590 clocks at any width, so the fewest
+  // rounds of pattern tiles over the widths whose weights fit, of equal ones the
+  // narrowest (halvings of 256 in place of steps of 32: 60,000 x 3072 -> 1024
+  // 770 us, now 507; 600 x 784 -> 2048 14.5, now 10.4).
+  const int words = (K + 63) / 64;   // of 64 neurons in a packed row
+  int nb = 64;
+  int64_t gy = 1, rounds = INT64_MAX;
+  for (int w = 64; w <= kXMaxN && w * blocks <= 18 * 64; w += 32) {
+    const int64_t nt = (64ll * words + w - 1) / w, g = std::min(tiles, std::max<int64_t>(1, sms / nt));
+    const int64_t r = (tiles + g - 1) / g * ((nt * g + sms - 1) / sms);
+    if (r < rounds) {
+      rounds = r;
+      nb = w;
+      gy = g;
+    }
+  }
+  const unsigned nt = (unsigned)((64ll * words + nb - 1) / nb);
   const cudaError_t e = cudaFuncSetAttribute(k_expand_tc<kBytes>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)kXSmem);
   if (e != cudaSuccess) return e;

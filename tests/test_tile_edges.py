@@ -96,12 +96,13 @@ def test_labels_of_every_layer(classes, n):
     gpu.close()
 
 
-# chunks of 64 inputs, blocks of 256, neuron tiles of 256 / 128 / 64, the widest
+# chunks of 64 inputs, blocks of 256, neuron tiles of 64 to 256 in steps of 32, the widest
 # tensor-core shape (4608) and the first past it, rows that allow copies of 16,
 # 4 and 1 bytes, more tiles than CTAs
 EXPAND = [(1, 1, 1), (127, 63, 64), (129, 64, 65), (130, 256, 128), (300, 257, 257), (128, 1024, 256),
           (200, 1025, 300), (260, 1280, 256), (100, 1284, 70), (64, 2561, 130), (33, 4608, 65),
-          (33, 4609, 65), (30000, 16, 300)]
+          (33, 4609, 65), (30000, 16, 300), (300, 1100, 449), (500, 1500, 1000), (140, 2900, 193), (2000, 700, 2100),
+          (700, 300, 1500), (4000, 3000, 96), (20000, 1600, 161)]
 
 
 @pytest.mark.parametrize("n,D,K", EXPAND)
