@@ -189,10 +189,6 @@ cudaError_t launch_kernel(void (*k)(KArgs...), dim3 grid, dim3 block, size_t sme
   return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
-__device__ __forceinline__ int clip_h(int h, int h_max) {
-  return h > h_max ? h_max : (h < -h_max ? -h_max : h);
-}
-
 // ---------------------------------------------------------------------------
 // Kernels
 // ---------------------------------------------------------------------------

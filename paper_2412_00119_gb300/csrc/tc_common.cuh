@@ -1,7 +1,8 @@
-// tc_common.cuh -- device helpers shared by the tcgen05 forward kernels:
-// mbarrier waits (bounded), shared-memory matrix descriptors, the
-// tcgen05.mma kind::f8f6f4 issue and commit, and the expansion of bit-packed
-// +-1 vectors into e4m3 bytes in the 128B-swizzled K-major stage layout.
+// tc_common.cuh -- device helpers shared by the tcgen05 kernels: mbarrier
+// waits (bounded), asynchronous copies, shared-memory matrix descriptors, the
+// tcgen05.mma issue (kind::mxf4; kind::f8f6f4 for the peak kernel) and commit,
+// the expansion of bit-packed +-1 vectors into e2m1, and the tensor-memory
+// loads and stores around them.
 #pragma once
 
 #include "bmlp_internal.cuh"
