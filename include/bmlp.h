@@ -303,8 +303,10 @@ int bmlp_debug_wait_probe(bmlp_t* h, int32_t arrive, double seconds);
  * the call ends (which then synchronises the stream).  kinds: 0 forward
  * (train), 1 local classifier + selection, 2 update (CP + R + repack),
  * 3 forward (predict), 4 predict output, 5 host-buffer copies, 6 drawing of
- * the reinforcement events (in the replayed step graph this kernel runs beside
- * the forward passes; in a sampled mini-batch it runs first, alone).
+ * the reinforcement events by a kernel of its own (models of more than 20 M
+ * hidden weights; in the replayed step graph it runs beside the forward
+ * passes, in a sampled mini-batch alone; the update kernel of smaller models
+ * draws them itself).
  * bmlp_launch_count: kernels this handle has launched since creation (graph
  * replays count each node). */
 int bmlp_set_profiling(bmlp_t* h, int32_t every);

@@ -11,8 +11,8 @@
 // k % 64 of word k / 64, pad bits 0), i.e. bmlp_train / bmlp_predict input
 // for K_0 = K.
 //
-// k_expand_tc (D <= kTcMaxD, x aligned to 4 bytes): the product on the tensor cores, exact in 4-bit
-// operands.  A byte is four base-4 digits, x = d0 + 4 d1 + 16 d2 + 64 d3, and 0,
+// k_expand_tc (D <= kTcMaxD, x aligned to 4 bytes): the product on the tensor
+// cores, exact in 4-bit operands.  A byte is four base-4 digits, x = d0 + 4 d1 + 16 d2 + 64 d3, and 0,
 // 1, 2, 3 and +-1 are e2m1 values, so z is the sum of four e2m1 x e2m1 products
 // with block scales 1, 4, 16 and 64 (UE8M0 holds powers of two); every product
 // is an integer and |z| <= 255 D < 2^24, so the fp32 sums are exact in any
@@ -27,9 +27,9 @@
 //     are read from shared memory and never written again;
 //   - 8 epilogue warps read the sums (a lane per pattern), shift the sign bits
 //     into words and store them.
-// Bound: the MMAs, 4 x 128 clocks per chunk of a 128 x 256 tile.  60,000 x 784
-// -> 1024: 76 us (the dp4a kernel 804 us), of which the MMAs are 43; a chunk takes
-// 590 clocks where its MMAs take 512, a tile 2,200 more for its epilogue.
+// Bound: the producers, 560 to 590 clocks per chunk at any width; at 256 neurons
+// its MMAs take 512.  A tile takes 2,200 more for its epilogue.  60,000 x 784 ->
+// 1024: 70 us (the dp4a kernel 804), of which the MMAs are 43.
 // Every mbarrier wait is bounded like all others of the library; this entry
 // point has no handle, so an expiry leaves its tiles unwritten.
 //
