@@ -29,7 +29,8 @@
 //     into words and store them.
 // Bound: the producers, 560 to 590 clocks per chunk at any width; at 256 neurons
 // its MMAs take 512.  A tile takes 2,200 more for its epilogue.  60,000 x 784 ->
-// 1024: 70 us (the dp4a kernel 804), of which the MMAs are 43.
+// 1024: 70 us repeated, 76 with x from memory (the dp4a kernel 804), of which the MMAs
+// are 43.
 // Every mbarrier wait is bounded like all others of the library; this entry
 // point has no handle, so an expiry leaves its tiles unwritten.
 //
