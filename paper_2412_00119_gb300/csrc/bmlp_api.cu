@@ -357,6 +357,11 @@ int ensure_graph(bmlp_t* h) {
 // Train on n device-resident patterns.
 int run_steps(bmlp_t* h, const uint64_t* xd, const int32_t* yd, int64_t n, cudaStream_t st) {
   const int64_t steps = (n + h->bs - 1) / h->bs;
+  // a captured step would be replayed past the host's step count
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  CK(h, cudaStreamIsCapturing(st, &cap));
+  if (cap != cudaStreamCaptureStatusNone)
+    return fail(h, BMLP_ECUDA, "bmlp_train: operation not permitted when stream is capturing");
   h->launches += steps * (h->L + 2 + (h->updRing ? 1 : 0) + (h->group_mode == BMLP_GROUPS_RESHUFFLED ? 1 : 0));
   if (steps == 1 && h->tc && h->profEvery == 0) {
     // one mini-batch: launched directly, its inputs as kernel parameters

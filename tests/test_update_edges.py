@@ -3,6 +3,8 @@ oracle: rows of fewer blocks than a warp has lanes, several warps per row, short
 last blocks, every plane count, and the ring kernel of large models (more than
 20 M hidden weights)."""
 import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -96,3 +98,34 @@ def test_calls_of_one_batch(widths, group_mode, bs):
         assert np.array_equal(Wb, W.pack(np.where(ref.H(l).T > 0, 1, -1)))
         assert step == ref.step
     gpu.close()
+
+
+CAPTURE = """
+import sys
+import numpy as np, torch
+import workloads as W
+from paper_2412_00119_gb300 import bmlp as B
+n = int(sys.argv[1])
+gpu = B.BMLP((70, 40), 5, seed=3, bs=20)
+x = torch.from_numpy(W.random_packed(5, n, 70).view(np.int64)).cuda()
+y = torch.zeros(n, dtype=torch.int32, device="cuda")
+gpu.train(x, y)
+try:
+    with torch.cuda.graph(torch.cuda.CUDAGraph()):
+        try:
+            gpu.train(x, y)
+            print("accepted", flush=True)
+        except B.BmlpError:
+            print("refused", flush=True)
+except Exception:
+    pass
+"""
+
+
+# a training call is refused while its stream is captured, whatever its length (in
+# a process of its own: the failed capture stays with it)
+@pytest.mark.parametrize("n", [20, 45])
+def test_training_is_refused_under_capture(n):
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    run = subprocess.run([sys.executable, "-c", CAPTURE, str(n)], cwd=root, capture_output=True, text=True, timeout=300)
+    assert run.stdout.split() == ["refused"], run.stdout + run.stderr
