@@ -327,6 +327,9 @@ __device__ __forceinline__ void run_tile(TileIn T, const Place& pl, int pat, boo
         if (two) mbar_arrive(&sh->full[s[1]]);
       }
     }
+    // no copy outlives its thread: the early weights of a tile without patterns
+    // are read by nobody
+    cp_async_wait_all();
   } else {
     // ---------------- MMA issuer ----------------
     const bool lead = elect_one();

@@ -58,6 +58,15 @@ def test_rows_kernel_batches(bs):
     check((300, 96, 200), 255, 2 * bs + 1, bs, p_r0=3.0, gamma=[96, 8], group_mode=2)
 
 
+# short last mini-batches that leave pattern tiles of the forward passes empty, whose
+# CTAs have their first weights in flight when they learn it: one tile to all but
+# one, with and without a K split
+@pytest.mark.parametrize("widths,bs,n", [((70, 200, 130), 100, 101), ((300, 1024, 1024), 100, 117), ((1100, 2100, 257), 64, 65),
+                                         ((300, 300, 300, 300), 512, 904), ((2100, 4100, 128), 300, 301)])
+def test_empty_pattern_tiles(widths, bs, n):
+    check(widths, 255, n, bs)
+
+
 # more than 20 M weights: the ring kernel, whole rows and ragged ones
 @pytest.mark.parametrize("h_max,widths", [(255, (5000, 4500)), (13, (5000, 4500)), (127, (6160, 3600)),
                                           (1001, (2100, 10010))])
