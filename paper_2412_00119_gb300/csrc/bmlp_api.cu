@@ -511,8 +511,8 @@ int bmlp_create(const int32_t* widths, int32_t n_widths, int32_t classes, int16_
     return fail(nullptr, BMLP_EINVAL, "group_mode must be 0, 1 or 2");
   int max_K = 0;
   for (int l = 1; l <= L; ++l) max_K = std::max(max_K, (int)widths[l]);
-  if (group_mode != BMLP_GROUPS_CONTIGUOUS && max_K > 16384)
-    return fail(nullptr, BMLP_EINVAL, "random group membership needs every K_l <= 16384");
+  if (group_mode != BMLP_GROUPS_CONTIGUOUS && max_K > kMaxOrderK)
+    return fail(nullptr, BMLP_EINVAL, "random group membership needs every K_l <= %d", kMaxOrderK);
   std::vector<int> gam(L + 1, 0);
   for (int l = 1; l <= L; ++l) {
     const int g = hp.gamma ? hp.gamma[l - 1] : bmlp_gamma_rule(widths[l]);
@@ -652,7 +652,7 @@ int bmlp_create(const int32_t* widths, int32_t n_widths, int32_t classes, int16_
   if ((rc = upload_thresholds(h, 0)) != BMLP_OK) return bail(rc);
   // the partition of step 0 (the fixed one, or the first redrawn one)
   if (group_mode != BMLP_GROUPS_CONTIGUOUS &&
-      ((e = prepare_group_order(max_K)) != cudaSuccess ||
+      ((e = prepare_group_order()) != cudaSuccess ||
        (e = launch_group_order(L, max_K, false, 0, false, h->dP)) != cudaSuccess))
     return bail(cuda_fail(h, e, "group order"));
   if ((e = cudaDeviceSynchronize()) != cudaSuccess) return bail(cuda_fail(h, e, "init"));

@@ -217,7 +217,8 @@ struct ClsArgs {
 cudaError_t launch_cls_select(const ClsArgs& C, int max_K, cudaStream_t st, bool pdl);
 // Group order of every layer with a random partition (DevLayer::member /
 // group_of); redraw: keyed by the current step (else by step 0).
-cudaError_t prepare_group_order(int max_K);  // shared-memory attribute, once
+constexpr int kMaxOrderK = 16384;   // widest layer that may have a random partition
+cudaError_t prepare_group_order();  // shared-memory attribute
 cudaError_t launch_group_order(int L, int max_K, bool redraw, cudaStream_t st, bool pdl, const StepParams* P);
 // Reinforcement events of every neuron row of every layer for the current
 // step into DevLayer::EV (Alg. 3 l.5-12).

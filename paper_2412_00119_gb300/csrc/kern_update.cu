@@ -330,9 +330,10 @@ __global__ void __launch_bounds__(kOrderThreads) k_group_order(const StepParams*
 
 static size_t group_order_smem(int max_K) { return sizeof(uint4) * (size_t)((max_K + 3) / 4); }
 
-cudaError_t prepare_group_order(int max_K) {
+// The widest layer's for every handle: the attribute belongs to the kernel, not to a handle.
+cudaError_t prepare_group_order() {
   return cudaFuncSetAttribute(k_group_order, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)group_order_smem(max_K));
+                              (int)group_order_smem(kMaxOrderK));
 }
 
 cudaError_t launch_group_order(int L, int max_K, bool redraw, cudaStream_t st, bool pdl, const StepParams* P) {

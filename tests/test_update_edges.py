@@ -109,6 +109,32 @@ def test_calls_of_one_batch(widths, group_mode, bs):
     gpu.close()
 
 
+# redrawn groups of a wide model beside a narrower one made after it: in a call of one
+# mini-batch, in a longer one, and in both again
+def test_group_order_of_two_models():
+    widths, bs = (70, 2048, 64), 20
+    wide = B.BMLP(widths, 5, seed=9, bs=bs, group_mode=2)
+    ref = O.OracleModel(list(widths), 5, seed=9, bs=bs)
+    ref.set_group_mode(2)
+    narrow = B.BMLP((70, 64), 5, seed=9, bs=bs, group_mode=2)
+    sizes = [bs, 3 * bs, bs, 2 * bs]
+    xp = W.random_packed(6, sum(sizes), widths[0])
+    y = np.random.default_rng(6).integers(0, 5, sum(sizes)).astype(np.int32)
+    x, yd, xpm = torch.from_numpy(xp.view(np.int64)).to(DEV), torch.from_numpy(y).to(DEV), W.unpack(xp, widths[0])
+    a = 0
+    for m in sizes:
+        wide.train(x[a:a + m], yd[a:a + m])
+        narrow.train(x[a:a + m], yd[a:a + m])
+        ref.train(xpm[a:a + m], y[a:a + m])
+        a += m
+    for l in (1, 2):
+        H, _, _, _, step = wide.state(l)
+        assert np.array_equal(H.astype(np.int32), ref.H(l).T)
+        assert step == ref.step
+    wide.close()
+    narrow.close()
+
+
 CAPTURE = """
 import sys
 import numpy as np, torch
