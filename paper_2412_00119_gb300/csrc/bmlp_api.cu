@@ -363,8 +363,13 @@ int run_steps(bmlp_t* h, const uint64_t* xd, const int32_t* yd, int64_t n, cudaS
   if (cap != cudaStreamCaptureStatusNone)
     return fail(h, BMLP_ECUDA, "bmlp_train: operation not permitted when stream is capturing");
   h->launches += steps * (h->L + 2 + (h->updRing ? 1 : 0) + (h->group_mode == BMLP_GROUPS_RESHUFFLED ? 1 : 0));
-  if (steps == 1 && h->tc && h->profEvery == 0) {
-    // one mini-batch: launched directly, its inputs as kernel parameters
+  if (steps == 1 && h->tc && h->profEvery == 0 && (!h->updRing || h->evLayer == 1)) {
+    // One mini-batch: launched directly, its inputs as kernel parameters.  Not
+    // where the draws go beside the later passes: in a direct step they follow the
+    // selection.  A call (us) among others, direct against the one-step graph:
+    // 784-256 12.0 / 16.4, 5120-5120 45.3 / 48.9, 8192-8192 52.5 / 54.8 (alone 59.0 /
+    // 56.8 and 66.8 / 63.4); with later draws 3072-2900x3 53.7 / 49.0, 3072-4096x4
+    // 72.4 / 65.7 (alone 67.6 / 57.7 and 86.4 / 74.2).
     const int rc = enqueue_step(h, st, kStepDirect, OneBatch{xd, yd, n});
     h->t_host += 1;
     return rc;

@@ -80,10 +80,11 @@ def test_ring_kernel_steps(widths):
     check(widths, 255, 18 * 10, 10)
 
 
-# calls of one mini-batch (their kernels get the inputs as parameters), whole and
-# short ones, mixed with a longer call and an evaluation
+# calls of one mini-batch (their kernels get the inputs as parameters, but for models
+# whose draws go beside the later passes), whole and short ones, mixed with a longer
+# call and an evaluation
 @pytest.mark.parametrize("widths,group_mode,bs", [((70, 40), 0, 16), ((200, 96, 130), 2, 30), ((130, 64, 64, 64), 1, 100),
-                                                  ((5000, 4500), 0, 20), ((3000, 4096, 4096), 2, 150)])
+                                                  ((5000, 4500), 0, 20), ((3000, 4096, 4096), 2, 150), ((300, 8000, 7400), 0, 20)])
 def test_calls_of_one_batch(widths, group_mode, bs):
     gpu = B.BMLP(widths, 5, seed=3, bs=bs, group_mode=group_mode)
     ref = O.OracleModel(list(widths), 5, seed=3, bs=bs)
