@@ -327,8 +327,8 @@ int64_t bmlp_launch_count(const bmlp_t* h);
 int bmlp_update_stats(bmlp_t* h, int64_t* rows_out, int64_t* streamed_out, int64_t* bytes_out,
                       int32_t reset);
 
-/* Failure injection for the allocation paths (no counterpart in the paper;
- * it tests the library's clean-up without a GPU fault).  After
+/* Failure injection for the allocation and launch paths (no counterpart in the
+ * paper; it tests the library's clean-up without a GPU fault).  After
  * bmlp_debug_fail_alloc(n), n >= 1, the n-th memory allocation the library
  * makes from then on -- counting every cudaMalloc of a device buffer and the
  * pinned host block of bmlp_create, in any handle of the process -- fails as
@@ -337,9 +337,14 @@ int bmlp_update_stats(bmlp_t* h, int64_t* rows_out, int64_t* streamed_out, int64
  * disarms itself.  n = 0 disarms it.  BMLP_EINVAL for n < 0.
  * bmlp_debug_alloc_stats: the number of allocations the library holds now,
  * over every live handle of the process, and their bytes (either output may
- * be NULL); a failed bmlp_create leaves both where they were.  Host only;
- * neither call touches the device. */
+ * be NULL); a failed bmlp_create leaves both where they were.
+ * bmlp_debug_fail_launch(n): the same for the n-th training mini-batch that is
+ * launched kernel by kernel from then on (a call of one mini-batch, or one that
+ * bmlp_set_profiling samples): its launch fails after the forward passes and
+ * the call returns BMLP_ECUDA ("... (injected)"), with that mini-batch trained
+ * on nothing.  Host only; none of these calls touches the device. */
 int bmlp_debug_fail_alloc(int64_t nth);
+int bmlp_debug_fail_launch(int64_t nth);
 int bmlp_debug_alloc_stats(int64_t* live_allocs, int64_t* live_bytes);
 
 /* Peak rate of one contraction unit on the current device (the engine

@@ -85,6 +85,7 @@ SIGNATURES = [
     ("bmlp_debug_wait_probe", C.c_int, [_vp, C.c_int32, C.c_double]),
     ("bmlp_engine_peak", C.c_int, [C.c_int32, C.c_int64, _f64p, _f64p]),
     ("bmlp_debug_fail_alloc", C.c_int, [C.c_int64]),
+    ("bmlp_debug_fail_launch", C.c_int, [C.c_int64]),
     ("bmlp_debug_alloc_stats", C.c_int, [_i64p, _i64p]),
     ("bmlp_layer_forward_engine", C.c_int, [_vp, C.c_int32, C.c_int32, _vp, C.c_int64, _vp, _vp]),
 ]
@@ -251,6 +252,12 @@ def bmlp_layer_forward_engine(h, layer, engine, a_in, a_out, n=None, stream=None
 def bmlp_debug_fail_alloc(nth):
     """Arm (nth >= 1) or disarm (0) the one-shot failure of the nth allocation."""
     _check(lib().bmlp_debug_fail_alloc(int(nth)), None)
+
+
+def bmlp_debug_fail_launch(nth):
+    """Arm (nth >= 1) or disarm (0) the one-shot failure of the nth training
+    mini-batch that is launched kernel by kernel."""
+    _check(lib().bmlp_debug_fail_launch(int(nth)), None)
 
 
 def bmlp_debug_alloc_stats():

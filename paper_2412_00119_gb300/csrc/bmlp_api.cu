@@ -33,18 +33,27 @@ namespace {
 thread_local std::string g_create_error;
 
 // Process-wide accounting of the memory the library holds (every handle's
-// device buffers and pinned host block), and the one-shot injected failure of
-// the n-th allocation from the moment bmlp_debug_fail_alloc armed it.
+// device buffers and pinned host block).
 std::atomic<int64_t> g_live_allocs{0}, g_live_bytes{0};
-std::atomic<int64_t> g_fail_at{0}, g_alloc_seq{0};
 
-// True when this allocation is the armed one (the injection then disarms).
-bool injected_alloc_failure() {
-  if (g_fail_at.load() <= 0) return false;
-  const int64_t seq = ++g_alloc_seq;
-  int64_t at = g_fail_at.load();
-  return seq == at && g_fail_at.compare_exchange_strong(at, 0);
-}
+// A one-shot injected failure of the n-th event from the moment it was armed.
+struct Injection {
+  std::atomic<int64_t> fail_at{0}, seq{0};
+  void arm(int64_t nth) {
+    fail_at.store(0);
+    seq.store(0);
+    fail_at.store(nth);
+  }
+  // True when this event is the armed one (the injection then disarms).
+  bool fires() {
+    if (fail_at.load() <= 0) return false;
+    const int64_t n = ++seq;
+    int64_t at = fail_at.load();
+    return n == at && fail_at.compare_exchange_strong(at, 0);
+  }
+};
+Injection g_fail_alloc, g_fail_launch;
+bool injected_alloc_failure() { return g_fail_alloc.fires(); }
 
 // NVTX range for the lifetime of an entry point call.
 struct TraceRange {
@@ -289,6 +298,7 @@ int enqueue_step(bmlp_t* h, cudaStream_t st, StepForm form, const OneBatch& one 
     // this step's partition (keyed by the step counter) before the selection
     CK(h, launch_group_order(h->L, h->max_K, true, st, pdl && h->tc, h->dP));
   }
+  if (!fork && g_fail_launch.fires()) return fail(h, BMLP_ECUDA, "kernel launch failed (injected)");
   prof_begin(h, kProfCls, st);
   // inside the step graph each kernel after the first is launched as a
   // programmatic dependent of the one before it (launch and prologue overlap
@@ -362,7 +372,12 @@ int run_steps(bmlp_t* h, const uint64_t* xd, const int32_t* yd, int64_t n, cudaS
   CK(h, cudaStreamIsCapturing(st, &cap));
   if (cap != cudaStreamCaptureStatusNone)
     return fail(h, BMLP_ECUDA, "bmlp_train: operation not permitted when stream is capturing");
-  h->launches += steps * (h->L + 2 + (h->updRing ? 1 : 0) + (h->group_mode == BMLP_GROUPS_RESHUFFLED ? 1 : 0));
+  // the host's counts follow what is in the stream, also when a launch fails
+  const int64_t kernels = h->L + 2 + (h->updRing ? 1 : 0) + (h->group_mode == BMLP_GROUPS_RESHUFFLED ? 1 : 0);
+  auto enqueued = [&](int64_t n_steps) {
+    h->t_host += n_steps;
+    h->launches += n_steps * kernels;
+  };
   if (steps == 1 && h->tc && h->profEvery == 0 && (!h->updRing || h->evLayer == 1)) {
     // One mini-batch: launched directly, its inputs as kernel parameters.  Not
     // where the draws go beside the later passes: in a direct step they follow the
@@ -371,7 +386,7 @@ int run_steps(bmlp_t* h, const uint64_t* xd, const int32_t* yd, int64_t n, cudaS
     // 56.8 and 66.8 / 63.4); with later draws 3072-2900x3 53.7 / 49.0, 3072-4096x4
     // 72.4 / 65.7 (alone 67.6 / 57.7 and 86.4 / 74.2).
     const int rc = enqueue_step(h, st, kStepDirect, OneBatch{xd, yd, n});
-    h->t_host += 1;
+    if (rc == BMLP_OK) enqueued(1);
     return rc;
   }
   h->hp.x = xd;
@@ -384,26 +399,27 @@ int run_steps(bmlp_t* h, const uint64_t* xd, const int32_t* yd, int64_t n, cudaS
     int rc = ensure_graph(h);
     if (rc != BMLP_OK) return rc;
   }
-  auto sampled = [&](int64_t s) {
-    return h->profEvery > 0 && ((h->t_host + s) % h->profEvery) == 0;
+  auto sampled = [&](int64_t ahead) {
+    return h->profEvery > 0 && ((h->t_host + ahead) % h->profEvery) == 0;
   };
   for (int64_t s = 0; s < steps;) {
     // sampled mini-batches are launched kernel by kernel between CUDA events;
     // the others as graphs of kGraphSteps steps, or of one step
-    h->profiling = sampled(s);
+    h->profiling = sampled(0);
+    int64_t took = 1;
     if (h->profiling) {
       int rc = enqueue_step(h, st, kStepPlain);
       if (rc != BMLP_OK) return rc;
-      ++s;
-      continue;
+    } else {
+      bool multi = s + kGraphSteps <= steps;
+      for (int64_t i = 1; multi && i < kGraphSteps; ++i) multi = !sampled(i);
+      CK(h, cudaGraphLaunch(multi ? h->multiExec : h->stepExec, st));
+      if (multi) took = kGraphSteps;
     }
-    bool multi = s + kGraphSteps <= steps;
-    for (int64_t i = 1; multi && i < kGraphSteps; ++i) multi = !sampled(s + i);
-    CK(h, cudaGraphLaunch(multi ? h->multiExec : h->stepExec, st));
-    s += multi ? kGraphSteps : 1;
+    s += took;
+    enqueued(took);
   }
   h->profiling = h->profEvery > 0;
-  h->t_host += steps;
   return BMLP_OK;
 }
 
@@ -1086,9 +1102,13 @@ int bmlp_debug_wait_probe(bmlp_t* h, int32_t arrive, double seconds) {
 
 int bmlp_debug_fail_alloc(int64_t nth) {
   if (nth < 0) return fail(nullptr, BMLP_EINVAL, "nth must be >= 0");
-  g_fail_at.store(0);
-  g_alloc_seq.store(0);
-  g_fail_at.store(nth);
+  g_fail_alloc.arm(nth);
+  return BMLP_OK;
+}
+
+int bmlp_debug_fail_launch(int64_t nth) {
+  if (nth < 0) return fail(nullptr, BMLP_EINVAL, "nth must be >= 0");
+  g_fail_launch.arm(nth);
   return BMLP_OK;
 }
 

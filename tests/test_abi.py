@@ -145,3 +145,5 @@ def test_alloc_injection_host_side():
         B.bmlp_debug_fail_alloc(-1)
     B.bmlp_debug_fail_alloc(3)
     B.bmlp_debug_fail_alloc(0)
+    with pytest.raises(B.BmlpError):
+        B.bmlp_debug_fail_launch(-1)

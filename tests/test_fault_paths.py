@@ -5,6 +5,9 @@ hang is involved:
     allocation point of bmlp_create, and in the host-buffer staging of
     bmlp_train: BMLP_ENOMEM, nothing leaked (bmlp_debug_alloc_stats), the
     handle (when there is one) still trains bit for bit like the oracle;
+  * a kernel launch that fails (injected: bmlp_debug_fail_launch) in a training
+    mini-batch: BMLP_ECUDA, no weight changes, and the host's step count stays
+    the device's, so that sampling and training go on at the right step;
   * an expired bounded device wait left pending across a training step (the
     wait probe with nothing arriving): that step changes neither H nor W, the
     error is reported by the next synchronising call, and training then
@@ -34,6 +37,7 @@ def _setup():
     B.lib()
     yield
     B.bmlp_debug_fail_alloc(0)
+    B.bmlp_debug_fail_launch(0)
 
 
 def _allocations_of_create(widths, classes, **kw):
@@ -84,6 +88,45 @@ def test_staging_allocation_failure_leaves_handle_usable():
     er = ref.train(tr.pm1(), tr.y, epoch_end=True)
     assert eg == er
     assert_same_state(gpu, ref, "after the retried call")
+    gpu.close()
+
+
+def test_launch_failure_leaves_the_step_count():
+    widths, c, bs = (200, 130, 70), 10, 50
+    cfg = W.small_config(widths, c, 400, 0, teacher_hidden=16)
+    tr = W.make_split(cfg, "train")
+    gpu = B.BMLP(widths, c, seed=8, bs=bs, gamma=[13, 7])
+    ref = O.OracleModel(list(widths), c, seed=8, bs=bs, gamma=[13, 7])
+    x, y, xo = dev_x(tr.xp), dev_y(tr.y), tr.pm1()
+
+    def fails(a, b, nth):
+        B.bmlp_debug_fail_launch(nth)
+        with pytest.raises(B.BmlpError) as ei:
+            gpu.train(x[a:b], y[a:b])
+        assert ei.value.code == B.BMLP_ECUDA and "injected" in str(ei.value)
+
+    def sampled():   # mini-batches sampled since the last reset
+        n = B.bmlp_get_profile(gpu.h)["update"][0]
+        B.bmlp_reset_profile(gpu.h)
+        return n
+
+    launches = B.bmlp_launch_count(gpu.h)
+    fails(0, bs, 1)   # a call of one mini-batch
+    assert B.bmlp_launch_count(gpu.h) == launches
+    assert_same_state(gpu, ref, "after the failed call")
+    B.bmlp_set_profiling(gpu.h, 2)
+    gpu.train(x[:bs], y[:bs])   # step 0
+    ref.train(xo[:bs], tr.y[:bs])
+    assert sampled() == 1
+    fails(bs, 4 * bs, 1)        # steps 1, and 2 (sampled), which fails
+    ref.train(xo[bs:2 * bs], tr.y[bs:2 * bs])
+    assert_same_state(gpu, ref, "after the call that failed at its second mini-batch")
+    B.bmlp_set_profiling(gpu.h, 3)
+    B.bmlp_reset_profile(gpu.h)
+    gpu.train(x[2 * bs:6 * bs], y[2 * bs:6 * bs])   # steps 2 .. 5: 3 is sampled
+    ref.train(xo[2 * bs:6 * bs], tr.y[2 * bs:6 * bs])
+    assert sampled() == 1
+    assert_same_state(gpu, ref, "after training on")
     gpu.close()
 
 
