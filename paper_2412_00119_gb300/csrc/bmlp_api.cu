@@ -367,11 +367,6 @@ int ensure_graph(bmlp_t* h) {
 // Train on n device-resident patterns.
 int run_steps(bmlp_t* h, const uint64_t* xd, const int32_t* yd, int64_t n, cudaStream_t st) {
   const int64_t steps = (n + h->bs - 1) / h->bs;
-  // a captured step would be replayed past the host's step count
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  CK(h, cudaStreamIsCapturing(st, &cap));
-  if (cap != cudaStreamCaptureStatusNone)
-    return fail(h, BMLP_ECUDA, "bmlp_train: operation not permitted when stream is capturing");
   // the host's counts follow what is in the stream, also when a launch fails
   const int64_t kernels = h->L + 2 + (h->updRing ? 1 : 0) + (h->group_mode == BMLP_GROUPS_RESHUFFLED ? 1 : 0);
   auto enqueued = [&](int64_t n_steps) {
@@ -713,6 +708,15 @@ int bmlp_train(bmlp_t* h, const uint64_t* x, const int32_t* labels, int64_t n, u
   if ((n + h->bs - 1) / h->bs > 0xffffffffLL) return fail(h, BMLP_EINVAL, "n too large");
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const bool want_count = n_errors_out != nullptr;
+  const bool epoch_end = (flags & BMLP_EPOCH_END) != 0;
+  if (n > 0 || want_count || epoch_end) {
+    // before any copy: a captured step would be replayed past the host's step
+    // count, and the counts are read here
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(h, cudaStreamIsCapturing(st, &cap));
+    if (cap != cudaStreamCaptureStatusNone)
+      return fail(h, BMLP_ECUDA, "bmlp_train: operation not permitted when stream is capturing");
+  }
   if (want_count) {
     CK(h, cudaMemcpyAsync(&h->hostPinned[0], &h->dCtrl->err, sizeof(unsigned long long),
                           cudaMemcpyDeviceToHost, st));
@@ -742,7 +746,6 @@ int bmlp_train(bmlp_t* h, const uint64_t* x, const int32_t* labels, int64_t n, u
     if (rc != BMLP_OK) return rc;
   }
   h->epoch_n += n;
-  const bool epoch_end = (flags & BMLP_EPOCH_END) != 0;
   if (want_count || epoch_end) {
     CK(h, cudaMemcpyAsync(&h->hostPinned[1], &h->dCtrl->err, sizeof(unsigned long long),
                           cudaMemcpyDeviceToHost, st));

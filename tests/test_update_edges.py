@@ -137,31 +137,43 @@ def test_group_order_of_two_models():
 
 
 CAPTURE = """
-import sys
+import ctypes, sys
 import numpy as np, torch
 import workloads as W
 from paper_2412_00119_gb300 import bmlp as B
-n = int(sys.argv[1])
+n, host, count = int(sys.argv[1]), sys.argv[2] == "host", sys.argv[3] == "count"
+rt = ctypes.CDLL("libcudart.so." + torch.version.cuda.split(".")[0])
 gpu = B.BMLP((70, 40), 5, seed=3, bs=20)
-x = torch.from_numpy(W.random_packed(5, n, 70).view(np.int64)).cuda()
-y = torch.zeros(n, dtype=torch.int32, device="cuda")
+x, y = W.random_packed(5, n, 70), np.zeros(n, np.int32)
+if not host:
+    x, y = torch.from_numpy(x.view(np.int64)).cuda(), torch.from_numpy(y).cuda()
 gpu.train(x, y)
+torch.cuda.synchronize()
+s = torch.cuda.Stream()
+st, g, nodes = ctypes.c_void_p(s.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
+assert rt.cudaStreamBeginCapture(st, 0) == 0
 try:
-    with torch.cuda.graph(torch.cuda.CUDAGraph()):
-        try:
-            gpu.train(x, y)
-            print("accepted", flush=True)
-        except B.BmlpError:
-            print("refused", flush=True)
-except Exception:
-    pass
+    gpu.train(x, y, count_errors=count, stream=s)
+    print("accepted")
+except B.BmlpError as e:
+    print("refused" if e.code == B.BMLP_ECUDA else e)
+# the capture is whole and empty: nothing had gone into the stream
+assert rt.cudaStreamEndCapture(st, ctypes.byref(g)) == 0
+assert rt.cudaGraphGetNodes(g, None, ctypes.byref(nodes)) == 0
+print(nodes.value)
+gpu.train(x, y)
+print(gpu.state(1)[4] == 2 * -(-n // 20))
 """
 
 
-# a training call is refused while its stream is captured, whatever its length (in
-# a process of its own: the failed capture stays with it)
+# a training call is refused while its stream is captured, before it touches the
+# stream, whatever its length, its inputs' place and its results (in a process of its
+# own)
+@pytest.mark.parametrize("count", ["count", "none"])
+@pytest.mark.parametrize("place", ["device", "host"])
 @pytest.mark.parametrize("n", [20, 45])
-def test_training_is_refused_under_capture(n):
+def test_training_is_refused_under_capture(n, place, count):
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-    run = subprocess.run([sys.executable, "-c", CAPTURE, str(n)], cwd=root, capture_output=True, text=True, timeout=300)
-    assert run.stdout.split() == ["refused"], run.stdout + run.stderr
+    run = subprocess.run([sys.executable, "-c", CAPTURE, str(n), place, count], cwd=root, capture_output=True, text=True,
+                         timeout=300)
+    assert run.stdout.split() == ["refused", "0", "True"], run.stdout + run.stderr
