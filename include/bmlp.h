@@ -208,11 +208,19 @@ int bmlp_expand_weights(uint64_t seed, int32_t K, int32_t D, uint64_t* E_out, vo
  *   E: device, K x ceil(D/64) words as written by bmlp_expand_weights (any
  *      +-1 matrix in that layout; pad bits ignored), 8-byte aligned.
  *   out: device, n x ceil(K/64) words, 8-byte aligned, caller-owned.
- * No handle (errors: bmlp_last_error(NULL)); asynchronous on cuda_stream.
+ * No handle (errors: bmlp_last_error(NULL)); asynchronous on cuda_stream.  A
+ * bounded device-side wait that expires costs time only: the affected tiles are
+ * computed again without waits, so the output is always whole.
  * BMLP_EINVAL for n < 0, K < 1, D < 1, D > 2^23 (the int32 sum bound),
  * NULL, host or misaligned pointers; BMLP_ECUDA if the launch fails. */
 int bmlp_expand_sign(const uint8_t* x, int64_t n, int32_t D, const uint64_t* E, int32_t K,
                      uint64_t* out, void* cuda_stream);
+
+/* bmlp_expand_sign with that path forced, for tests: every CTA of the
+ * tensor-core kernel takes its device-side wait for its tile number
+ * expired_tile (0, 1, ..) as expired.  expired_tile < 0: none. */
+int bmlp_debug_expand_sign(const uint8_t* x, int64_t n, int32_t D, const uint64_t* E, int32_t K,
+                           uint64_t* out, void* cuda_stream, int64_t expired_tile);
 
 /* One layer of forward-only evaluation (Sec. 3.1; Alg. 1 l.8-9):
  * a_out = sign(a_in W_l), sign(0) = +1, for n packed rows.  a_in: n rows of

@@ -82,6 +82,7 @@ SIGNATURES = [
     ("bmlp_binarize_median", C.c_int, [_vp, C.c_int64, C.c_int32, _vp, _vp]),
     ("bmlp_expand_weights", C.c_int, [C.c_uint64, C.c_int32, C.c_int32, _vp, _vp]),
     ("bmlp_expand_sign", C.c_int, [_vp, C.c_int64, C.c_int32, _vp, C.c_int32, _vp, _vp]),
+    ("bmlp_debug_expand_sign", C.c_int, [_vp, C.c_int64, C.c_int32, _vp, C.c_int32, _vp, _vp, C.c_int64]),
     ("bmlp_debug_wait_probe", C.c_int, [_vp, C.c_int32, C.c_double]),
     ("bmlp_engine_peak", C.c_int, [C.c_int32, C.c_int64, _f64p, _f64p]),
     ("bmlp_debug_fail_alloc", C.c_int, [C.c_int64]),
@@ -226,6 +227,13 @@ def bmlp_expand_sign(x, E, K, out, stream=None):
     """Expansion layer: n x D uint8 patterns (device) -> packed sign(x E^T)."""
     n, D = x.shape
     _check(lib().bmlp_expand_sign(_ptr(x), n, D, _ptr(E), K, _ptr(out), _stream(stream)), None)
+
+
+def bmlp_debug_expand_sign(x, E, K, out, expired_tile, stream=None):
+    """bmlp_expand_sign with every CTA's wait for its tile expired_tile taken as
+    expired."""
+    n, D = x.shape
+    _check(lib().bmlp_debug_expand_sign(_ptr(x), n, D, _ptr(E), K, _ptr(out), _stream(stream), int(expired_tile)), None)
 
 
 def bmlp_debug_wait_probe(h, arrive, seconds=0.05, leave_pending=False):

@@ -907,6 +907,11 @@ int bmlp_expand_weights(uint64_t seed, int32_t K, int32_t D, uint64_t* E_out, vo
 
 int bmlp_expand_sign(const uint8_t* x, int64_t n, int32_t D, const uint64_t* E, int32_t K,
                      uint64_t* out, void* cuda_stream) {
+  return bmlp_debug_expand_sign(x, n, D, E, K, out, cuda_stream, -1);
+}
+
+int bmlp_debug_expand_sign(const uint8_t* x, int64_t n, int32_t D, const uint64_t* E, int32_t K,
+                           uint64_t* out, void* cuda_stream, int64_t expired_tile) {
   TraceRange trace("bmlp_expand_sign");
   if (n < 0 || K < 1 || D < 1 || D > (1 << 23))
     return fail(nullptr, BMLP_EINVAL, "bmlp_expand_sign: n < 0, K < 1, D < 1 or D > 2^23");
@@ -915,7 +920,7 @@ int bmlp_expand_sign(const uint8_t* x, int64_t n, int32_t D, const uint64_t* E, 
     return fail(nullptr, BMLP_EINVAL, "bmlp_expand_sign: x, E and out must be device pointers");
   if ((reinterpret_cast<uintptr_t>(E) & 7) || (reinterpret_cast<uintptr_t>(out) & 7))
     return fail(nullptr, BMLP_EINVAL, "bmlp_expand_sign: misaligned E or out");
-  const cudaError_t e = launch_expand_sign(x, n, D, E, K, out, static_cast<cudaStream_t>(cuda_stream));
+  const cudaError_t e = launch_expand_sign(x, n, D, E, K, out, static_cast<cudaStream_t>(cuda_stream), expired_tile);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "k_expand_sign");
   return BMLP_OK;
 }

@@ -273,8 +273,10 @@ void launch_binarize_median(const float* x, int64_t n, int K, int nw, uint64_t* 
 // Expansion layer for uint8 inputs: E (K x ceil(D/64) words) from the
 // expansion-weight stream, and out = packed sign(x E^T) (n x ceil(K/64)).
 void launch_expand_weights(uint64_t seed, int K, int D, uint64_t* E, cudaStream_t st);
+// fail_tile >= 0: the tensor-core kernel's CTAs take their wait for the tile of
+// this number as expired.
 cudaError_t launch_expand_sign(const uint8_t* x, int64_t n, int D, const uint64_t* E, int K,
-                               uint64_t* out, cudaStream_t st);
+                               uint64_t* out, cudaStream_t st, int64_t fail_tile = -1);
 // SMs of the current device (looked up once).
 int sm_count();
 // Tensor-core forward for evaluation on large batches: A (M x nw_in) against W

@@ -31,8 +31,9 @@
 // its MMAs take 512.  A tile takes 2,200 more for its epilogue.  60,000 x 784 ->
 // 1024: 70 us repeated, 76 with x from memory (the dp4a kernel 804), of which the MMAs
 // are 43.
-// Every mbarrier wait is bounded like all others of the library; this entry
-// point has no handle, so an expiry leaves its tiles unwritten.
+// Every mbarrier wait is bounded like all others of the library.  This entry
+// point has no handle that could report an expiry, so a CTA whose waits gave up
+// writes its tiles again by a plain loop (expand_plain): the output is whole.
 //
 // k_expand_sign (the rest): a 128-pattern x 128-neuron tile per CTA of 256 threads, the
 // inputs in chunks of 64 (one word of E per neuron): the chunk's bytes of x
@@ -186,6 +187,7 @@ constexpr int kXMma = kXProdWarps, kXLoad0 = kXMma + 1, kXEpi0 = kXLoad0 + kXLoa
 constexpr int kXTcThreads = 32 * (kXEpi0 + kXEpiWarps);
 constexpr int kXSfA = kXMaxN, kXSfB = kXSfA + 4 * 16, kXStageCol = kXSfB + 16;
 static_assert(kXStageCol + 32 * kXStages <= 512, "TMEM budget");
+constexpr uint32_t kNoTile = 0xFFFFFFFFu;
 constexpr int kXWeightBytes = 4 * kXMaxN * 128;   // 4 blocks of 256 inputs x 256 neurons, and the like
 constexpr int kTcMaxD = 4608;                     // 18 blocks of 256 inputs x 64 neurons
 
@@ -193,8 +195,9 @@ struct __align__(8) XShared {
   unsigned long long piece_full[kXPieces], piece_empty[kXPieces];
   unsigned long long full[kXStages], empty[kXStages];
   unsigned long long done, drained;
+  unsigned long long left;   // the MMAs of an issuer that gave up completed
   uint32_t tmem_base;
-  int failed;
+  int failed, left_failed;
 };
 constexpr size_t kXSmem = 1024 + 18 * 64 * 128 + kXPieces * kXPieceBytes + sizeof(XShared);
 static_assert(18 * 64 * 128 >= kXWeightBytes, "the weight buffer holds every choice of tile");
@@ -224,15 +227,48 @@ __device__ __forceinline__ uint32_t weight_nibbles(uint32_t byte) {
   return 0x22222222u | even | (odd << 4);
 }
 
+// The tiles of this CTA without the tensor cores, barriers or shared memory, by one
+// warp (only that one looks for a failure: a check by every warp at the end of the
+// kernel cost small calls 0.2 to 0.4 us): a 32-bit word of the output per lane
+// and turn.
+__device__ __noinline__ void expand_plain(const uint8_t* x, int64_t n, int D, const uint64_t* E, int K, int nwD,
+                                          uint64_t* out, int nwK, int nb) {
+  const int words = nb / 32;
+#pragma unroll 1
+  for (int64_t t = blockIdx.y; t * XM < n; t += gridDim.y) {
+#pragma unroll 1
+    for (int i = threadIdx.x & 31; i < XM * words; i += 32) {
+      const int64_t m = t * XM + i / words;
+      const int nn = (int)blockIdx.x * nb + 32 * (i % words);
+      if (m >= n || (nn >> 5) >= 2 * nwK) continue;
+      uint32_t word = 0u;
+#pragma unroll 1
+      for (int j = 0; j < 32 && nn + j < K; ++j) {
+        const uint64_t* e = E + (int64_t)(nn + j) * nwD;
+        int z = 0;
+#pragma unroll 1
+        for (int c = 0; c < D; ++c) {
+          const int v = x[m * D + c];
+          z += (e[c >> 6] >> (c & 63) & 1u) != 0u ? v : -v;
+        }
+        word |= z >= 0 ? 1u << j : 0u;
+      }
+      reinterpret_cast<uint32_t*>(out + m * nwK)[nn >> 5] = word;
+    }
+  }
+}
+
 // kBytes: 16 or 4, the copies that every row of x allows, or 1: rows that start at
 // any byte of an x aligned to words.  Those are copied as the words that hold
 // them, zeros past the row's end, and shifted by the producers: 600 x 70 -> 1024
 // 7.3 us, 20,000 x 785 -> 1024 53 (byte loads in the loaders 16.5 and 100, the dp4a
 // kernel 12.4 and 357).
+// fail_tile: the wait for the sums of each CTA's tile of this number is taken as
+// expired (tests; kNoTile: none).
 template <int kBytes>
 __global__ void __launch_bounds__(kXTcThreads, 1)
     k_expand_tc(const uint8_t* __restrict__ x, int64_t n, int D, const uint64_t* __restrict__ E, int K, int nwD,
-                uint64_t* __restrict__ out, int nwK, int nb) {
+                uint64_t* __restrict__ out, int nwK, int nb, uint32_t fail_tile) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -255,7 +291,8 @@ __global__ void __launch_bounds__(kXTcThreads, 1)
     }
     mbar_init(&sh->done, 1);
     mbar_init(&sh->drained, kXEpiWarps);
-    sh->failed = 0;
+    mbar_init(&sh->left, 1);
+    sh->failed = sh->left_failed = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == kXMma) {
@@ -446,6 +483,12 @@ __global__ void __launch_bounds__(kXTcThreads, 1)
       if (ok && lead) mma_commit(&sh->done);
       __syncwarp();
     }
+    if (!ok && lead) {
+      // no MMA outlives its operands and its tensor memory
+      mma_commit(&sh->left);
+      mbar_wait(&sh->left, 0, &sh->left_failed);
+    }
+    __syncwarp();
   } else if (warp >= kXEpi0) {
     // ---------------- epilogue ----------------
     const int sub = warp & 3, half = (warp - kXEpi0) >> 2;
@@ -455,6 +498,10 @@ __global__ void __launch_bounds__(kXTcThreads, 1)
 #pragma unroll 1
     for (int64_t t = blockIdx.y; t < tiles; t += gridDim.y, ++tile) {
       if (!__all_sync(0xffffffffu, mbar_wait(&sh->done, tile & 1u, failed))) break;
+      if (tile == fail_tile) {
+        *failed = 1;
+        break;
+      }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       uint32_t word[4] = {0u, 0u, 0u, 0u};
       sign_words<4>(word, tmem + ((uint32_t)(32 * sub) << 16) + (uint32_t)(32 * first), words, 0.0f);
@@ -478,13 +525,16 @@ __global__ void __launch_bounds__(kXTcThreads, 1)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (warp == kXMma)
+  if (warp == kXMma) {
+    const bool redo = *failed != 0;
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    if (redo) expand_plain(x, n, D, E, K, nwD, out, nwK, nb);
+  }
 }
 
 template <int kBytes>
 cudaError_t launch_expand_tc(const uint8_t* x, int64_t n, int D, const uint64_t* E, int K, uint64_t* out,
-                             cudaStream_t st) {
+                             cudaStream_t st, uint32_t fail_tile) {
   const int blocks = (D + kXPiece - 1) / kXPiece;   // of 256 inputs
   const int64_t tiles = (n + XM - 1) / XM;
   const int sms = sm_count();
@@ -509,7 +559,7 @@ cudaError_t launch_expand_tc(const uint8_t* x, int64_t n, int D, const uint64_t*
                                              (int)kXSmem);
   if (e != cudaSuccess) return e;
   k_expand_tc<kBytes><<<dim3(nt, (unsigned)gy), kXTcThreads, kXSmem, st>>>(x, n, D, E, K, (D + 63) / 64, out,
-                                                                          (K + 63) / 64, nb);
+                                                                          (K + 63) / 64, nb, fail_tile);
   return cudaGetLastError();
 }
 
@@ -545,13 +595,14 @@ void launch_expand_weights(uint64_t seed, int K, int D, uint64_t* E, cudaStream_
 }
 
 cudaError_t launch_expand_sign(const uint8_t* x, int64_t n, int D, const uint64_t* E, int K, uint64_t* out,
-                               cudaStream_t st) {
+                               cudaStream_t st, int64_t fail_tile) {
   const int nwD = (D + 63) / 64, nwK = (K + 63) / 64;
+  const uint32_t ft = fail_tile < 0 ? kNoTile : (uint32_t)fail_tile;
   if (D <= kTcMaxD && reinterpret_cast<uintptr_t>(x) % 4 == 0) {
     const uintptr_t a = reinterpret_cast<uintptr_t>(x) | (uintptr_t)(uint32_t)D;
-    return (a & 15) == 0 ? launch_expand_tc<16>(x, n, D, E, K, out, st)
-                         : ((a & 3) == 0 ? launch_expand_tc<4>(x, n, D, E, K, out, st)
-                                         : launch_expand_tc<1>(x, n, D, E, K, out, st));
+    return (a & 15) == 0 ? launch_expand_tc<16>(x, n, D, E, K, out, st, ft)
+                         : ((a & 3) == 0 ? launch_expand_tc<4>(x, n, D, E, K, out, st, ft)
+                                         : launch_expand_tc<1>(x, n, D, E, K, out, st, ft));
   }
   const unsigned ntiles = (unsigned)((K + kXN - 1) / kXN);
   // patterns in launches of at most 65,535 tiles of 128 (the grid's y limit)

@@ -117,6 +117,21 @@ def test_expand_edges(n, D, K, kind):
     assert np.array_equal(out.cpu().numpy().view(np.uint64), W.pack(O.expand_sign(x, e)))
 
 
+# a device-side wait taken as expired at a CTA's first tile, one in the middle and the
+# last: the CTA's tiles are whole all the same, for each kind of copy, a short last
+# tile, two neuron tiles and words past K
+@pytest.mark.parametrize("tile", [0, 1, 2])
+@pytest.mark.parametrize("n,D,K", [(39000, 64, 64), (20000, 132, 257), (40001, 77, 33), (70, 784, 1000)])
+def test_expand_after_an_expired_wait(n, D, K, tile):
+    x = W.pixel_bytes(n + D, n, D, "pixels")
+    e = O.expand_weights(5 + K, K, D)
+    E = torch.empty((K, W.words(D)), dtype=torch.int64, device=DEV)
+    B.bmlp_expand_weights(5 + K, K, D, E)
+    out = torch.full((n, W.words(K)), -1, dtype=torch.int64, device=DEV)
+    B.bmlp_debug_expand_sign(torch.from_numpy(x).to(DEV), E, K, out, tile)
+    assert np.array_equal(out.cpu().numpy().view(np.uint64), W.pack(O.expand_sign(x, e)))
+
+
 # rows that start at any byte of a 32-bit word, also the first; other bytes all
 # around them
 @pytest.mark.parametrize("off", [0, 1, 2, 3])
