@@ -59,7 +59,7 @@ def test_small_batch_forward(K, N, n):
     gpu.close()
 
 
-# more than 512 patterns: pairs of CTAs on 256 x 256 tiles, several tiles per pair
+# more patterns: several pattern tiles, most of them still too few for the pairs
 LARGE = [(1, 1, 513), (255, 255, 700), (784, 257, 1300), (1000, 525, 2000), (2049, 300, 1025),
          (4096, 512, 900), (32767, 33, 600), (64, 2048, 11000)]
 
@@ -76,6 +76,83 @@ def test_large_batch_forward(K, N, n):
         x2[:, -1] |= ~np.uint64((1 << (K % 64)) - 1)   # pad bits set: ignored
     B.bmlp_layer_forward(gpu.h, 1, dev(x2), out)
     assert np.array_equal(out.cpu().numpy().view(np.uint64), W.pack(a))
+    gpu.close()
+
+
+# pairs of CTAs on 256 x 256 tiles, several tiles per pair: ragged neuron tiles (one
+# CTA of a pair short or empty), rows and outputs of odd word counts, one to 32 pieces
+# of K, a short last pattern tile
+PAIRS = [(1000, 255, 20000), (1000, 525, 4096), (1060, 130, 10007), (2049, 300, 12000), (5000, 257, 9000), (32767, 33, 3000),
+         (960, 640, 5000)]
+
+
+@pytest.mark.parametrize("off", [0, 1])
+@pytest.mark.parametrize("K,N,n", PAIRS)
+def test_pair_forward(K, N, n, off):
+    # (the dispatch takes the small tiles while they fit the SMs once and their
+    # pieces 1.6 times)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    tiles = -(-n // 112) * -(-N // 128)
+    assert tiles > sms or 5 * tiles * -(-K // 1024) > 8 * sms
+    gpu = B.BMLP((K, N), 4, seed=K + N, bs=64)
+    ref = O.OracleModel([K, N], 4, seed=K + N, bs=64)
+    xp = W.random_packed(n, n, K)
+    _, a = O.layer_forward(W.unpack(xp, K), ref.H(1))
+    # rows from a word's offset on, pad bits set (ignored), the output's neighbours kept
+    buf = np.zeros(n * W.words(K) + off, np.uint64)
+    rows = buf[off:].reshape(n, -1)
+    rows[:] = xp
+    if K % 64:
+        rows[:, -1] |= ~np.uint64((1 << (K % 64)) - 1)
+    out = torch.full((n * W.words(N) + off + 2,), -1, dtype=torch.int64, device=DEV)
+    B.bmlp_layer_forward(gpu.h, 1, dev(buf)[off:].view(n, -1), out[off:-2].view(n, -1))
+    assert np.array_equal(out[off:-2].view(n, -1).cpu().numpy().view(np.uint64), W.pack(a))
+    assert (out[:off] == -1).all() and (out[-2:] == -1).all()
+    gpu.close()
+
+
+# evaluation captured into a graph right behind a memset, a copy and a kernel of another
+# library that write its input, and replayed on other inputs
+@pytest.mark.parametrize("before", ["memset", "copy", "kernel"])
+@pytest.mark.parametrize("n", [100, 20000])
+def test_evaluation_in_a_graph(n, before):
+    widths = [300, 257, 130]
+    gpu = B.BMLP(widths, 10, seed=n, bs=64)
+    src = dev(W.random_packed(n, n, widths[0]))
+    x = src.clone()
+    last, every = (torch.empty(s, dtype=torch.int32, device=DEV) for s in ((n,), (2, n)))
+    layer = torch.empty((n, W.words(widths[1])), dtype=torch.int64, device=DEV)
+
+    def write():
+        if before == "memset":
+            x.zero_()
+        elif before == "copy":
+            x.copy_(src)
+        else:
+            torch.bitwise_not(src, out=x)
+
+    def calls():
+        write()
+        gpu.predict(x, last)
+        write()
+        gpu.predict_layers(x, every)
+        write()
+        B.bmlp_layer_forward(gpu.h, 1, x, layer)
+
+    calls()   # allocates the scratch
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        calls()
+    for seed in (1, 2):
+        src.copy_(dev(W.random_packed(seed, n, widths[0])))
+        calls()
+        want = [t.clone() for t in (last, every, layer)]
+        for t in (last, every, layer, x):
+            t.fill_(-1)
+        g.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(t, w) for t, w in zip((last, every, layer), want))
     gpu.close()
 
 
@@ -168,3 +245,25 @@ def test_binarize_edges(K, kind):
     out = torch.full((n, W.words(K)), -1, dtype=torch.int64, device=DEV)
     B.bmlp_binarize_median(torch.from_numpy(x).to(DEV), out)
     assert np.array_equal(out.cpu().numpy().view(np.uint64), W.pack(O.binarize_median(x)))
+
+
+# NaNs of both signs and several payloads (the padding's key among them), as few and as
+# many as half: keys ordered by their bits, x > m as floats (false for a NaN)
+@pytest.mark.parametrize("K", [1, 2, 33, 300, 784, 1200, 2048, 3000, 4096, 4097])
+def test_binarize_nan(K):
+    rng = np.random.default_rng(K)
+    n = 40
+    x = rng.standard_normal((n, K)).astype(np.float32)
+    nans = np.array([0x7FC00000, 0xFFC00000, 0x7FFFFFFF, 0xFFFFFFFF, 0x7F800001], np.uint32).view(np.float32)
+    for i in range(n):
+        hit = rng.random(K) < (i % 10) / 9.0
+        x[i, hit] = nans[rng.integers(0, 5, hit.sum())] if i < 20 else nans[i % 5]
+    x[0, 0], x[-1] = np.inf, nans[2]
+    u = x.view(np.uint32)
+    key = np.where(u >> 31, ~u, u | np.uint32(1 << 31))
+    m = np.sort(key, axis=1)[:, (K + 1) // 2 - 1]
+    m = np.where(m >> 31, m & np.uint32(0x7FFFFFFF), ~m).astype(np.uint32).view(np.float32)
+    out = torch.full((n, W.words(K)), -1, dtype=torch.int64, device=DEV)
+    B.bmlp_binarize_median(torch.from_numpy(x).to(DEV), out)
+    want = W.pack(np.where(x > m[:, None], 1, -1))
+    assert np.array_equal(out.cpu().numpy().view(np.uint64), want)
