@@ -76,7 +76,7 @@ EVAL_TRAFFIC_SRC_SHA = "836aa23ec25e3529"
 # >= 2): the layer's 8 MiB of visible weights and the activation words read, z
 # and the sign bits still in the write-back L2 when the launch ends.
 FWD_TRAFFIC_BYTES = 8_559_104 + 0
-FWD_TRAFFIC_SRC_SHA = "c48c2018bcc1744a"
+FWD_TRAFFIC_SRC_SHA = "ab2762fe999b3e9d"
 
 
 def bitpairs_per_sample(widths, classes):

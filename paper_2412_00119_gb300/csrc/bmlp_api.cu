@@ -252,9 +252,13 @@ constexpr int kGraphSteps = 8;
 // Models of more hidden weights than this update through the shared-memory ring
 // with their events drawn by a kernel of its own on a branch of the graph; the
 // others in one kernel that draws them too.  Step time at bs 100 (us), ring with
-// branch / one kernel: 63 M weights (3072-4096x4) 67.0 / 70.4, 105 M (5120x4) 98.7 /
-// 113.6, 268 M (8192x4) 152.7 / 198.7; 2.9 M (784-1024x3) 41.3 / 30.0, and at 15 M
-// (3072-2048x3) the ring alone, without the draws, 36.7 / 35.5.
+// branch / one kernel: 2.9 M weights (784-1024x3) 41.3 / 30.0, 18.9 M (3072-2400x3)
+// 42.2 / 41.0, 21.5 M (3072-2600x3) 43.1 / 43.3, 22.5 M (5000-4500) 37.5 / 37.2, 25.7 M
+// (3072-2900x3) 45.5 / 45.9, 26.2 M (5120-5120) 35.4 / 37.3, 44.3 M (3072-4000x3)
+// 54.8 / 57.1, 52.4 M (5120-5120x2) 52.4 / 63.0, 62.9 M (3072-4096x4) 64.1 / 69.7,
+// 268 M (8192x4) 152.7 / 198.7.  Above the line one kernel still wins where one layer
+// is small or the draws have less beside them: 23.4 M (784-4800-4096) 41.8 / 36.8, 30.2 M
+// (784-5120x2) 46.1 / 44.6, 33.6 M (4096-4096x2) 39.7 / 38.8.
 constexpr int64_t kRowsWeights = 20ll << 20;
 // Where the draws of the ring's models branch off (they read only the step counter
 // and the tables): before the first pass with one layer, or with a layer of this
@@ -263,13 +267,17 @@ constexpr int64_t kRowsWeights = 20ll << 20;
 // 5120-5120 35.4 / 43.2, 8192-8192 45.9 / 52.0, 3072-8192x2 69.1 / 73.2,
 // 8192x4 138.9 / 146.4; 3072-4096x4 66.8 / 63.6, 6144x2 60.0 / 59.1,
 // 6144-8192-6144 70.9 / 70.6, 7168x4 128.6 / 127.6, 8192x4 at 300 patterns
-// 236.9 / 235.5.
+// 236.9 / 235.5.  Near the line, by the largest layer: 49 Mi (7168-7168x2) 74.1 / 74.5,
+// 52.6 Mi (7424-7424x2) 76.8 / 76.9, (x4) 134.7 / 133.8, 56.2 Mi (7680-7680x2)
+// 77.9 / 79.0, (x4) 135.8 / 135.3, 60.1 Mi (7936-7936x2) 78.0 / 82.2, (x4)
+// 137.7 / 142.9.
 constexpr int64_t kEarlyDrawWeights = 56ll << 20;
 
 // One mini-batch step.  How it is launched:
 //   kStepPlain    kernel by kernel with full dependencies (sampled mini-batches);
 //   kStepDirect   kernel by kernel as programmatic dependents, with the call's
-//                 inputs as kernel parameters (a call of one mini-batch);
+//                 inputs as kernel parameters (calls of one mini-batch, but for
+//                 models whose draws go beside the later passes);
 //   kStepGraph    captured: programmatic dependents, the event draws of large
 //                 models on a branch;
 //   kStepChained  the same after another step of the graph, so that its first

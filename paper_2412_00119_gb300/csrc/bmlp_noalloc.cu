@@ -5,8 +5,9 @@
 // allow that: code running inside a region that forbids allocation (a host
 // callback, a real-time or safety loop with a fixed memory plan, a process
 // whose allocator is owned by another runtime).  bmlp_predict_noalloc runs the
-// same kernels with its scratch in the fixed, file-scope device array below, so
-// it never calls cudaMalloc, cudaFree or any allocating library routine.
+// popcount kernels, whatever the model's engine (their labels are the same), with
+// its scratch in the fixed, file-scope device array below, so it never calls
+// cudaMalloc, cudaFree or any allocating library routine.
 #include <mutex>
 
 #include "bmlp_internal.cuh"
