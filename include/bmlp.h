@@ -140,7 +140,9 @@ void bmlp_destroy(bmlp_t* h);
  * If a bounded device-side wait of a training forward pass expires (tensor-
  * core engine), that mini-batch and every later one until the expiry is
  * reported change neither H nor W (no marks, no update; the step counter
- * still advances); the next call that synchronises returns BMLP_ETIMEOUT. */
+ * still advances); the next call that synchronises returns BMLP_ETIMEOUT.
+ * While cuda_stream is being captured the call returns BMLP_ECUDA and puts
+ * nothing into it (a replay would run past the host's step count). */
 int bmlp_train(bmlp_t* h, const uint64_t* x_packed, const int32_t* labels, int64_t n,
                uint32_t flags, void* cuda_stream, int64_t* n_errors_out);
 
